@@ -29,6 +29,7 @@
 // issued and the products it has issued are waited for (they always
 // complete; those waits carry a separate, much larger bound).
 #include <cuda.h>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -41,10 +42,13 @@ namespace bst {
 
 namespace oz {
 
+namespace cg = cooperative_groups;
+
 constexpr int kTM = 128;           // tile rows (M)
 constexpr int kTK = 32;            // K per stage (64 bytes of BF16)
 constexpr int kABytes = kTM * kTK * 2;   // 8 KB per slice
-constexpr int kThreads = 320;            // 10 warps: TMA, MMA, 8 epilogue
+constexpr int kEpiWarps = 16;            // four per quarter of the 128 tensor-memory lanes
+constexpr int kThreads = 32 * (2 + kEpiWarps);  // TMA, MMA and epilogue warps
 constexpr long long kSpinLimit = 1ll << 28;   // default bound of a pipeline wait (tries)
 constexpr long long kDrainLimit = 1ll << 30;  // bound of the waits for issued copies and products
 
@@ -93,12 +97,15 @@ struct Scatter {
 };
 
 struct Tile {
-  int32_t prob, m0, n0, pad;
+  int32_t prob, m0, n0;
+  int32_t nk;          // K chunks of kTK
+  int32_t arow, brow;  // the tile's first rows in the split A / B buffers
+  int32_t pad[2];
 };
 
 struct SplitTask {
   int32_t rows, K;
-  int32_t row0, pad;  // first row in the split buffer
+  int32_t row0, cta0;  // first row in the split buffer, first CTA of the task in its operand's range
   int64_t base, s_r, s_k;
 };
 
@@ -126,6 +133,17 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
+// The same look without the time slice that try_wait may spend asleep.
+__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait; returns false (and raises the abort flag) on expiry or when
 // another role already aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, int* err,
@@ -139,25 +157,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
   return false;
 }
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
+// All S slices of a tile's rows for one K chunk: box {kTK, rows, S}
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
           smem_u32(dst)),
-      "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar))
+      "l"(map), "r"(c0), "r"(c1), "r"(0), "r"(smem_u32(bar))
       : "memory");
 }
 
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups
-// 512 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= uint64_t((addr >> 4) & 0x3FFF);
-  d |= uint64_t(1) << 16;                    // leading byte offset (unused with swizzle)
-  d |= uint64_t((512 >> 4) & 0x3FFF) << 32;  // stride byte offset
-  d |= uint64_t(1) << 46;                    // descriptor version
-  d |= uint64_t(4) << 61;                    // SWIZZLE_64B
-  return d;
-}
+// 512 bytes apart.  Low word: address / 16 (14 bits; the tiles lie below 227
+// KB, so offsets are added without a carry out) and the leading byte offset
+// (unused with swizzle); high word: stride, descriptor version, SWIZZLE_64B.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr >> 4) & 0x3FFF) | (1u << 16); }
+constexpr uint32_t kDescHi = (512u >> 4) | (1u << 14) | (4u << 29);
 
 // kind::f16 instruction descriptor: BF16 x BF16 -> F32, both K-major.
 template <int TN>
@@ -165,14 +179,16 @@ __host__ __device__ constexpr uint32_t instr_desc() {
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(TN >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
 }
 
-// D[128 x N] (+)= A[128 x 16] B[N x 16]^T; N a multiple of 16, at most 256
+// D[128 x N] (+)= A[128 x 16] B[N x 16]^T; N a multiple of 16, at most 256;
+// a, b: low words of the operands' descriptors.
 template <int N>
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t acc) {
   static_assert(N % 16 == 0 && N >= 16 && N <= 256, "tcgen05.mma kind::f16 with M = 128");
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(instr_desc<N>()), "r"(acc));
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n"
+      " mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a), "r"(b), "r"(instr_desc<N>()), "r"(acc), "r"(kDescHi));
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -180,44 +196,42 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-
-// kHalf (32 or 16) consecutive columns of this warp's 32 lanes
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld32(taddr, r); }
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld16(taddr, r); }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 2^e as a double for e in [-1022, 1023] (built from the bit pattern)
-__device__ __forceinline__ double pow2i(int e) {
-  e = max(-1022, min(1023, e));
-  return __longlong_as_double((long long)(e + 1023) << 52);
+// X 2^e rounded to nearest even, built from the IEEE fields: the FP64 pipe
+// of this part issues about two operations per clock and SM, so a conversion
+// and two products per output cost a 128 x 64 tile ~12000 cycles, more than
+// the products of a K = 128 tile.  Results outside the normal range take the
+// FP64 route.
+__device__ __forceinline__ double scaled_double(long long X, int e) {
+  const unsigned long long u = X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X;
+  const int lz = __clzll((long long)u);
+  const unsigned long long n = u << (lz & 63);
+  const int ex = 1085 - lz + e;  // biased exponent less one of the leading bit's weight 2^(63 - lz + e)
+  // mantissa with its leading bit, plus the round bit (ties to even)
+  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull & ((n & 0x3ffull) || (n & 0x800ull) ? 1ull : 0ull));
+  const unsigned long long bits = ((unsigned long long)(unsigned)ex << 52) + m;
+  if (ex < 1 || ex > 2043 || u == 0) {
+    const int h = max(-1022, min(1023, e >> 1)), l = max(-1022, min(1023, e - (e >> 1)));
+    return double(X) * __longlong_as_double((long long)(h + 1023) << 52) *
+           __longlong_as_double((long long)(l + 1023) << 52);
+  }
+  return __longlong_as_double((long long)(bits | (X < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
+constexpr int kOutLd = 9;  // 8 columns (odd stride: rows fall on different banks)
 template <int S, int TN>
 struct Smem {
   alignas(1024) uint8_t stage[Cfg<S, TN>::kStages][Cfg<S, TN>::kStageBytes];
+  long long out[kEpiWarps][32][kOutLd];  // per epilogue warp: 8 columns of its rows
   uint64_t full[Cfg<S, TN>::kStages], empty[Cfg<S, TN>::kStages];
   uint64_t acc_full[2], acc_empty[2];
   uint64_t acc34_empty;  // the epilogue has read d3, d4 of the previous tile
@@ -238,8 +252,7 @@ template <int S, int TN>
 __global__ void __launch_bounds__(kThreads, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                       const Prob* __restrict__ probs, const Tile* __restrict__ tiles, int ntiles,
-                      const int* __restrict__ expA, const int* __restrict__ expB, int rowsA, int rowsB,
-                      double* __restrict__ C, const Scatter sc, int* err, long long spin) {
+                      const int* __restrict__ expA, const int* __restrict__ expB, double* __restrict__ C, const Scatter sc, int* err, long long spin) {
   using CF = Cfg<S, TN>;
   constexpr int kStages = CF::kStages;
   constexpr int kStageBytes = CF::kStageBytes;
@@ -256,9 +269,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sm.acc_full[b], 1);
-      mbar_init(&sm.acc_empty[b], 256);
+      mbar_init(&sm.acc_empty[b], 32 * kEpiWarps);
     }
-    mbar_init(&sm.acc34_empty, 256);
+    mbar_init(&sm.acc34_empty, 32 * kEpiWarps);
     mbar_init(&sm.mma_drain, 1);
     sm.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -275,36 +288,40 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort_flag = &sm.abort_flag;
 
+  // Ring positions are counted as (stage, phase) and (buffer, phase) pairs:
+  // the roles run one instruction stream each, so a 64-bit division by the
+  // stage count per chunk is time the tensor core waits for.
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      long long g = 0;  // chunks issued so far (all tiles)
+      uint32_t s = 0, ph = 0;
+      int issued = 0;  // chunks issued so far, up to kStages
       bool ok = true;
-      for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
-        const Tile t = tiles[ti];
-        const Prob p = probs[t.prob];
-        const int nk = (p.K + kTK - 1) / kTK;
-        for (int c = 0; c < nk; ++c, ++g) {
-          const int s = int(g % kStages);
-          if (g >= kStages && !mbar_wait(&sm.empty[s], int((g / kStages) - 1) & 1, abort_flag, err, spin)) {
+      Tile t = tiles[blockIdx.x];  // (the grid has at most ntiles CTAs)
+      for (int ti = blockIdx.x; ti < ntiles && ok;) {
+        ti += gridDim.x;
+        const Tile nxt = ti < ntiles ? tiles[ti] : t;  // in flight during this tile
+        for (int c = 0; c < t.nk; ++c) {
+          if (issued == kStages && !mbar_wait(&sm.empty[s], ph ^ 1u, abort_flag, err, spin)) {
             ok = false;
             break;
           }
+          issued += issued < kStages;
           mbar_expect_tx(&sm.full[s], kStageBytes);
           uint8_t* base = sm.stage[s];
-          const int k0 = c * kTK;
-          for (int i = 0; i < S; ++i)
-            tma_load_2d(base + i * kABytes, &mapA, k0, i * rowsA + p.arow + t.m0, &sm.full[s]);
-          for (int j = 0; j < S; ++j)
-            tma_load_2d(base + S * kABytes + j * kBBytes, &mapB, k0, j * rowsB + p.brow + t.n0, &sm.full[s]);
+          tma_load_3d(base, &mapA, c * kTK, t.arow, &sm.full[s]);
+          tma_load_3d(base + S * kABytes, &mapB, c * kTK, t.brow, &sm.full[s]);
+          if (++s == kStages) s = 0, ph ^= 1u;
         }
+        t = nxt;
       }
       // every copy issued has landed before the CTA may exit, whichever
       // role aborted and when (after a normal run these phases are already
       // complete: the products consumed them)
-      for (long long c = (g > kStages ? g - kStages : 0); c < g; ++c) {
-        const int s = int(c % kStages);
-        for (long long i = 0; i < kDrainLimit && !mbar_try(&sm.full[s], int(c / kStages) & 1); ++i) {
+      for (int i = 0; i < issued; ++i) {
+        if (s == 0) s = kStages, ph ^= 1u;
+        --s;
+        for (long long w = 0; w < kDrainLimit && !mbar_try(&sm.full[s], ph); ++w) {
         }
       }
     }
@@ -314,176 +331,230 @@ __global__ void __launch_bounds__(kThreads, 1)
     // exact integers below 2^24 (at most 3 * 64 products of magnitude
     // <= 2^16 per diagonal entry)
     if (lane == 0) {
-      long long g = 0, pg = 0;  // chunks and chunk pairs consumed so far (all tiles)
-      int tn = 0;               // tiles of this CTA so far
-      bool ok = true;
-      for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x, ++tn) {
-        const Prob p = probs[tiles[ti].prob];
-        const int nk = (p.K + kTK - 1) / kTK;
-        for (int c = 0; c < nk; ++c, ++g) {
-          const int s = int(g % kStages);
-          const long long pc = pg + (c >> 1);
-          const int buf = int(pc & 1);
-          const bool first = (c & 1) == 0;
-          if (!mbar_wait(&sm.full[s], int(g / kStages) & 1, abort_flag, err, spin)) {
+    uint32_t s = 0, ph = 0;          // stage ring
+    uint32_t buf = 0, bph = 0;       // d0..d2 buffers
+    int pairs = 0;                   // pairs begun so far, up to 2
+    uint32_t tph = 0;                // phase of acc34_empty
+    bool ok = true, first_tile = true;
+    bool have_full = false, have_buf = false;  // this chunk's waits found done ahead of time
+    int nk = tiles[blockIdx.x].nk;
+    for (int ti = blockIdx.x; ti < ntiles && ok;) {
+      ti += gridDim.x;
+      const int nk_next = ti < ntiles ? tiles[ti].nk : 0;
+      for (int c = 0; c < nk; ++c) {
+        const bool first = (c & 1) == 0;
+        if (!have_full && !mbar_wait(&sm.full[s], ph, abort_flag, err, spin)) {
+          ok = false;
+          break;
+        }
+        if (first) {
+          if (pairs == 2 && !have_buf && !mbar_wait(&sm.acc_empty[buf], bph ^ 1u, abort_flag, err, spin)) {
             ok = false;
             break;
           }
-          if (first && pc >= 2 && !mbar_wait(&sm.acc_empty[buf], int((pc >> 1) - 1) & 1, abort_flag, err, spin)) {
-            ok = false;
-            break;
-          }
-          if (S == 5 && c == 0 && tn > 0 && !mbar_wait(&sm.acc34_empty, (tn - 1) & 1, abort_flag, err, spin)) {
+          if (S == 5 && c == 0 && !first_tile && !mbar_wait(&sm.acc34_empty, tph ^ 1u, abort_flag, err, spin)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sm.stage[s]);
-          const uint32_t b0 = a0 + S * kABytes;
-          // The slices of B are stacked in the stage (slice j: rows
-          // j TN .. j TN + TN - 1), so B slices j .. j + n - 1 form one
-          // operand of n TN rows; in tensor memory the diagonals of a
-          // buffer lie side by side (d at buf 3 TN + d TN; d3, d4 at
-          // kColD3).  A slice i times B slices j .. j + n - 1 thus adds into
-          // diagonals i + j .. i + j + n - 1 with one product: 8 products
-          // of width TN .. 3 TN per 16 K instead of 15 of width TN (S = 5),
-          // 3 instead of 6 (S = 3), each reading its A slice once.
-          const uint32_t cb = tmem + uint32_t(buf * 3 * TN);
-          const uint32_t c3 = tmem + uint32_t(kColD3);
-          for (int ks = 0; ks < kTK / 16; ++ks) {
-            const uint32_t acc_b = (!first || ks > 0) ? 1u : 0u;  // first writer of d0..d2 in this pair
-            const uint32_t acc_3 = (c > 0 || ks > 0) ? 1u : 0u;   // first writer of d3, d4 in this tile
-            auto ad = [&](int i) { return smem_desc(a0 + i * kABytes + ks * 32); };
-            auto bd = [&](int j) { return smem_desc(b0 + j * kBBytes + ks * 32); };
-            mma_bf16<3 * TN>(cb, ad(0), bd(0), acc_b);           // d0 d1 d2 += A0 [B0 B1 B2]
-            if constexpr (S == 5) mma_bf16<2 * TN>(c3, ad(0), bd(3), acc_3);  // d3 d4 += A0 [B3 B4]
-            mma_bf16<2 * TN>(cb + TN, ad(1), bd(0), 1u);         // d1 d2 += A1 [B0 B1]
-            if constexpr (S == 5) mma_bf16<2 * TN>(c3, ad(1), bd(2), 1u);     // d3 d4 += A1 [B2 B3]
-            mma_bf16<TN>(cb + 2 * TN, ad(2), bd(0), 1u);         // d2 += A2 B0
-            if constexpr (S == 5) {
-              mma_bf16<2 * TN>(c3, ad(2), bd(1), 1u);            // d3 d4 += A2 [B1 B2]
-              mma_bf16<2 * TN>(c3, ad(3), bd(0), 1u);            // d3 d4 += A3 [B0 B1]
-              mma_bf16<TN>(c3 + TN, ad(4), bd(0), 1u);           // d4 += A4 B0
-            }
-          }
-          mma_commit(&sm.empty[s]);
-          if (!first || c == nk - 1) mma_commit(&sm.acc_full[buf]);
         }
-        pg += (nk + 1) >> 1;
+        const uint32_t sn = s + 1 == kStages ? 0u : s + 1, phn = s + 1 == kStages ? ph ^ 1u : ph;
+        const uint32_t a0 = desc_lo(smem_u32(sm.stage[s]));
+        const uint32_t b0 = a0 + ((S * kABytes) >> 4);
+        // The slices of B are stacked in the stage (slice j: rows
+        // j TN .. j TN + TN - 1), so B slices j .. j + n - 1 form one
+        // operand of n TN rows; in tensor memory the diagonals of a
+        // buffer lie side by side (d at buf 3 TN + d TN; d3, d4 at
+        // kColD3).  A slice i times B slices j .. j + n - 1 thus adds into
+        // diagonals i + j .. i + j + n - 1 with one product: 8 products
+        // of width TN .. 3 TN per 16 K instead of 15 of width TN (S = 5),
+        // 3 instead of 6 (S = 3), each reading its A slice once.
+        const uint32_t cb = tmem + uint32_t(buf * 3 * TN);
+        const uint32_t c3 = tmem + uint32_t(kColD3);
+#pragma unroll
+        for (int ks = 0; ks < kTK / 16; ++ks) {
+          const uint32_t acc_b = (!first || ks > 0) ? 1u : 0u;  // first writer of d0..d2 in this pair
+          const uint32_t acc_3 = (c > 0 || ks > 0) ? 1u : 0u;   // first writer of d3, d4 in this tile
+          auto ad = [&](int i) { return a0 + uint32_t((i * kABytes + ks * 32) >> 4); };
+          auto bd = [&](int j) { return b0 + uint32_t((j * kBBytes + ks * 32) >> 4); };
+          // (d3, d4 accumulate with rounding: their products keep this
+          // order; d0..d2 are exact.  The widest product goes first or last
+          // so that the tensor core is busy longest around the waits.)
+          if (ks == 0) mma_bf16<3 * TN>(cb, ad(0), bd(0), acc_b);           // d0 d1 d2 += A0 [B0 B1 B2]
+          if constexpr (S == 5) mma_bf16<2 * TN>(c3, ad(0), bd(3), acc_3);  // d3 d4 += A0 [B3 B4]
+          mma_bf16<2 * TN>(cb + TN, ad(1), bd(0), 1u);                      // d1 d2 += A1 [B0 B1]
+          if constexpr (S == 5) mma_bf16<2 * TN>(c3, ad(1), bd(2), 1u);     // d3 d4 += A1 [B2 B3]
+          mma_bf16<TN>(cb + 2 * TN, ad(2), bd(0), 1u);                      // d2 += A2 B0
+          if (ks == 1) {
+            // the next chunk's barriers, looked at while this one's products
+            // queue: a wait that starts after the last product leaves the
+            // tensor core idle for its latency
+            have_full = mbar_test(&sm.full[sn], phn);
+            have_buf = mbar_test(&sm.acc_empty[buf ^ 1u], buf ? bph : bph ^ 1u);
+          }
+          if constexpr (S == 5) {
+            mma_bf16<2 * TN>(c3, ad(2), bd(1), 1u);            // d3 d4 += A2 [B1 B2]
+            mma_bf16<2 * TN>(c3, ad(3), bd(0), 1u);            // d3 d4 += A3 [B0 B1]
+            mma_bf16<TN>(c3 + TN, ad(4), bd(0), 1u);           // d4 += A4 B0
+          }
+          if (ks == 1) mma_bf16<3 * TN>(cb, ad(0), bd(0), 1u);
+        }
+        mma_commit(&sm.empty[s]);
+        s = sn;
+        ph = phn;
+        if (!first || c == nk - 1) {
+          mma_commit(&sm.acc_full[buf]);
+          pairs += pairs < 2;
+          buf ^= 1u;
+          if (buf == 0) bph ^= 1u;
+        }
       }
-      // every product issued has written tensor memory before it is freed,
-      // whichever role aborted and when (the commit arrives once they have
-      // all completed; with none issued, at once)
-      mma_commit(&sm.mma_drain);
-      for (long long i = 0; i < kDrainLimit && !mbar_try(&sm.mma_drain, 0); ++i) {
-      }
+      first_tile = false;
+      tph ^= 1u;
+      nk = nk_next;
+    }
+    // every product issued has written tensor memory before it is freed,
+    // whichever role aborted and when (the commit arrives once they have
+    // all completed; with none issued, at once)
+    mma_commit(&sm.mma_drain);
+    for (long long i = 0; i < kDrainLimit && !mbar_try(&sm.mma_drain, 0); ++i) {
+    }
     }
   } else {
-    // ---------------- epilogue: warps 2..9 ----------------
-    // warp w may access tensor-memory lanes 32*(w%4)..+31; the two warps of a
-    // lane quarter split the 64 columns
-    constexpr int kHalf = TN / 2;
+    // ---------------- epilogue: warps 2..17 ----------------
+    // warp w may access tensor-memory lanes 32*(w%4)..+31; the four warps of
+    // a lane quarter split the TN columns (with two of them and twice the
+    // columns each, a tile's waits, conversions and stores left the tensor
+    // core waiting for its accumulators)
+    constexpr int kCols = TN / 4;
     const int q = warp & 3;
-    const int c0 = ((warp - 2) >> 2) * kHalf;
+    const int c0 = ((warp - 2) >> 2) * kCols;
     const int row = q * 32 + lane;
     const uint32_t lane_base = tmem + (uint32_t(q * 32) << 16);
-    long long pg = 0;
+    uint32_t buf = 0, bph = 0;
     bool ok = true;
-    for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
-      const Tile t = tiles[ti];
+    Tile t = tiles[blockIdx.x];
+    for (int ti = blockIdx.x; ti < ntiles && ok;) {
+      ti += gridDim.x;
+      const Tile nxt = ti < ntiles ? tiles[ti] : t;
       const Prob p = probs[t.prob];
-      const int nk = (p.K + kTK - 1) / kTK;
-      // T = sum over chunk pairs of (S0 2^18 + S1 2^9 + S2): exact in 64 bits
-      long long T[kHalf];
+      // the tile's rows and columns, loaded while its products run: lane l
+      // holds row l's exponent and scatter entry, and those of the columns
+      // that it writes, c0 + (l & 7) (+ 8)
+      const bool row_ok = t.m0 + row < p.M;
+      const int ea = row_ok ? expA[t.arow + row] - CF::kShift : 0;
+      int2 ri = make_int2(0, 0);
+      if (p.scatter && row_ok) ri = sc.rowtab[p.rt_off + t.m0 + row];
+      int eb[kCols / 8];
+      int4 ci[kCols / 8];
 #pragma unroll
-      for (int j = 0; j < kHalf; ++j) T[j] = 0;
-      const int npair = (nk + 1) >> 1;
+      for (int h = 0; h < kCols / 8; ++h) {
+        const int gn = t.n0 + c0 + h * 8 + (lane & 7);
+        eb[h] = gn < p.N ? expB[p.brow + gn] : 0;
+        ci[h] = p.scatter && gn < p.N ? sc.coltab[p.ct_off + gn] : make_int4(0, 0, 0, 0);
+      }
+      // T = sum over chunk pairs of (S0 2^18 + S1 2^9 + S2): exact in 64 bits
+      long long T[kCols];
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) T[j] = 0;
+      const int npair = (t.nk + 1) >> 1;
       for (int pp = 0; pp < npair; ++pp) {
-        const long long pc = pg + pp;
-        const int buf = int(pc & 1);
-        ok = mbar_wait(&sm.acc_full[buf], int(pc >> 1) & 1, abort_flag, err, spin);
+        ok = mbar_wait(&sm.acc_full[buf], bph, abort_flag, err, spin);
         if (!ok) break;
         tc_fence_after();
-        // exact FP32 integers below 2^24: one round-to-nearest conversion
-        // each; 16 columns at a time (the 64-bit sums hold the registers)
+        // The three diagonals of 8 columns per wait; the buffer goes back
+        // to the products as soon as its last load has landed, before the
+        // conversions.  |S0| <= 64 2^16 = 2^22: adding 3 2^22 puts it in the
+        // low bits of the FP32 pattern, so the patterns stand for S0 (npair
+        // times the constant's pattern is taken off at the end) without the
+        // slow conversion that S1 and S2 (up to 3 2^22) need.
 #pragma unroll
-        for (int h = 0; h < kHalf; h += 16) {
-          uint32_t v[16];
-          tmem_ld16(lane_base + buf * 3 * TN + 0 * TN + c0 + h, v);
+        for (int h = 0; h < kCols; h += 8) {
+          uint32_t v0[8], v1[8], v2[8];
+          tmem_ld8(lane_base + buf * 3 * TN + 0 * TN + c0 + h, v0);
+          tmem_ld8(lane_base + buf * 3 * TN + 1 * TN + c0 + h, v1);
+          tmem_ld8(lane_base + buf * 3 * TN + 2 * TN + c0 + h, v2);
           tmem_wait_ld();
+          if (h + 8 == kCols) {
+            tc_fence_before();
+            mbar_arrive(&sm.acc_empty[buf]);
+          }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) T[h + j] += (long long)__float2int_rn(__uint_as_float(v[j])) << 18;
-          tmem_ld16(lane_base + buf * 3 * TN + 1 * TN + c0 + h, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) T[h + j] += (long long)__float2int_rn(__uint_as_float(v[j])) << 9;
-          tmem_ld16(lane_base + buf * 3 * TN + 2 * TN + c0 + h, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) T[h + j] += __float2int_rn(__uint_as_float(v[j]));
+          for (int j = 0; j < 8; ++j) {
+            T[h + j] += (long long)__float_as_int(__uint_as_float(v0[j]) + 12582912.0f) * (1 << 18);
+            T[h + j] += (long long)__float2int_rn(__uint_as_float(v1[j])) * (1 << 9);
+            T[h + j] += __float2int_rn(__uint_as_float(v2[j]));
+          }
         }
-        tc_fence_before();
-        mbar_arrive(&sm.acc_empty[buf]);
+        buf ^= 1u;
+        if (buf == 0) bph ^= 1u;
       }
       if (!ok) break;
-      pg += npair;
-      // S = 5: X = S0 2^27 + S1 2^18 + S2 2^9 + (S3 + S4 2^-9), folded into
-      // T; then d3 and d4 are released to the next tile's products
-      if constexpr (S == 5) {
+      const long long off0 = ((long long)npair * 0x4B400000ll) << 18;
+      // S = 5: X = T 2^9 + (S3 + S4 2^-9); d3 and d4 go back to the next
+      // tile's products, which wait for them, before any output is written
 #pragma unroll
-        for (int h = 0; h < kHalf / 16; ++h) {
-          uint32_t w3[16], w4[16];
-          if (nk > 0) {
-            tmem_ld16(lane_base + kColD3 + 0 * TN + c0 + h * 16, w3);
-            tmem_ld16(lane_base + kColD3 + 1 * TN + c0 + h * 16, w4);
-            tmem_wait_ld();
-          } else {
+      for (int h = 0; h < kCols; h += 8) {
+        if constexpr (S == 5) {
+          uint32_t w3[8], w4[8];
+          tmem_ld8(lane_base + kColD3 + 0 * TN + c0 + h, w3);
+          tmem_ld8(lane_base + kColD3 + 1 * TN + c0 + h, w4);
+          tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) w3[j] = w4[j] = 0u;
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
+          for (int j = 0; j < 8; ++j) {
             const float small = __uint_as_float(w3[j]) + __uint_as_float(w4[j]) * (1.0f / 512.0f);
-            T[h * 16 + j] = (T[h * 16 + j] << 9) + __float2ll_rn(small);
+            T[h + j] = ((T[h + j] - off0) << 9) + __float2ll_rn(small);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) T[h + j] -= off0;
+        }
+      }
+      if constexpr (S == 5) {
+        tc_fence_before();
+        mbar_arrive(&sm.acc34_empty);
+      }
+      // C = X 2^(ea + eb - shift).  A lane holds a row of 8 or 16 columns,
+      // which written by itself would touch 32 lines per store: 8 columns at
+      // a time go through shared memory, and a store writes 8 columns of
+      // four rows.  Scatter: straight into the output tensor's canonical
+      // blocks, row (ri.x, ri.y) and column (ci.x, ci.y) of the block (ri.x,
+      // ci.x) of width ci.z; else the sector matrix.
+      long long(*st)[kOutLd] = sm.out[warp - 2];
+      const bool plain = !p.scatter || (sc.alpha == 1.0 && sc.beta == 0.0);
+      const int mrows = p.M - t.m0 - q * 32;
+#pragma unroll
+      for (int h = 0; h < kCols / 8; ++h) {
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) st[lane][j] = T[h * 8 + j];
+        __syncwarp();
+        const int gn = t.n0 + c0 + h * 8 + (lane & 7);
+        const bool col_ok = gn < p.N;
+        int rblk = -1;
+        long long cbase = 0;
+#pragma unroll 4
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3);
+          const double v = scaled_double(st[r][lane & 7], __shfl_sync(0xffffffffu, ea, r) + eb[h]);
+          const bool live = col_ok && r < mrows;
+          if (p.scatter) {
+            const int rx = __shfl_sync(0xffffffffu, ri.x, r), ry = __shfl_sync(0xffffffffu, ri.y, r);
+            if (live) {
+              if (rx != rblk) {
+                rblk = rx;
+                cbase = sc.bbase[p.bb_off + (long long)rx * p.ncc + ci[h].x] + ci[h].y;
+              }
+              double* dst = C + cbase + (long long)ry * ci[h].z;
+              if (plain) *dst = v;
+              else *dst = sc.beta == 0.0 ? sc.alpha * v : fma(sc.alpha, v, sc.beta * *dst);
+            }
+          } else if (live) {
+            C[p.c_off + (long long)(t.m0 + q * 32 + r) * p.c_m + (long long)gn * p.c_n] = v;
           }
         }
       }
-      tc_fence_before();
-      mbar_arrive(&sm.acc34_empty);
-      // C = X 2^(ea+eb-43)
-      const int gm = t.m0 + row;
-      const bool row_ok = gm < p.M;
-      const int ea = row_ok ? expA[p.arow + gm] : 0;
-      if (p.scatter) {
-        // straight into the output tensor's canonical blocks: this row's
-        // block row r and row mi inside it; the columns' block, column and
-        // block width are the same for every lane (broadcast loads)
-        const int2 ri = row_ok ? sc.rowtab[p.rt_off + gm] : make_int2(0, 0);
-        const long long* bb = sc.bbase + p.bb_off + (long long)ri.x * p.ncc;
-        const bool plain = sc.alpha == 1.0 && sc.beta == 0.0;
-#pragma unroll
-        for (int jj = 0; jj < kHalf; ++jj) {
-          const int gn = t.n0 + c0 + jj;
-          if (row_ok && gn < p.N) {
-            const int4 ci = sc.coltab[p.ct_off + gn];
-            const long long dst = bb[ci.x] + (long long)ri.y * ci.z + ci.y;
-            const int e = ea + expB[p.brow + gn] - CF::kShift;
-            const double v = (double)T[jj] * pow2i(e >> 1) * pow2i(e - (e >> 1));
-            if (plain) C[dst] = v;
-            else C[dst] = sc.beta == 0.0 ? sc.alpha * v : fma(sc.alpha, v, sc.beta * C[dst]);
-          }
-        }
-      } else {
-        double* crow = C + p.c_off + (long long)gm * p.c_m;
-#pragma unroll
-        for (int jj = 0; jj < kHalf; ++jj) {
-          const int gn = t.n0 + c0 + jj;
-          if (row_ok && gn < p.N) {
-            const int e = ea + expB[p.brow + gn] - CF::kShift;
-            crow[(long long)gn * p.c_n] = (double)T[jj] * pow2i(e >> 1) * pow2i(e - (e >> 1));
-          }
-        }
-      }
+      t = nxt;
     }
   }
   tc_fence_before();
@@ -532,10 +603,24 @@ __device__ __forceinline__ void zero_part(const ZeroJob& z, int cta) {
 }
 
 // Split FP64 rows into S BF16 digit slices (integer arithmetic on the bit
-// pattern).  One warp per row; digits for k in [K, roundup(K, 32)) are 0.
-// One launch splits both operands: CTAs [0, ga) take the rows of A, the
-// others those of B.  The task of a row is found by binary search over the
-// tasks' first rows (ascending).
+// pattern); digits for k in [K, roundup(K, 32)) are 0.  One launch splits
+// both operands: CTAs [0, ga) take the tasks of A, the next gb those of B;
+// a CTA finds its task by binary search over the tasks' first CTAs.
+//
+// The kernel moves 8 bytes in and 2 S out per element, so what bounds it is
+// how the rows lie in memory:
+//   * rows contiguous along k (s_k = 1): four consecutive k per lane (two
+//     16-byte loads where the row is 16-byte aligned, 8-byte stores).  Rows
+//     up to 512 long stay in registers between the maximum and the digits;
+//     longer ones are read again;
+//   * rows interleaved (s_r = 1, the columns of a row-major block, as every
+//     product with the iterated block has them): lanes along the rows, 16
+//     consecutive k per thread, so the loads of a warp are 256 contiguous
+//     bytes and every thread stores whole 32-byte sectors.  A cluster of up
+//     to 8 CTAs shares the k range of 32 rows and exchanges the row maxima
+//     through distributed shared memory: one launch, no atomics.  With lanes
+//     along k instead, as for contiguous rows, every load of a warp touched
+//     32 sectors of which 8 bytes each were used.
 struct SplitJob {
   const SplitTask* tasks;
   int ntasks, rows_total;
@@ -544,80 +629,244 @@ struct SplitJob {
   int* ex;
 };
 
+constexpr int kSplitThreads = 256;
+constexpr int kSplitRowMax = 512;  // longest contiguous row kept in registers (4 x 4 per lane)
+
+// The digits of the value with bit pattern b against the row exponent e
+// (|x| < 2^e), as the bit patterns of the FP32 numbers (BF16 in the upper
+// half): X = round(|x| 2^(9 S - 1 - e)) with the sign of x, X = sum_i a_i
+// 2^(9 (S - 1 - i)) with a_i in [-256, 255] for i > 0.  Adding 256 at every
+// digit but the first makes all of them non-negative bit fields.
 template <int S>
-__global__ void ozaki_split_kernel(SplitJob ja, SplitJob jb, int ga, int gab, int kpitch, ZeroJob zj) {
+__device__ __forceinline__ void split_digits(unsigned long long b, int e, uint32_t (&f)[S]) {
+  const int E = int(b >> 52) & 0x7FF;
+  long long X = 0;
+  if (E != 0) {  // subnormals of a row with a normal maximum are below 2^-44 of it
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+    // E <= e + 1022 and 9 S - 1 <= 44: the shift is to the right by 9 or more
+    const int rs = 1075 + e - E - (9 * S - 1);
+    if (rs < 64) X = (long long)((m + (1ull << (rs - 1))) >> rs);
+    if ((long long)b < 0) X = -X;
+  }
+  long long bias = 0;
+#pragma unroll
+  for (int i = 0; i < S - 1; ++i) bias |= 256ll << (9 * i);
+  X += bias;
+#pragma unroll
+  for (int i = S - 1; i >= 1; --i)
+    // a + 2^23 + 2^22 as an FP32 integer, minus that constant: a, exact
+    f[i] = __float_as_uint(__uint_as_float(0x4B400000u - 256u + (uint32_t(X >> (9 * (S - 1 - i))) & 511u)) -
+                           12582912.0f);
+  f[0] = __float_as_uint(__uint_as_float(0x4B400000u + uint32_t(int(X >> (9 * (S - 1))))) - 12582912.0f);
+}
+
+// two BF16 numbers (the upper halves of their FP32 patterns), lower k first
+__device__ __forceinline__ uint32_t pack_bf16(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
+
+__device__ __forceinline__ unsigned long long abs_bits(unsigned long long b) { return b & 0x7FFFFFFFFFFFFFFFull; }
+
+// Rows contiguous along k: how many a CTA takes.  Four k per lane: rows up
+// to 32 (64, 128) long take 8 (16, 32) lanes and a warp does four passes of
+// 4 (2, 1) rows, all loads first; longer rows take a warp each.
+__host__ __device__ inline int split_cta_rows(int K) {
+  const int per_warp = K <= 32 ? 16 : K <= 64 ? 8 : K <= 128 ? 4 : 1;
+  return per_warp * (kSplitThreads / 32);
+}
+
+template <int S>
+__device__ __forceinline__ void split_rows(const SplitJob& J, const SplitTask& tk, int cta, int kpitch) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kend = (tk.K + 31) & ~31;
+  auto load4 = [&](const double* xr, int k, unsigned long long (&v)[4]) {
+    if (k + 3 < tk.K && (reinterpret_cast<uintptr_t>(xr) & 15) == 0) {
+      const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(xr + k);
+      const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(xr + k + 2);
+      v[0] = p.x, v[1] = p.y, v[2] = q.x, v[3] = q.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = k + j < tk.K ? (unsigned long long)__double_as_longlong(xr[k + j]) : 0ull;
+    }
+  };
+  auto store4 = [&](long long grow, int k, int e, const unsigned long long (&v)[4]) {
+    uint32_t f[4][S];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) split_digits<S>(v[j], e, f[j]);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+      *reinterpret_cast<uint2*>(J.S + ((long long)i * J.rows_total + grow) * kpitch + k) =
+          make_uint2(pack_bf16(f[0][i], f[1][i]), pack_bf16(f[2][i], f[3][i]));
+  };
+  unsigned long long x[4][4];
+  if (tk.K <= 128) {
+    const int lpr = tk.K <= 32 ? 8 : tk.K <= 64 ? 16 : 32;  // lanes per row
+    const int rpw = 32 / lpr, k = (lane % lpr) * 4;
+    const int r0 = (cta * (kSplitThreads / 32) + warp) * 4 * rpw + lane / lpr;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      const int r = r0 + it * rpw;
+      if (r < tk.rows) load4(J.X + tk.base + (long long)r * tk.s_r, k, x[it]);
+      else x[it][0] = x[it][1] = x[it][2] = x[it][3] = 0;
+    }
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      unsigned long long mx = max(max(abs_bits(x[it][0]), abs_bits(x[it][1])),
+                                  max(abs_bits(x[it][2]), abs_bits(x[it][3])));
+      for (int o = lpr >> 1; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      // |x| < 2^e for every entry of the row (e from the largest exponent field)
+      const int e = int(mx >> 52) - 1022;
+      const int r = r0 + it * rpw;
+      if (r >= tk.rows) continue;
+      if (k == 0) J.ex[tk.row0 + r] = e;
+      if (k < kend) store4(tk.row0 + r, k, e, x[it]);
+    }
+    return;
+  }
+  const int r = cta * (kSplitThreads / 32) + warp;
+  if (r >= tk.rows) return;
+  const double* xr = J.X + tk.base + (long long)r * tk.s_r;
+  unsigned long long mx = 0;
+  const bool keep = tk.K <= kSplitRowMax;
+  if (keep) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) load4(xr, g * 128 + lane * 4, x[g]);
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mx = max(mx, abs_bits(x[g][j]));
+  } else {
+#pragma unroll 4
+    for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_bits(__double_as_longlong(xr[k])));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const int e = int(mx >> 52) - 1022;
+  const long long grow = tk.row0 + r;
+  if (lane == 0) J.ex[grow] = e;
+  if (keep) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int k = g * 128 + lane * 4;
+      if (k < kend) store4(grow, k, e, x[g]);
+    }
+  } else {
+    for (int k = lane * 4; k < kend; k += 128) {
+      unsigned long long v[4];
+      load4(xr, k, v);
+      store4(grow, k, e, v);
+    }
+  }
+}
+
+// One cluster, 32 interleaved rows (lane l: row r0 + l at xr[k s_k]).
+template <int S>
+__device__ __forceinline__ void split_cols(const SplitJob& J, const SplitTask& tk, int r0, int crank, int csize,
+                                           int kpitch) {
+  __shared__ unsigned long long wmax[kSplitThreads / 32][32];
+  __shared__ unsigned long long cmax[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = r0 + lane;
+  const bool live = r < tk.rows;
+  const double* xr = J.X + tk.base + (live ? r : tk.rows - 1);
+  const int step = csize * (kSplitThreads / 32) * 16;        // k per pass of the cluster
+  const int k0 = (crank * (kSplitThreads / 32) + warp) * 16;  // this thread's first 16
+  auto load16 = [&](int k, unsigned long long (&v)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      v[j] = k + j < tk.K ? (unsigned long long)__double_as_longlong(xr[(long long)(k + j) * tk.s_k]) : 0ull;
+  };
+  unsigned long long x[16];
+  unsigned long long mx = 0;
+  // the first pass's values stay in registers (the only pass when the
+  // cluster covers K), the others are read again below
+  load16(k0, x);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) mx = max(mx, abs_bits(x[j]));
+  for (int k = k0 + step; k < tk.K; k += step) {
+    unsigned long long v[16];
+    load16(k, v);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) mx = max(mx, abs_bits(v[j]));
+  }
+  wmax[warp][lane] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSplitThreads / 32; ++w) mx = max(mx, wmax[w][lane]);
+  if (csize > 1) {
+    cg::cluster_group cl = cg::this_cluster();
+    if (warp == 0) cmax[lane] = mx;
+    cl.sync();
+    for (int c = 0; c < csize; ++c) mx = max(mx, cl.map_shared_rank(cmax, c)[lane]);
+    cl.sync();  // no CTA leaves while another still reads its maxima
+  }
+  const int e = int(mx >> 52) - 1022;
+  const long long grow = tk.row0 + r;
+  if (live && crank == 0 && warp == 0) J.ex[grow] = e;
+  if (!live) return;
+  const int kend = (tk.K + 31) & ~31;
+  for (int k = k0; k < kend; k += step) {
+    if (k != k0) load16(k, x);
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+      uint32_t f[8][S];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) split_digits<S>(x[h + j], e, f[j]);
+#pragma unroll
+      for (int i = 0; i < S; ++i)
+        *reinterpret_cast<uint4*>(J.S + ((long long)i * J.rows_total + grow) * kpitch + k + h) =
+            make_uint4(pack_bf16(f[0][i], f[1][i]), pack_bf16(f[2][i], f[3][i]), pack_bf16(f[4][i], f[5][i]),
+                       pack_bf16(f[6][i], f[7][i]));
+    }
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob ja, SplitJob jb, int ga, int gab,
+                                                                    int csize, int kpitch, ZeroJob zj) {
   if (int(blockIdx.x) >= gab) {
-    zero_part(zj, int(blockIdx.x) - gab);
+    const int z = int(blockIdx.x) - gab;
+    if (z < zj.nz * kZeroCtas) zero_part(zj, z);
     return;
   }
   const bool is_a = int(blockIdx.x) < ga;
   const SplitJob& J = is_a ? ja : jb;
-  const SplitTask* __restrict__ tasks = J.tasks;
-  const int ntasks = J.ntasks, rows_total = J.rows_total;
-  const double* __restrict__ X = J.X;
-  __nv_bfloat16* __restrict__ Sd = J.S;
-  int* __restrict__ ex = J.ex;
-  const int warp_g = ((int(blockIdx.x) - (is_a ? 0 : ga)) * int(blockDim.x) + int(threadIdx.x)) >> 5;
+  const int cta = int(blockIdx.x) - (is_a ? 0 : ga);
+  int lo = 0, hi = J.ntasks - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (J.tasks[mid].cta0 <= cta) lo = mid;
+    else hi = mid - 1;
+  }
+  const SplitTask tk = J.tasks[lo];
+  const int c = cta - tk.cta0;
+  if (tk.s_k != 1 && tk.s_r == 1) {
+    // (a task's CTAs are whole clusters: the branch is the same for all of one)
+    const int r0 = (c / csize) * 32;
+    if (r0 < tk.rows) split_cols<S>(J, tk, r0, c % csize, csize, kpitch);
+    return;
+  }
+  if (tk.s_k == 1) {
+    split_rows<S>(J, tk, c, kpitch);
+    return;
+  }
+  const int r = c * (kSplitThreads / 32) + int(threadIdx.x >> 5);
+  if (r >= tk.rows) return;
+  // any other strides: one warp per row, lanes along k
   const int lane = threadIdx.x & 31;
-  if (warp_g >= rows_total || ntasks == 0) return;
-  // locate (task, row): last task whose first row is <= warp_g
-  int tlo = 0, thi = ntasks - 1;
-  while (tlo < thi) {
-    const int mid = (tlo + thi + 1) >> 1;
-    if (tasks[mid].row0 <= warp_g) tlo = mid;
-    else thi = mid - 1;
-  }
-  const int t = tlo;
-  const int r = warp_g - tasks[t].row0;
-  if (r < 0 || r >= tasks[t].rows) return;
-  const SplitTask tk = tasks[t];
-  const double* xr = X + tk.base + (long long)r * tk.s_r;
+  const double* xr = J.X + tk.base + (long long)r * tk.s_r;
   unsigned long long mx = 0;
-  for (int k = lane; k < tk.K; k += 32) {
-    unsigned long long b = __double_as_longlong(xr[(long long)k * tk.s_k]) & 0x7FFFFFFFFFFFFFFFull;
-    mx = b > mx ? b : mx;
-  }
+  for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_bits(__double_as_longlong(xr[(long long)k * tk.s_k])));
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = y > mx ? y : mx;
-  }
-  // |x| < 2^e for every entry of the row (e from the largest exponent field)
-  const int emax = int(mx >> 52);
-  const int e = emax - 1022;
-  const int grow = tk.row0 + r;
-  if (lane == 0) ex[grow] = e;
-  const int kend = (tk.K + 31) & ~31;
-  for (int k = lane; k < kend; k += 32) {
-    long long Xi = 0;
-    if (k < tk.K && mx != 0) {
-      const unsigned long long b = __double_as_longlong(xr[(long long)k * tk.s_k]);
-      const int E = int((b >> 52) & 0x7FF);
-      if (E != 0) {  // subnormals of a row with a normal maximum are below 2^-44 of it
-        const long long m = (long long)((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull);
-        // X = round(m * 2^(E - 1075 - e + 9 S - 1)), |X| < 2^(9 S - 1)
-        const int sh = E - 1075 - e + 9 * S - 1;
-        if (sh >= 0) {
-          Xi = m << sh;
-        } else if (sh > -64) {
-          const int rs = -sh;
-          Xi = (m + (1ll << (rs - 1))) >> rs;
-        }
-        if (b >> 63) Xi = -Xi;
-      }
-    }
-    // signed digits: X = sum_i a_i 2^(9 (S - 1 - i)), |a_i| <= 256
-    int dig[S];
-#pragma unroll
-    for (int i = S - 1; i >= 1; --i) {
-      long long lo = ((Xi + 256) & 511) - 256;
-      dig[i] = int(lo);
-      Xi = (Xi - lo) >> 9;
-    }
-    dig[0] = int(Xi);
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const int e = int(mx >> 52) - 1022;
+  const long long grow = tk.row0 + r;
+  if (lane == 0) J.ex[grow] = e;
+  for (int k = lane; k < ((tk.K + 31) & ~31); k += 32) {
+    uint32_t f[S];
+    split_digits<S>(k < tk.K ? (unsigned long long)__double_as_longlong(xr[(long long)k * tk.s_k]) : 0ull, e, f);
 #pragma unroll
     for (int i = 0; i < S; ++i)
-      Sd[((long long)i * rows_total + grow) * kpitch + k] = __int2bfloat16_rn(dig[i]);
+      J.S[((long long)i * J.rows_total + grow) * kpitch + k] = __ushort_as_bfloat16((unsigned short)(f[i] >> 16));
   }
 }
 
@@ -736,31 +985,6 @@ __global__ void __launch_bounds__(256) pack_split_kernel(PackJob ja, PackJob jb,
     }
     return base[o];
   };
-  // the digits of x against the row exponent e (the same integer
-  // arithmetic as ozaki_split_kernel<S>)
-  auto digits = [&](double x, int e, int (&dig)[S]) {
-    long long Xi = 0;
-    const unsigned long long b = __double_as_longlong(x);
-    const int E = int((b >> 52) & 0x7FF);
-    if (E != 0) {
-      const long long m = (long long)((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull);
-      const int sh = E - 1075 - e + 9 * S - 1;
-      if (sh >= 0) {
-        Xi = m << sh;
-      } else if (sh > -64) {
-        const int rs = -sh;
-        Xi = (m + (1ll << (rs - 1))) >> rs;
-      }
-      if (b >> 63) Xi = -Xi;
-    }
-#pragma unroll
-    for (int i = S - 1; i >= 1; --i) {
-      const long long lo9 = ((Xi + 256) & 511) - 256;
-      dig[i] = int(lo9);
-      Xi = (Xi - lo9) >> 9;
-    }
-    dig[0] = int(Xi);
-  };
   const int kend = (G.K + 31) & ~31;
   enter(0);
   unsigned long long mx = 0;
@@ -778,16 +1002,11 @@ __global__ void __launch_bounds__(256) pack_split_kernel(PackJob ja, PackJob jb,
   si = 0;
   enter(0);
   for (int k = lane; k < kend; k += 32) {
-    int dig[S];
-    if (k < G.K && mx != 0) {
-      digits(load(k), e, dig);
-    } else {
-#pragma unroll
-      for (int i = 0; i < S; ++i) dig[i] = 0;
-    }
+    uint32_t f[S];
+    split_digits<S>(k < G.K ? (unsigned long long)__double_as_longlong(load(k)) : 0ull, e, f);
 #pragma unroll
     for (int i = 0; i < S; ++i)
-      J.S[((long long)i * J.rows_total + grow) * kpitch + k] = __int2bfloat16_rn(dig[i]);
+      J.S[((long long)i * J.rows_total + grow) * kpitch + k] = __ushort_as_bfloat16((unsigned short)(f[i] >> 16));
   }
 }
 
@@ -812,14 +1031,17 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-static CUtensorMap make_map(void* base, int kpitch, int rows, int box_rows) {
+// Map of a split buffer (S slices of `rows` rows of kpitch): one box is all
+// slices of box_rows rows of a K chunk.  Rows past a slice's end belong to
+// the next slice (past the last one: to the buffer's spare rows).
+static CUtensorMap make_map(void* base, int kpitch, int rows, int box_rows, int S) {
   CUtensorMap m;
   std::memset(&m, 0, sizeof(m));
-  cuuint64_t dims[2] = {cuuint64_t(kpitch), cuuint64_t(rows)};
-  cuuint64_t strides[1] = {cuuint64_t(kpitch) * 2};
-  cuuint32_t box[2] = {cuuint32_t(oz::kTK), cuuint32_t(box_rows)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
+  cuuint64_t dims[3] = {cuuint64_t(kpitch), cuuint64_t(std::max(rows, box_rows)), cuuint64_t(S)};
+  cuuint64_t strides[2] = {cuuint64_t(kpitch) * 2, cuuint64_t(rows) * kpitch * 2};
+  cuuint32_t box[3] = {cuuint32_t(oz::kTK), cuuint32_t(box_rows), cuuint32_t(S)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   BST_REQUIRE(r == CUDA_SUCCESS, BST_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string(int(r)));
@@ -834,6 +1056,8 @@ struct OzakiPlan {
   oz::Tile* d_tiles = nullptr;
   oz::SplitTask *d_sa = nullptr, *d_sb = nullptr;
   int nsa = 0, nsb = 0;
+  int split_ca = 0, split_cb = 0;  // CTAs of the split of A and of B
+  int split_cluster = 1;           // CTAs that share 32 interleaved rows of an operand
   __nv_bfloat16 *SA = nullptr, *SB = nullptr;
   int *eA = nullptr, *eB = nullptr;
   CUtensorMap mapA, mapB;
@@ -1031,20 +1255,24 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
       q.ct_off = sc->ct_off[pi];
       q.bb_off = sc->bb_off[pi];
     }
-    sa.push_back({g.M, g.K, P->rowsA, 0, g.a_off, g.a_m, g.a_k});
-    sb.push_back({g.N, g.K, P->rowsB, 0, g.b_off, g.b_n, g.b_k});
+    // (a one-column or one-row operand counts as contiguous)
+    sa.push_back({g.M, g.K, P->rowsA, 0, g.a_off, g.a_m, g.K <= 1 ? 1 : g.a_k});
+    sb.push_back({g.N, g.K, P->rowsB, 0, g.b_off, g.b_n, g.K <= 1 ? 1 : g.b_k});
     P->rowsA += g.M;
     P->rowsB += g.N;
     const int pi = int(hp.size());
     hp.push_back(q);
+    auto add_tile = [&](int i, const oz::Prob& o, int m0, int n0) {
+      ht.push_back({i, m0, n0, (o.K + oz::kTK - 1) / oz::kTK, o.arow + m0, o.brow + n0, {0, 0}});
+    };
     if (g.K == 0) {
       zp.push_back(g);
     } else if (order == 2) {
       for (int n0 = 0; n0 < g.N; n0 += TN)
-        for (int m0 = 0; m0 < g.M; m0 += oz::kTM) ht.push_back({pi, m0, n0, 0});
+        for (int m0 = 0; m0 < g.M; m0 += oz::kTM) add_tile(pi, q, m0, n0);
     } else {
       for (int m0 = 0; m0 < g.M; m0 += oz::kTM)
-        for (int n0 = 0; n0 < g.N; n0 += TN) ht.push_back({pi, m0, n0, 0});
+        for (int n0 = 0; n0 < g.N; n0 += TN) add_tile(pi, q, m0, n0);
     }
     P->flops += 2.0 * double(g.M) * g.N * g.K;
     P->split_bytes += double(g.M + g.N) * g.K * (8.0 + 2.0 * S) + 4.0 * (g.M + g.N);
@@ -1056,6 +1284,26 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   P->ntiles = int(ht.size());
   P->nsa = int(sa.size());
   P->nsb = int(sb.size());
+  // CTAs of the split: eight contiguous rows each, or a cluster per 32
+  // interleaved rows (128 k per CTA and pass: one pass up to K = 1024)
+  int kcol = 0;
+  for (auto* v : {&sa, &sb})
+    for (auto& t : *v)
+      if (t.s_k != 1 && t.s_r == 1) kcol = std::max(kcol, t.K);
+  while (P->split_cluster < 8 && P->split_cluster * 128 < kcol) P->split_cluster *= 2;
+  const int sc_ = P->split_cluster;
+  auto place = [&](std::vector<oz::SplitTask>& v) {
+    int cta = 0;
+    for (auto& t : v) {
+      t.cta0 = cta;
+      const int per = t.s_k == 1 ? oz::split_cta_rows(t.K) : 8;
+      const int n = t.s_k != 1 && t.s_r == 1 ? (t.rows + 31) / 32 * sc_ : (t.rows + per - 1) / per;
+      cta += (n + sc_ - 1) / sc_ * sc_;
+    }
+    return cta;
+  };
+  P->split_ca = place(sa);
+  P->split_cb = place(sb);
   BST_REQUIRE(int64_t(P->rowsA) * S < (1ll << 31) && int64_t(P->rowsB) * S < (1ll << 31),
               BST_E_UNSUPPORTED, "Ozaki GEMM: too many rows");
   auto up = [](auto** dst, const auto& v) {
@@ -1090,9 +1338,9 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   BST_CUDA(cudaMemset(P->SB, 0, sizeof(__nv_bfloat16) * rb * P->kpitch));
   BST_CUDA(cudaMalloc(&P->eA, sizeof(int) * std::max(P->rowsA, 1)));
   BST_CUDA(cudaMalloc(&P->eB, sizeof(int) * std::max(P->rowsB, 1)));
-  P->mapA = make_map(P->SA, P->kpitch, int(ra), oz::kTM);
-  P->mapB = make_map(P->SB, P->kpitch, int(rb), TN);
-  if (P->ab_same) P->mapBA = make_map(P->SA, P->kpitch, int(ra), TN);
+  P->mapA = make_map(P->SA, P->kpitch, std::max(P->rowsA, 1), oz::kTM, S);
+  P->mapB = make_map(P->SB, P->kpitch, std::max(P->rowsB, 1), TN, S);
+  if (P->ab_same) P->mapBA = make_map(P->SA, P->kpitch, std::max(P->rowsA, 1), TN, S);
   return P;
 }
 
@@ -1125,16 +1373,27 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
     // the split of both operands; the K == 0 problems' outputs are written
     // by the same launch
     ProfScope ps(ctx, s, "split_bf16", 0.0, b_from_a ? 0.5 * P->split_bytes : P->split_bytes);
-    const int wa = (split_a && P->ntiles) ? P->rowsA : 0, wb = (b_from_a || !P->ntiles) ? 0 : P->rowsB;
-    const int ga = (wa + 7) / 8, gb = (wb + 7) / 8;  // 8 rows (warps) per CTA
-    const int gz = P->nzprobs * oz::kZeroCtas;
+    const int cs = P->split_cluster;
+    const int ga = (split_a && P->ntiles) ? P->split_ca : 0, gb = (b_from_a || !P->ntiles) ? 0 : P->split_cb;
+    const int gz = (P->nzprobs * oz::kZeroCtas + cs - 1) / cs * cs;
     const oz::ZeroJob zj{P->nzprobs, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
     if (ga + gb + gz > 0) {
       const oz::SplitJob ja{P->d_sa, P->nsa, P->rowsA, A, P->SA, P->eA};
       const oz::SplitJob jb{P->d_sb, P->nsb, P->rowsB, B, P->SB, P->eB};
-      if (P->S == 5) oz::ozaki_split_kernel<5><<<ga + gb + gz, 256, 0, s>>>(ja, jb, ga, ga + gb, P->kpitch, zj);
-      else oz::ozaki_split_kernel<3><<<ga + gb + gz, 256, 0, s>>>(ja, jb, ga, ga + gb, P->kpitch, zj);
-      BST_CUDA(cudaGetLastError());
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(unsigned(ga + gb + gz));
+      cfg.blockDim = dim3(oz::kSplitThreads);
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = unsigned(cs);
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = cs > 1 ? 1 : 0;
+      if (P->S == 5)
+        BST_CUDA(cudaLaunchKernelEx(&cfg, oz::ozaki_split_kernel<5>, ja, jb, ga, ga + gb, cs, P->kpitch, zj));
+      else
+        BST_CUDA(cudaLaunchKernelEx(&cfg, oz::ozaki_split_kernel<3>, ja, jb, ga, ga + gb, cs, P->kpitch, zj));
       count_launch(ctx);
     }
     if (P->ntiles == 0) return;
@@ -1145,8 +1404,8 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
   const CUtensorMap& mB = b_from_a ? P->mapBA : P->mapB;
   const int* eB = b_from_a ? P->eA : P->eB;
   auto launch = [&](auto kern, size_t smem) {
-    kern<<<grid, oz::kThreads, smem, s>>>(P->mapA, mB, P->d_probs, P->d_tiles, P->ntiles, P->eA, eB, P->rowsA,
-                                           P->rowsB, C, sc, ctx->d_err, spin);
+    kern<<<grid, oz::kThreads, smem, s>>>(P->mapA, mB, P->d_probs, P->d_tiles, P->ntiles, P->eA, eB, C, sc,
+                                         ctx->d_err, spin);
   };
   if (P->S == 5 && P->TN == 64) {
     set_kernel_attrs<5, 64>();
