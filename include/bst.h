@@ -341,8 +341,9 @@ BST_API bst_status bst_contract_noalloc(bst_ctx ctx, bst_layout A, const double*
  * order) is its innermost leg: one gathers every operand row of every
  * contraction from its blocks and splits it into digits, one grouped GEMM
  * writes every output block in its epilogue (alpha, beta applied there);
- * otherwise three: one gather of both operands' sector matrices, one split,
- * the GEMM.  BST_FP64 takes one gather, one grouped DMMA GEMM and one
+ * otherwise three: one gather and split of the A operands, one of the B
+ * operands,
+ * and the GEMM.  BST_FP64 takes one gather, one grouped DMMA GEMM and one
  * scatter.  The first call with a given list of layouts builds and
  * caches the plan, and the first call with a given list of data pointers
  * uploads a pointer table (both allocate and synchronise); a repeated call

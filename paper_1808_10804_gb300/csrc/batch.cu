@@ -4,12 +4,14 @@
 // contraction alone is small (Sec. 2: the block pairs of a contraction are
 // independent of one another, and so are separate contractions).
 //
-// Tensor-core arithmetic: two launches.  One pack launch gathers the rows
-// of every contraction's operand sector matrices straight from the operand
-// tensors and splits them into digits (each segment carries the index of
-// its tensor in a device pointer table); one GEMM launch over all problems
-// writes every product into its contraction's output blocks (the scatter
-// tables address each output relative to the first output's pointer).
+// Tensor-core arithmetic: the pack gathers the rows of every contraction's
+// operand sector matrices straight from the operand tensors and splits them
+// into digits (each segment carries the index of its tensor in a device
+// pointer table), in one launch when every operand's innermost leg is its
+// last contracted one, else in one launch per operand; one GEMM launch over
+// all problems writes every product into its contraction's output blocks
+// (the scatter tables address each output relative to the first output's
+// pointer).
 // FP64: one gather per operand into combined sector-matrix buffers, one
 // grouped DMMA GEMM, one scatter.
 //
@@ -53,7 +55,6 @@ struct BatchPlan {
   // one gather of both operands (B's tasks point past A's matrices and at
   // the second half of the pointer table), the FP64 path's scatter
   BatchRel rab, rc;
-  bool packed = false;  // every contraction ozaki_packable
   std::vector<GemmProb> probs;
   DevGemm g;
   // schedule chosen by the autotuner (defaults until tuned)
@@ -143,7 +144,7 @@ static OzakiPlan* batch_oz(Ctx* ctx, BatchPlan* bp, int order, int S, int TN) {
   const std::string key = std::to_string(S) + "/" + std::to_string(TN) + "/" + std::to_string(order);
   auto it = bp->ozp.find(key);
   if (it != bp->ozp.end()) return it->second;
-  OzakiPlan* P = ozaki_batch_plan(ctx, bp->plans, bp->probs, order, S, TN, bp->packed, &bp->bb_rel, &bp->bb_src);
+  OzakiPlan* P = ozaki_batch_plan(ctx, bp->plans, bp->probs, order, S, TN, &bp->bb_rel, &bp->bb_src);
   bp->ozp[key] = P;
   return P;
 }
@@ -184,7 +185,7 @@ static void autotune(Ctx* ctx, BatchPlan* bp, double* const* bases, size_t n, bs
   const bool prof = ctx->prof;
   ctx->prof = false;
   char line[256];
-  if (!bp->tuned_rel && !(prec != BST_FP64 && bp->packed)) {
+  if (!bp->tuned_rel && prec == BST_FP64) {
     float best = 1e30f;
     int bc = 2048;
     for (int c : kChunkChoices) {
@@ -204,7 +205,7 @@ static void autotune(Ctx* ctx, BatchPlan* bp, double* const* bases, size_t n, bs
   }
   const int pi = int(prec);
   if (!bp->tuned[pi]) {
-    if (!(prec != BST_FP64 && bp->packed)) launch_rel(ctx, bp->rab, bases, bp->Am, 0, 1.0, 0.0, s);
+    if (prec == BST_FP64) launch_rel(ctx, bp->rab, bases, bp->Am, 0, 1.0, 0.0, s);
     // the tensor-core candidates write every output through the scatter
     // epilogue: while tuning they write a scratch copy of the outputs
     double* scratch = nullptr;
@@ -234,7 +235,7 @@ static void autotune(Ctx* ctx, BatchPlan* bp, double* const* bases, size_t n, bs
           t = time_ms(s, 3, [&] { launch_gemm_f64(ctx, bp->g, bp->Am, bp->Bm, bp->Cm, s); });
         } else {
           OzakiPlan* P = batch_oz(ctx, bp, o, S, tn);
-          t = time_ms(s, 3, [&] { run_ozaki_batch(ctx, P, bases, int(n), bp->Am, bp->Bm, scratch, sbb, 1.0, 0.0, s); });
+          t = time_ms(s, 3, [&] { run_ozaki_batch(ctx, P, bases, int(n), scratch, sbb, 1.0, 0.0, s); });
         }
         snprintf(line, sizeof(line), "batch %p %s tile 128x%d order %d: %.4f ms\n", (void*)bp, kname,
                  prec == BST_FP64 ? kF64TileN : tn, o, t);
@@ -276,10 +277,8 @@ static BatchPlan* get_batch_plan(Ctx* ctx, const std::vector<Layout*>& A, const 
   bp->plans = plans;
   const int32_t n = int32_t(plans.size());
   std::vector<BatchTask> btasks;
-  bp->packed = true;
   for (size_t i = 0; i < plans.size(); ++i) {
     ContractPlan* p = plans[i];
-    bp->packed = bp->packed && ozaki_packable(p);
     for (auto t : p->va.tasks) {
       t.mat_base += bp->amat;
       bp->rab.host.push_back({t, int32_t(i), 0});
@@ -354,10 +353,8 @@ void contract_batched(Ctx* ctx, const std::vector<Layout*>& A, const std::vector
     launch_rel(ctx, bp->rc, bases + 2 * n, bp->Cm, 1, alpha, beta, s);
     return;
   }
-  // packed: one pack launch over every operand; else one gather of both
-  // operands and one split; then one GEMM whose epilogue writes every
+  // the pack of the operands, then one GEMM whose epilogue writes every
   // output block (alpha, beta applied there)
-  if (!bp->packed) launch_rel(ctx, bp->rab, bases, bp->Am, 0, 1.0, 0.0, s);
   const int pi = int(prec);
   OzakiPlan* P = batch_oz(ctx, bp, bp->order[pi], ozaki_slices(prec), bp->tn[pi] ? bp->tn[pi] : ozaki_pick_tn(bp->probs));
   if (!it->second.bbase) {
@@ -366,7 +363,7 @@ void contract_batched(Ctx* ctx, const std::vector<Layout*>& A, const std::vector
     BST_CUDA(cudaMalloc(&it->second.bbase, sizeof(long long) * std::max<size_t>(abs.size(), 1)));
     BST_CUDA(cudaMemcpy(it->second.bbase, abs.data(), sizeof(long long) * abs.size(), cudaMemcpyHostToDevice));
   }
-  run_ozaki_batch(ctx, P, bases, int(n), bp->Am, bp->Bm, c[0], it->second.bbase, alpha, beta, s);
+  run_ozaki_batch(ctx, P, bases, int(n), c[0], it->second.bbase, alpha, beta, s);
 }
 
 }  // namespace bst

@@ -21,8 +21,22 @@
 // 128 x 32) output tiles; warp 0 drives TMA (64-byte swizzled K-major tiles,
 // a ring of 3 stages for five slices, up to 6 for three), warp 1 issues
 // tcgen05.mma from one thread (the 15 digit products of a 16-K step as 8
-// products, each an A slice times a run of stacked B slices), warps 2..9
-// drain tensor memory.  Every wait of the pipeline
+// products, each an A slice times a run of stacked B slices), warps 2..17
+// drain tensor memory.
+//
+// What bounds it: a 32-K chunk's 16 products take the tensor core 1014 cycles
+// (measured alone; 960 at its peak rate), a chunk of a running tile 1450 with
+// the epilogue idle and 1850 with it.  The rest is the issuing thread, whose
+// products queue only a few deep: whatever it does between the last product
+// of a chunk and the first of the next leaves the tensor core idle, and it
+// shares its issue slots with the epilogue.  Hence counters in place of
+// divisions, tile tables that hold all a role needs, one copy per operand and
+// chunk, barriers looked at ahead of time, and no conversion instruction in
+// the epilogue that an addition replaces.  2432 x 2432 x 2432, five digits:
+// 430 -> 375 us (1.15 PFLOP/s of digit products); four of 2048 x 2048 x 512:
+// 347 -> 287 us; 2432^3 with three digits: 292 -> 229 us.
+//
+// Every wait of the pipeline
 // is bounded by the launch's spin limit: on expiry the kernel records
 // BST_E_TIMEOUT in the context's error word and every role leaves its loop;
 // before tensor memory is freed and the CTA exits, the TMA copies it has
@@ -105,7 +119,7 @@ struct Tile {
 
 struct SplitTask {
   int32_t rows, K;
-  int32_t row0, cta0;  // first row in the split buffer, first CTA of the task in its operand's range
+  int32_t row0, pad;  // first row in the split buffer
   int64_t base, s_r, s_k;
 };
 
@@ -605,7 +619,8 @@ __device__ __forceinline__ void zero_part(const ZeroJob& z, int cta) {
 // Split FP64 rows into S BF16 digit slices (integer arithmetic on the bit
 // pattern); digits for k in [K, roundup(K, 32)) are 0.  One launch splits
 // both operands: CTAs [0, ga) take the tasks of A, the next gb those of B;
-// a CTA finds its task by binary search over the tasks' first CTAs.
+// a table gives every CTA its task (a search over hundreds of tasks is a
+// chain of that many loads, longer than the CTA's work).
 //
 // The kernel moves 8 bytes in and 2 S out per element, so what bounds it is
 // how the rows lie in memory:
@@ -623,7 +638,8 @@ __device__ __forceinline__ void zero_part(const ZeroJob& z, int cta) {
 //     32 sectors of which 8 bytes each were used.
 struct SplitJob {
   const SplitTask* tasks;
-  int ntasks, rows_total;
+  const int2* ctas;  // per CTA: its task and its number inside it
+  int rows_total;
   const double* X;
   __nv_bfloat16* S;
   int* ex;
@@ -636,34 +652,56 @@ constexpr int kSplitRowMax = 512;  // longest contiguous row kept in registers (
 // (|x| < 2^e), as the bit patterns of the FP32 numbers (BF16 in the upper
 // half): X = round(|x| 2^(9 S - 1 - e)) with the sign of x, X = sum_i a_i
 // 2^(9 (S - 1 - i)) with a_i in [-256, 255] for i > 0.  Adding 256 at every
-// digit but the first makes all of them non-negative bit fields.
+// digit but the first makes those bit fields; a field under the pattern of
+// 1.5 2^23 is that number plus the field, so one subtraction gives the digit.
 template <int S>
 __device__ __forceinline__ void split_digits(unsigned long long b, int e, uint32_t (&f)[S]) {
-  const int E = int(b >> 52) & 0x7FF;
-  long long X = 0;
-  if (E != 0) {  // subnormals of a row with a normal maximum are below 2^-44 of it
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-    // E <= e + 1022 and 9 S - 1 <= 44: the shift is to the right by 9 or more
-    const int rs = 1075 + e - E - (9 * S - 1);
-    if (rs < 64) X = (long long)((m + (1ull << (rs - 1))) >> rs);
-    if ((long long)b < 0) X = -X;
-  }
+  const uint32_t hi = uint32_t(b >> 32);
+  const int E = int(hi >> 20) & 0x7FF;
+  // E <= e + 1022 and 9 S - 1 <= 44: the shift is to the right by 9 or more
+  const int rs = 1074 + e - (9 * S - 1) - E;
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  long long X = (long long)(((m >> (rs & 63)) + 1) >> 1);  // half a unit up: round to nearest
+  if (rs > 62 || E == 0) X = 0;  // (subnormals of a row with a normal maximum are below 2^-44 of it)
+  if (int(hi) < 0) X = -X;
   long long bias = 0;
 #pragma unroll
   for (int i = 0; i < S - 1; ++i) bias |= 256ll << (9 * i);
   X += bias;
 #pragma unroll
   for (int i = S - 1; i >= 1; --i)
-    // a + 2^23 + 2^22 as an FP32 integer, minus that constant: a, exact
-    f[i] = __float_as_uint(__uint_as_float(0x4B400000u - 256u + (uint32_t(X >> (9 * (S - 1 - i))) & 511u)) -
-                           12582912.0f);
+    f[i] = __float_as_uint(__uint_as_float((uint32_t(X >> (9 * (S - 1 - i))) & 511u) | 0x4B400000u) - 12583168.0f);
   f[0] = __float_as_uint(__uint_as_float(0x4B400000u + uint32_t(int(X >> (9 * (S - 1))))) - 12582912.0f);
 }
 
 // two BF16 numbers (the upper halves of their FP32 patterns), lower k first
 __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
 
-__device__ __forceinline__ unsigned long long abs_bits(unsigned long long b) { return b & 0x7FFFFFFFFFFFFFFFull; }
+// |x|'s upper word: enough for a row's exponent
+__device__ __forceinline__ uint32_t abs_hi(unsigned long long b) { return uint32_t(b >> 32) & 0x7FFFFFFFu; }
+__device__ __forceinline__ int row_exp(uint32_t mx) { return int(mx >> 20) - 1022; }  // |x| < 2^e
+
+// The digits of 16 consecutive k of one row.
+template <int S>
+__device__ __forceinline__ void store16(__nv_bfloat16* Sd, int rows_total, long long grow, int kpitch, int k, int e,
+                                        const unsigned long long (&x)[16]) {
+#pragma unroll
+  for (int h = 0; h < 16; h += 8) {
+    uint32_t w[4][S];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      uint32_t f[S], g[S];
+      split_digits<S>(x[h + j], e, f);
+      split_digits<S>(x[h + j + 1], e, g);
+#pragma unroll
+      for (int i = 0; i < S; ++i) w[j / 2][i] = pack_bf16(f[i], g[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+      *reinterpret_cast<uint4*>(Sd + ((long long)i * rows_total + grow) * kpitch + k + h) =
+          make_uint4(w[0][i], w[1][i], w[2][i], w[3][i]);
+  }
+}
 
 // Rows contiguous along k: how many a CTA takes.  Four k per lane: rows up
 // to 32 (64, 128) long take 8 (16, 32) lanes and a warp does four passes of
@@ -710,11 +748,11 @@ __device__ __forceinline__ void split_rows(const SplitJob& J, const SplitTask& t
     }
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-      unsigned long long mx = max(max(abs_bits(x[it][0]), abs_bits(x[it][1])),
-                                  max(abs_bits(x[it][2]), abs_bits(x[it][3])));
+      uint32_t mx = max(max(abs_hi(x[it][0]), abs_hi(x[it][1])),
+                                  max(abs_hi(x[it][2]), abs_hi(x[it][3])));
       for (int o = lpr >> 1; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       // |x| < 2^e for every entry of the row (e from the largest exponent field)
-      const int e = int(mx >> 52) - 1022;
+      const int e = row_exp(mx);
       const int r = r0 + it * rpw;
       if (r >= tk.rows) continue;
       if (k == 0) J.ex[tk.row0 + r] = e;
@@ -725,7 +763,7 @@ __device__ __forceinline__ void split_rows(const SplitJob& J, const SplitTask& t
   const int r = cta * (kSplitThreads / 32) + warp;
   if (r >= tk.rows) return;
   const double* xr = J.X + tk.base + (long long)r * tk.s_r;
-  unsigned long long mx = 0;
+  uint32_t mx = 0;
   const bool keep = tk.K <= kSplitRowMax;
   if (keep) {
 #pragma unroll
@@ -733,14 +771,14 @@ __device__ __forceinline__ void split_rows(const SplitJob& J, const SplitTask& t
 #pragma unroll
     for (int g = 0; g < 4; ++g)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) mx = max(mx, abs_bits(x[g][j]));
+      for (int j = 0; j < 4; ++j) mx = max(mx, abs_hi(x[g][j]));
   } else {
 #pragma unroll 4
-    for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_bits(__double_as_longlong(xr[k])));
+    for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_hi(__double_as_longlong(xr[k])));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int e = int(mx >> 52) - 1022;
+  const int e = row_exp(mx);
   const long long grow = tk.row0 + r;
   if (lane == 0) J.ex[grow] = e;
   if (keep) {
@@ -762,8 +800,8 @@ __device__ __forceinline__ void split_rows(const SplitJob& J, const SplitTask& t
 template <int S>
 __device__ __forceinline__ void split_cols(const SplitJob& J, const SplitTask& tk, int r0, int crank, int csize,
                                            int kpitch) {
-  __shared__ unsigned long long wmax[kSplitThreads / 32][32];
-  __shared__ unsigned long long cmax[32];
+  __shared__ uint32_t wmax[kSplitThreads / 32][32];
+  __shared__ uint32_t cmax[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = r0 + lane;
   const bool live = r < tk.rows;
@@ -776,17 +814,17 @@ __device__ __forceinline__ void split_cols(const SplitJob& J, const SplitTask& t
       v[j] = k + j < tk.K ? (unsigned long long)__double_as_longlong(xr[(long long)(k + j) * tk.s_k]) : 0ull;
   };
   unsigned long long x[16];
-  unsigned long long mx = 0;
+  uint32_t mx = 0;
   // the first pass's values stay in registers (the only pass when the
   // cluster covers K), the others are read again below
   load16(k0, x);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) mx = max(mx, abs_bits(x[j]));
+  for (int j = 0; j < 16; ++j) mx = max(mx, abs_hi(x[j]));
   for (int k = k0 + step; k < tk.K; k += step) {
     unsigned long long v[16];
     load16(k, v);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) mx = max(mx, abs_bits(v[j]));
+    for (int j = 0; j < 16; ++j) mx = max(mx, abs_hi(v[j]));
   }
   wmax[warp][lane] = mx;
   __syncthreads();
@@ -799,24 +837,14 @@ __device__ __forceinline__ void split_cols(const SplitJob& J, const SplitTask& t
     for (int c = 0; c < csize; ++c) mx = max(mx, cl.map_shared_rank(cmax, c)[lane]);
     cl.sync();  // no CTA leaves while another still reads its maxima
   }
-  const int e = int(mx >> 52) - 1022;
+  const int e = row_exp(mx);
   const long long grow = tk.row0 + r;
   if (live && crank == 0 && warp == 0) J.ex[grow] = e;
   if (!live) return;
   const int kend = (tk.K + 31) & ~31;
   for (int k = k0; k < kend; k += step) {
     if (k != k0) load16(k, x);
-#pragma unroll
-    for (int h = 0; h < 16; h += 8) {
-      uint32_t f[8][S];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) split_digits<S>(x[h + j], e, f[j]);
-#pragma unroll
-      for (int i = 0; i < S; ++i)
-        *reinterpret_cast<uint4*>(J.S + ((long long)i * J.rows_total + grow) * kpitch + k + h) =
-            make_uint4(pack_bf16(f[0][i], f[1][i]), pack_bf16(f[2][i], f[3][i]), pack_bf16(f[4][i], f[5][i]),
-                       pack_bf16(f[6][i], f[7][i]));
-    }
+    store16<S>(J.S, J.rows_total, grow, kpitch, k, e, x);
   }
 }
 
@@ -830,15 +858,9 @@ __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob 
   }
   const bool is_a = int(blockIdx.x) < ga;
   const SplitJob& J = is_a ? ja : jb;
-  const int cta = int(blockIdx.x) - (is_a ? 0 : ga);
-  int lo = 0, hi = J.ntasks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (J.tasks[mid].cta0 <= cta) lo = mid;
-    else hi = mid - 1;
-  }
-  const SplitTask tk = J.tasks[lo];
-  const int c = cta - tk.cta0;
+  const int2 tc = J.ctas[int(blockIdx.x) - (is_a ? 0 : ga)];
+  const SplitTask tk = J.tasks[tc.x];
+  const int c = tc.y;
   if (tk.s_k != 1 && tk.s_r == 1) {
     // (a task's CTAs are whole clusters: the branch is the same for all of one)
     const int r0 = (c / csize) * 32;
@@ -854,11 +876,11 @@ __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob 
   // any other strides: one warp per row, lanes along k
   const int lane = threadIdx.x & 31;
   const double* xr = J.X + tk.base + (long long)r * tk.s_r;
-  unsigned long long mx = 0;
-  for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_bits(__double_as_longlong(xr[(long long)k * tk.s_k])));
+  uint32_t mx = 0;
+  for (int k = lane; k < tk.K; k += 32) mx = max(mx, abs_hi(__double_as_longlong(xr[(long long)k * tk.s_k])));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int e = int(mx >> 52) - 1022;
+  const int e = row_exp(mx);
   const long long grow = tk.row0 + r;
   if (lane == 0) J.ex[grow] = e;
   for (int k = lane; k < ((tk.K + 31) & ~31); k += 32) {
@@ -870,24 +892,46 @@ __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob 
   }
 }
 
-// Gather and split in one pass (the operand's sector matrix is never
-// formed): one warp per row of a sector matrix reads the row's K elements
-// straight from the operand tensor's canonical blocks, takes the row's
-// exponent and writes its S digit slices.  A row of sector s and row
-// configuration r meets one block per column configuration c (a segment
-// [k0, k0 + w) of the row); inside block (r, c) the element of row mi and
-// column kk sits at  off + sum_rowlegs idx * str + sum_collegs idx * str,
-// the indices from mi and kk row-major over the legs in matrix order.
-// One warp per row, lanes along k: the reads are coalesced when the operand
-// block's innermost leg is a contracted leg (consecutive k are consecutive
-// in memory); plans whose operands are not laid out so gather and split in
-// two passes instead (ozaki_packable).
+// Gather and split in one pass: the rows of an operand's sector matrices are
+// read straight from the tensor's canonical blocks, and only their digits
+// are written (8 bytes in, 2 S out per element; a gather followed by a split
+// moves 16 + 8 + 2 S).  A row of sector s and row configuration r meets one
+// block per column configuration c (a segment [k0, k0 + w) of the row);
+// inside block (r, c) the element of row mi and column kk sits at  off +
+// sum_rowlegs idx * str + sum_collegs idx * str, the indices from mi and kk
+// row-major over the legs in matrix order.
+//
+// The loads coalesce when the lanes run along the tensor's innermost leg, so
+// a group (one sector and row configuration) is read in one of two ways:
+//   * innermost leg contracted: lanes along k, four k per lane (as
+//     split_rows, several short rows per warp);
+//   * innermost leg open: lanes along the rows of the group, 16 consecutive
+//     k per thread (as split_cols).  Up to 128 k, the 8 warps of a CTA take
+//     8, 4, 2 or 1 blocks of 32 rows; a block of more k is shared by up to 8
+//     CTAs of a cluster, which exchange the row maxima, so that values wait
+//     for them in registers.  Past 1024 k a thread's later passes are read
+//     again (from cache).
+// An element's address is that of its row in the segment's block plus an
+// offset of k alone: a CTA tabulates both in shared memory (up to 1024 k and
+// 4096 rows x segments at a time), so the index arithmetic over the legs is
+// paid once per row and segment and once per k, not per element.
+//
+// What bounds it: the latency of the loads, with 24 warps an SM (registers),
+// at a third of the memory's rate.  Against the gather and split it replaced:
+// the batch of 64 corners 3.30 -> 2.05 ms, the D=6 corner (22 MB) 0.045 ->
+// 0.029 ms, the D=8, chi=192 single-layer move's contractions 44 -> 28 ms;
+// with the innermost leg contracted, 2432 x 2432 twice, 200 -> 90 us.
 struct PackGroup {
-  int32_t pw0;    // first warp of this group
-  int32_t row0;   // its first row in the split buffer
-  int32_t h, K;   // rows of this (sector, row configuration), columns
-  int64_t seg0;   // its segments (one per column configuration), k0 ascending
-  int32_t nseg, pad;
+  int32_t row0;         // its first row in the split buffer
+  int32_t h, K;         // rows of this (sector, row configuration), columns
+  int64_t seg0;         // its segments (one per column configuration), k0 ascending
+  int32_t nseg, along;  // along: 0 lanes along k, 1 lanes along the rows
+  int32_t pad;
+};
+
+struct alignas(16) PackLeg {
+  int32_t dim, str;     // extent, stride inside the block
+  uint32_t fm, fl;      // FastDiv of dim
 };
 
 struct PackSeg {
@@ -895,15 +939,13 @@ struct PackSeg {
   int32_t k0, w;        // columns [k0, k0 + w) of the row
   int32_t nr, nc;       // row legs, column legs
   int32_t src, pad;     // index of the tensor in the job's pointer table
-  int32_t dim[kMaxRank];  // row legs then column legs, matrix order
-  int32_t str[kMaxRank];  // their strides inside the block
-  uint32_t fm[kMaxRank], fl[kMaxRank];  // FastDiv of dim
+  PackLeg leg[kMaxRank];  // row legs then column legs, matrix order
 };
 
 struct PackJob {
   const PackGroup* groups;
   const PackSeg* segs;
-  int ngroups, nwarps;         // groups, warps
+  const int2* ctas;            // per CTA: its group and its number inside it
   int rows_total;              // rows of the split buffer (slice stride)
   const double* src;           // the operand tensor (tab == nullptr)
   const double* const* tab;    // per-segment tensors (batched contractions)
@@ -913,101 +955,269 @@ struct PackJob {
 
 __device__ __forceinline__ uint32_t fdiv(uint32_t n, uint32_t m, uint32_t l) { return (__umulhi(n, m) + n) >> l; }
 
+// CTAs of a group
+__host__ __device__ inline int pack_col_warps(int K) { return K <= 16 ? 1 : K <= 32 ? 2 : K <= 64 ? 4 : 8; }
+// CTAs along k of one block of rows: enough for one pass of 128 k each, as
+// far as the cluster goes (powers of two)
+__host__ __device__ inline int pack_col_ctas(int K, int csize) {
+  int c = 1;
+  while (c < csize && c * 128 < K) c *= 2;
+  return c;
+}
+inline int pack_ctas(int h, int K, int along, int csize) {
+  if (!along) return ((h + split_cta_rows(K) - 1) / split_cta_rows(K) + csize - 1) / csize * csize;
+  const int blocks = (h + 31) / 32, per = 8 / pack_col_warps(K);
+  return ((blocks + per - 1) / per * pack_col_ctas(K, csize) + csize - 1) / csize * csize;
+}
+
+constexpr int kPackTab = 1024;   // k per table
+constexpr int kPackRows = 4096;  // rows x segments per table
+constexpr int kPackSegs = 128;   // segments searched on chip
+
+struct PackShared {
+  int2 k[kPackTab];                 // element offset inside the block, segment of the table
+  const double* row[kPackRows];     // [segment][row]: the row's first element in the segment's block
+  uint32_t wmax[kSplitThreads / 32][32];
+  uint32_t cmax[32];
+  int k0[kPackSegs];
+};
+
+// Tables of R rows from r0 for k in [kc, kb); returns the end of their k
+// range (kb, or a multiple of 32 past kc).
+__device__ __forceinline__ int pack_table(PackShared& sm, const PackJob& J, const PackGroup& G, int r0, int R, int kc,
+                                          int kb) {
+  const PackSeg* segs = J.segs + G.seg0;
+  // the segments' first k, so that the searches below stay on chip (groups
+  // of more than kPackSegs segments search the rest in memory)
+  for (int i = int(threadIdx.x); i < min(G.nseg, kPackSegs); i += kSplitThreads) sm.k0[i] = segs[i].k0;
+  __syncthreads();
+  auto seg_of = [&](int k) {
+    int lo = 0, hi = G.nseg - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if ((mid < kPackSegs ? sm.k0[mid] : segs[mid].k0) <= k) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  };
+  const int s0 = seg_of(kc), smax = s0 + kPackRows / R;
+  int ke = min(kb, kc + kPackTab);
+  if (smax < G.nseg) ke = min(ke, segs[smax].k0);
+  if (ke < kb) ke = kc + ((ke - kc) & ~31);
+  const int s1 = seg_of(ke - 1) + 1;
+  for (int k = kc + int(threadIdx.x); k < ke; k += kSplitThreads) {
+    const int si = seg_of(k);
+    const PackSeg& sg = segs[si];
+    uint32_t rem = uint32_t(k - sg.k0);
+    int o = 0;
+    for (int j = sg.nr + sg.nc - 1; j >= sg.nr; --j) {
+      const PackLeg l = sg.leg[j];
+      const uint32_t q = fdiv(rem, l.fm, l.fl);
+      o += int(rem - q * uint32_t(l.dim)) * l.str;
+      rem = q;
+    }
+    sm.k[k - kc] = make_int2(o, si - s0);
+  }
+  for (int t = int(threadIdx.x); t < (s1 - s0) * R; t += kSplitThreads) {
+    const int si = t / R;
+    const PackSeg& sg = segs[s0 + si];
+    uint32_t rem = uint32_t(min(r0 + t - si * R, G.h - 1));
+    long long o = sg.off;
+    for (int j = sg.nr - 1; j >= 0; --j) {
+      const PackLeg l = sg.leg[j];
+      const uint32_t q = fdiv(rem, l.fm, l.fl);
+      o += (long long)(rem - q * uint32_t(l.dim)) * l.str;
+      rem = q;
+    }
+    sm.row[t] = (J.tab ? J.tab[sg.src] : J.src) + o;
+  }
+  __syncthreads();
+  return ke;
+}
+
+// n consecutive elements of table row r from k on (zeros from ke on)
+template <int n>
+__device__ __forceinline__ void pack_load(const PackShared& sm, int r, int R, int k, int kc, int ke,
+                                          unsigned long long (&v)[n]) {
+#pragma unroll
+  for (int j = 0; j < n; ++j) {
+    v[j] = 0ull;
+    if (k + j < ke) {
+      const int2 t = sm.k[k + j - kc];
+      v[j] = (unsigned long long)__double_as_longlong(__ldg(sm.row[t.y * R + r] + t.x));
+    }
+  }
+}
 
 template <int S>
-__global__ void __launch_bounds__(256) pack_split_kernel(PackJob ja, PackJob jb, int ga, int gab, int kpitch,
-                                                         ZeroJob zj) {
+__device__ __forceinline__ void pack_rows(PackShared& sm, const PackJob& J, const PackGroup& G, int cta, int kpitch) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int R = split_cta_rows(G.K), r0 = cta * R;
+  const int kend = (G.K + 31) & ~31;
+  auto store4 = [&](int mi, int k, int e, const unsigned long long (&v)[4]) {
+    uint32_t f[4][S];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) split_digits<S>(v[j], e, f[j]);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+      *reinterpret_cast<uint2*>(J.S + ((long long)i * J.rows_total + G.row0 + mi) * kpitch + k) =
+          make_uint2(pack_bf16(f[0][i], f[1][i]), pack_bf16(f[2][i], f[3][i]));
+  };
+  int ke = pack_table(sm, J, G, r0, R, 0, G.K);
+  unsigned long long x[4][4];
+  if (G.K <= 128) {  // (at most 128 segments: one table)
+    const int lpr = G.K <= 32 ? 8 : G.K <= 64 ? 16 : 32;  // lanes per row
+    const int rpw = 32 / lpr, k = (lane % lpr) * 4;
+    const int lr = warp * 4 * rpw + lane / lpr;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) pack_load(sm, lr + it * rpw, R, k, 0, ke, x[it]);
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      uint32_t mx = max(max(abs_hi(x[it][0]), abs_hi(x[it][1])), max(abs_hi(x[it][2]), abs_hi(x[it][3])));
+      for (int o = lpr >> 1; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const int e = row_exp(mx);
+      const int r = r0 + lr + it * rpw;
+      if (r >= G.h) continue;
+      if (k == 0) J.ex[G.row0 + r] = e;
+      if (k < kend) store4(r, k, e, x[it]);
+    }
+    return;
+  }
+  const int r = r0 + warp;
+  uint32_t mx = 0;
+  const bool one = ke == G.K, keep = one && G.K <= kSplitRowMax;
+  if (keep) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) pack_load(sm, warp, R, g * 128 + lane * 4, 0, ke, x[g]);
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mx = max(mx, abs_hi(x[g][j]));
+  } else {
+    for (int kc = 0;;) {
+      for (int k = kc + lane * 4; k < ke; k += 512) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) pack_load(sm, warp, R, k + g * 128, kc, ke, x[g]);
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mx = max(mx, abs_hi(x[g][j]));
+      }
+      if (ke == G.K) break;
+      __syncthreads();
+      kc = ke;
+      ke = pack_table(sm, J, G, r0, R, kc, G.K);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const int e = row_exp(mx);
+  if (lane == 0 && r < G.h) J.ex[G.row0 + r] = e;
+  if (keep) {
+    if (r >= G.h) return;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int k = g * 128 + lane * 4;
+      if (k < kend) store4(r, k, e, x[g]);
+    }
+    return;
+  }
+  for (int kc = 0; kc < G.K; kc = ke) {
+    if (!one) {
+      __syncthreads();
+      ke = pack_table(sm, J, G, r0, R, kc, G.K);
+    }
+    if (r >= G.h) continue;
+    for (int k = kc + lane * 4; k < ((ke + 31) & ~31); k += 512) {
+#pragma unroll
+      for (int g = 0; g < 4; ++g) pack_load(sm, warp, R, k + g * 128, kc, ke, x[g]);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        if (k + g * 128 < ((ke + 31) & ~31)) store4(r, k + g * 128, e, x[g]);
+    }
+  }
+}
+
+template <int S>
+__device__ __forceinline__ void pack_cols(PackShared& sm, const PackJob& J, const PackGroup& G, int cta, int csize,
+                                          int kpitch) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wk = pack_col_warps(G.K);       // warps along k of one block of 32 rows
+  const int cpb = pack_col_ctas(G.K, csize);  // CTAs along k of one block
+  const int first = warp - warp % wk;
+  const int R = 8 / wk * 32, r0 = cta / cpb * R;
+  const int lr = warp / wk * 32 + lane, mi = r0 + lr;
+  const bool live = mi < G.h;
+  // this CTA's k: one pass of 128 (or of all, below) where cpb covers K
+  const int kr = (G.K + 128 * cpb - 1) / (128 * cpb) * 128;
+  const int ka = cta % cpb * kr, kb = min(G.K, ka + kr);
+  const int k0 = (warp % wk) * 16, step = wk * 16;
+  unsigned long long x[16];
+  uint32_t mx = 0;
+  int ke = kb;
+  bool one = true;  // one table holds the CTA's k
+  if (ka < kb) {
+    ke = pack_table(sm, J, G, r0, R, ka, kb);
+    one = ke == kb;
+    pack_load(sm, lr, R, ka + k0, ka, ke, x);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) mx = max(mx, abs_hi(x[j]));
+    for (int kc = ka;;) {
+      for (int k = kc + k0 + (kc == ka ? step : 0); k < ke; k += step) {
+        unsigned long long v[16];
+        pack_load(sm, lr, R, k, kc, ke, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) mx = max(mx, abs_hi(v[j]));
+      }
+      if (ke == kb) break;
+      __syncthreads();
+      kc = ke;
+      ke = pack_table(sm, J, G, r0, R, kc, kb);
+    }
+  }
+  sm.wmax[warp][lane] = mx;
+  __syncthreads();
+  for (int c = 0; c < wk; ++c) mx = max(mx, sm.wmax[first + c][lane]);
+  if (cpb > 1) {
+    // (wk is 8: the CTA holds one block; all of a cluster take this branch)
+    cg::cluster_group cl = cg::this_cluster();
+    if (warp == 0) sm.cmax[lane] = mx;
+    cl.sync();
+    const int base = int(cl.block_rank()) - cta % cpb;
+    for (int c = 0; c < cpb; ++c) mx = max(mx, cl.map_shared_rank(sm.cmax, base + c)[lane]);
+    cl.sync();  // no CTA leaves while another still reads its maxima
+  }
+  const int e = row_exp(mx);
+  const long long grow = G.row0 + mi;
+  if (live && warp == first && ka == 0) J.ex[grow] = e;
+  for (int kc = ka; kc < kb; kc = ke) {
+    if (!one) {
+      __syncthreads();
+      ke = pack_table(sm, J, G, r0, R, kc, kb);
+    }
+    if (!live) continue;
+    for (int k = kc + k0; k < ((ke + 31) & ~31); k += step) {
+      if (k != ka + k0) pack_load(sm, lr, R, k, kc, ke, x);
+      store16<S>(J.S, J.rows_total, grow, kpitch, k, e, x);
+    }
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(kSplitThreads, 3) pack_split_kernel(PackJob ja, PackJob jb, int ga, int gab,
+                                                                      int csize, int kpitch, ZeroJob zj) {
   if (int(blockIdx.x) >= gab) {
-    zero_part(zj, int(blockIdx.x) - gab);
+    const int z = int(blockIdx.x) - gab;
+    if (z < zj.nz * kZeroCtas) zero_part(zj, z);
     return;
   }
   const bool is_a = int(blockIdx.x) < ga;
   const PackJob& J = is_a ? ja : jb;
-  const int w = ((int(blockIdx.x) - (is_a ? 0 : ga)) * int(blockDim.x) + int(threadIdx.x)) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= J.nwarps || J.ngroups == 0) return;
-  int lo = 0, hi = J.ngroups - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (J.groups[mid].pw0 <= w) lo = mid;
-    else hi = mid - 1;
-  }
-  const PackGroup G = J.groups[lo];
-  const PackSeg* segs = J.segs + G.seg0;
-  const int mi = w - G.pw0;
-  if (mi < 0 || mi >= G.h) return;
-  const int grow = G.row0 + mi;
-  // row-leg indices of mi (the row legs' extents are those of every
-  // segment of the group)
-  int ridx[kMaxRank];
-  {
-    const PackSeg& s0 = segs[0];
-    uint32_t rem = uint32_t(mi);
-#pragma unroll
-    for (int j = kMaxRank - 1; j >= 0; --j) {
-      ridx[j] = 0;
-      if (j < s0.nr) {
-        const uint32_t q = fdiv(rem, s0.fm[j], s0.fl[j]);
-        ridx[j] = int(rem - q * uint32_t(s0.dim[j]));
-        rem = q;
-      }
-    }
-  }
-  // element k of the row (k < K), walking the segments forward
-  int si = 0;
-  long long rp = 0;
-  const double* base = nullptr;
-  auto enter = [&](int i) {
-    const PackSeg& sg = segs[i];
-    long long o = sg.off;
-#pragma unroll
-    for (int j = 0; j < kMaxRank; ++j)
-      if (j < sg.nr) o += (long long)ridx[j] * sg.str[j];
-    rp = o;
-    base = J.tab ? J.tab[sg.src] : J.src;
-  };
-  auto load = [&](int k) -> double {
-    while (k >= segs[si].k0 + segs[si].w) {
-      ++si;
-      enter(si);
-    }
-    const PackSeg& sg = segs[si];
-    uint32_t rem = uint32_t(k - sg.k0);
-    long long o = rp;
-#pragma unroll
-    for (int j = kMaxRank - 1; j >= 0; --j) {
-      if (j < sg.nc) {
-        const int jj = sg.nr + j;
-        const uint32_t q = fdiv(rem, sg.fm[jj], sg.fl[jj]);
-        o += (long long)(rem - q * uint32_t(sg.dim[jj])) * sg.str[jj];
-        rem = q;
-      }
-    }
-    return base[o];
-  };
-  const int kend = (G.K + 31) & ~31;
-  enter(0);
-  unsigned long long mx = 0;
-  for (int k = lane; k < G.K; k += 32) {
-    const unsigned long long b = __double_as_longlong(load(k)) & 0x7FFFFFFFFFFFFFFFull;
-    mx = b > mx ? b : mx;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = y > mx ? y : mx;
-  }
-  const int e = int(mx >> 52) - 1022;
-  if (lane == 0) J.ex[grow] = e;
-  si = 0;
-  enter(0);
-  for (int k = lane; k < kend; k += 32) {
-    uint32_t f[S];
-    split_digits<S>(k < G.K ? (unsigned long long)__double_as_longlong(load(k)) : 0ull, e, f);
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-      J.S[((long long)i * J.rows_total + grow) * kpitch + k] = __ushort_as_bfloat16((unsigned short)(f[i] >> 16));
-  }
+  const int2 c = J.ctas[int(blockIdx.x) - (is_a ? 0 : ga)];
+  const PackGroup G = J.groups[c.x];
+  __shared__ PackShared sm;
+  if (G.along) pack_cols<S>(sm, J, G, c.y, csize, kpitch);
+  else if (c.y * split_cta_rows(G.K) < G.h) pack_rows<S>(sm, J, G, c.y, kpitch);
 }
 
 }  // namespace oz
@@ -1055,7 +1265,7 @@ struct OzakiPlan {
   oz::Prob* d_probs = nullptr;
   oz::Tile* d_tiles = nullptr;
   oz::SplitTask *d_sa = nullptr, *d_sb = nullptr;
-  int nsa = 0, nsb = 0;
+  int2 *d_ca = nullptr, *d_cb = nullptr;  // the split's CTA tables
   int split_ca = 0, split_cb = 0;  // CTAs of the split of A and of B
   int split_cluster = 1;           // CTAs that share 32 interleaved rows of an operand
   __nv_bfloat16 *SA = nullptr, *SB = nullptr;
@@ -1087,12 +1297,19 @@ struct OzakiPlan {
   bool packed = false;
   oz::PackGroup *d_pgA = nullptr, *d_pgB = nullptr;
   oz::PackSeg *d_psA = nullptr, *d_psB = nullptr;
-  int ngA = 0, ngB = 0, nrA = 0, nrB = 0;  // groups and warps of each operand
+  int2 *d_pcA = nullptr, *d_pcB = nullptr;
+  int ncA = 0, ncB = 0;                    // CTAs of each operand
+  bool pack_apart = false;                 // one launch per operand
+  int pack_cluster = 1;                    // CTAs that share the k of a block of rows
   ~OzakiPlan() {
     cudaFree(d_pgA);
     cudaFree(d_pgB);
     cudaFree(d_psA);
     cudaFree(d_psB);
+    cudaFree(d_pcA);
+    cudaFree(d_pcB);
+    cudaFree(d_ca);
+    cudaFree(d_cb);
     cudaFree(d_rowtab);
     cudaFree(d_coltab);
     cudaFree(d_bbase);
@@ -1132,7 +1349,16 @@ static int num_sms() {
 struct PackTables {
   std::vector<oz::PackGroup> g;
   std::vector<oz::PackSeg> sg;
-  int nwarps = 0;
+  std::vector<int2> ctas;
+  int kcol = 0;    // longest k read with the lanes along the rows
+  int blocks = 0;  // CTAs without sharing of k
+  void place(int csize) {
+    ctas.clear();
+    for (size_t i = 0; i < g.size(); ++i) {
+      const int n = oz::pack_ctas(g[i].h, g[i].K, g[i].along, csize);
+      for (int c = 0; c < n; ++c) ctas.push_back(make_int2(int(i), c));
+    }
+  }
 };
 
 // Appends the pack groups and segments of one operand of one contraction:
@@ -1161,7 +1387,7 @@ static void append_pack(PackTables& T, const Layout* L, const MatView& v, const 
       for (size_t rc = 0; rc < sec.rcfg.size(); ++rc) {
         const int64_t h = (rc + 1 < sec.rcfg.size() ? sec.roff[rc + 1] : sec.rows) - sec.roff[rc];
         oz::PackGroup pg{};
-        pg.pw0 = T.nwarps;
+        pg.along = nc > 0 && v.collegs.back() == r - 1 ? 0 : 1;
         pg.row0 = int32_t(row + sec.roff[rc]);
         pg.h = int32_t(h);
         pg.K = g.K;
@@ -1185,12 +1411,9 @@ static void append_pack(PackTables& T, const Layout* L, const MatView& v, const 
           int64_t hh = 1, w = 1;
           for (int j = 0; j < nr + nc; ++j) {
             const int leg = j < nr ? v.rowlegs[j] : v.collegs[j - nr];
-            sg.dim[j] = int32_t(sh[leg]);
-            sg.str[j] = int32_t(bst[leg]);
             FastDiv f;
             f.init(uint32_t(sh[leg]));
-            sg.fm[j] = f.m;
-            sg.fl[j] = f.l;
+            sg.leg[j] = {int32_t(sh[leg]), int32_t(bst[leg]), f.m, f.l};
             (j < nr ? hh : w) *= sh[leg];
           }
           sg.w = int32_t(w);
@@ -1199,8 +1422,9 @@ static void append_pack(PackTables& T, const Layout* L, const MatView& v, const 
           T.sg.push_back(sg);
         }
         BST_REQUIRE(kcov == g.K, BST_E_SHAPE, "pack: segments do not cover K");
+        if (pg.along) T.kcol = std::max(T.kcol, pg.K);
+        T.blocks += oz::pack_ctas(pg.h, pg.K, pg.along, 1);
         T.g.push_back(pg);
-        T.nwarps += int32_t(h);
       }
     }
     row += rows;
@@ -1282,8 +1506,6 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
                      [&](const oz::Tile& x, const oz::Tile& y) { return hp[x.prob].K > hp[y.prob].K; });
   P->nprobs = int(hp.size());
   P->ntiles = int(ht.size());
-  P->nsa = int(sa.size());
-  P->nsb = int(sb.size());
   // CTAs of the split: eight contiguous rows each, or a cluster per 32
   // interleaved rows (128 k per CTA and pass: one pass up to K = 1024)
   int kcol = 0;
@@ -1292,18 +1514,20 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
       if (t.s_k != 1 && t.s_r == 1) kcol = std::max(kcol, t.K);
   while (P->split_cluster < 8 && P->split_cluster * 128 < kcol) P->split_cluster *= 2;
   const int sc_ = P->split_cluster;
-  auto place = [&](std::vector<oz::SplitTask>& v) {
-    int cta = 0;
-    for (auto& t : v) {
-      t.cta0 = cta;
+  auto place = [&](const std::vector<oz::SplitTask>& v) {
+    std::vector<int2> ctas;
+    for (size_t i = 0; i < v.size(); ++i) {
+      const oz::SplitTask& t = v[i];
       const int per = t.s_k == 1 ? oz::split_cta_rows(t.K) : 8;
-      const int n = t.s_k != 1 && t.s_r == 1 ? (t.rows + 31) / 32 * sc_ : (t.rows + per - 1) / per;
-      cta += (n + sc_ - 1) / sc_ * sc_;
+      int n = t.s_k != 1 && t.s_r == 1 ? (t.rows + 31) / 32 * sc_ : (t.rows + per - 1) / per;
+      n = (n + sc_ - 1) / sc_ * sc_;
+      for (int c = 0; c < n; ++c) ctas.push_back(make_int2(int(i), c));
     }
-    return cta;
+    return ctas;
   };
-  P->split_ca = place(sa);
-  P->split_cb = place(sb);
+  const std::vector<int2> ca = place(sa), cb = place(sb);
+  P->split_ca = int(ca.size());
+  P->split_cb = int(cb.size());
   BST_REQUIRE(int64_t(P->rowsA) * S < (1ll << 31) && int64_t(P->rowsB) * S < (1ll << 31),
               BST_E_UNSUPPORTED, "Ozaki GEMM: too many rows");
   auto up = [](auto** dst, const auto& v) {
@@ -1318,6 +1542,8 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   P->nzprobs = int(zp.size());
   up(&P->d_sa, sa);
   up(&P->d_sb, sb);
+  up(&P->d_ca, ca);
+  up(&P->d_cb, cb);
   if (sc) {
     P->scatter = true;
     up(&P->d_rowtab, sc->rowtab);
@@ -1344,6 +1570,22 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   return P;
 }
 
+// Launch of `grid` CTAs in clusters of csize (grid a multiple of it).
+template <class... P, class... A>
+static void launch_clusters(void (*kern)(P...), int grid, int threads, int csize, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(grid));
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = unsigned(csize);
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = csize > 1 ? 1 : 0;
+  BST_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+}
+
 // A, B: the operands' sector matrices, or for a packed plan the operand
 // tensors themselves (tabA / tabB: per-segment tensor tables of a batch)
 static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, double* C, cudaStream_t s,
@@ -1353,20 +1595,28 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
   const oz::Scatter sc{P->d_rowtab, P->d_coltab, bbase ? bbase : P->d_bbase, alpha, beta};
   const bool b_from_a = P->ab_same && A == B && split_a;
   if (P->packed) {
-    // gather + split: FP64 read once per element (and once more from cache),
-    // S digits written; the byte count is that of the split of gathered
-    // rows without the FP64 row write and read of a separate gather.  The
-    // K == 0 problems' outputs are written by the same launch.
+    // gather + split: FP64 read once per element (rows of more than 128 or
+    // 512 once more from cache), S digits written; the byte count is that of
+    // the split of gathered rows without the FP64 row write and read of a
+    // separate gather.  The K == 0 problems' outputs are written by the same
+    // launch.
     ProfScope ps(ctx, s, "pack_bf16", 0.0, P->split_bytes);
-    const oz::PackJob ja{P->d_pgA, P->d_psA, P->ngA, P->nrA, P->rowsA, A, tabA, P->SA, P->eA};
-    const oz::PackJob jb{P->d_pgB, P->d_psB, P->ngB, P->nrB, P->rowsB, B, tabB, P->SB, P->eB};
+    const oz::PackJob ja{P->d_pgA, P->d_psA, P->d_pcA, P->rowsA, A, tabA, P->SA, P->eA};
+    const oz::PackJob jb{P->d_pgB, P->d_psB, P->d_pcB, P->rowsB, B, tabB, P->SB, P->eB};
     const oz::ZeroJob zj{P->nzprobs, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
-    const int ga = (P->nrA + 7) / 8, gb = (P->nrB + 7) / 8, gz = P->nzprobs * oz::kZeroCtas;
-    if (ga + gb + gz > 0) {
-      if (P->S == 5) oz::pack_split_kernel<5><<<ga + gb + gz, 256, 0, s>>>(ja, jb, ga, ga + gb, P->kpitch, zj);
-      else oz::pack_split_kernel<3><<<ga + gb + gz, 256, 0, s>>>(ja, jb, ga, ga + gb, P->kpitch, zj);
-      BST_CUDA(cudaGetLastError());
+    const int cs = P->pack_cluster;
+    const int gz = (P->nzprobs * oz::kZeroCtas + cs - 1) / cs * cs;
+    auto pack = [&](int ga, int gb, int z) {
+      if (ga + gb + z == 0) return;
+      launch_clusters(P->S == 5 ? oz::pack_split_kernel<5> : oz::pack_split_kernel<3>, ga + gb + z, oz::kSplitThreads,
+                      cs, s, ja, jb, ga, ga + gb, cs, P->kpitch, zj);
       count_launch(ctx);
+    };
+    if (P->pack_apart) {
+      pack(P->ncA, 0, 0);
+      pack(0, P->ncB, gz);
+    } else {
+      pack(P->ncA, P->ncB, gz);
     }
     if (P->ntiles == 0) return;
   } else {
@@ -1378,22 +1628,10 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
     const int gz = (P->nzprobs * oz::kZeroCtas + cs - 1) / cs * cs;
     const oz::ZeroJob zj{P->nzprobs, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
     if (ga + gb + gz > 0) {
-      const oz::SplitJob ja{P->d_sa, P->nsa, P->rowsA, A, P->SA, P->eA};
-      const oz::SplitJob jb{P->d_sb, P->nsb, P->rowsB, B, P->SB, P->eB};
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(unsigned(ga + gb + gz));
-      cfg.blockDim = dim3(oz::kSplitThreads);
-      cfg.stream = s;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = unsigned(cs);
-      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = cs > 1 ? 1 : 0;
-      if (P->S == 5)
-        BST_CUDA(cudaLaunchKernelEx(&cfg, oz::ozaki_split_kernel<5>, ja, jb, ga, ga + gb, cs, P->kpitch, zj));
-      else
-        BST_CUDA(cudaLaunchKernelEx(&cfg, oz::ozaki_split_kernel<3>, ja, jb, ga, ga + gb, cs, P->kpitch, zj));
+      const oz::SplitJob ja{P->d_sa, P->d_ca, P->rowsA, A, P->SA, P->eA};
+      const oz::SplitJob jb{P->d_sb, P->d_cb, P->rowsB, B, P->SB, P->eB};
+      launch_clusters(P->S == 5 ? oz::ozaki_split_kernel<5> : oz::ozaki_split_kernel<3>, ga + gb + gz,
+                      oz::kSplitThreads, cs, s, ja, jb, ga, ga + gb, cs, P->kpitch, zj);
       count_launch(ctx);
     }
     if (P->ntiles == 0) return;
@@ -1493,7 +1731,15 @@ static OzakiPlan* prepare_scatter(Ctx* ctx, ContractPlan* p, int S) {
 }
 
 // Device tables of the packed operands of a contraction plan.
-static void attach_pack(OzakiPlan* P, const PackTables& ta, const PackTables& tb) {
+static void attach_pack(OzakiPlan* P, PackTables& ta, PackTables& tb) {
+  // CTAs along k only while the blocks of rows alone leave SMs idle: a CTA
+  // pays for its tables whatever its share (the batch of 64 corners takes
+  // 3.3 ms with clusters of 8 and 2.05 without, the D=6 corner 28 us with
+  // clusters and 31 without)
+  P->pack_cluster = oz::pack_col_ctas(std::max(ta.kcol, tb.kcol), 8);
+  while (P->pack_cluster > 1 && (ta.blocks + tb.blocks) * P->pack_cluster > 4 * num_sms()) P->pack_cluster /= 2;
+  ta.place(P->pack_cluster);
+  tb.place(P->pack_cluster);
   auto up = [](auto** dst, const auto& v) {
     using T = typename std::remove_reference<decltype(v)>::type::value_type;
     if (v.empty()) return;
@@ -1504,10 +1750,10 @@ static void attach_pack(OzakiPlan* P, const PackTables& ta, const PackTables& tb
   up(&P->d_psA, ta.sg);
   up(&P->d_pgB, tb.g);
   up(&P->d_psB, tb.sg);
-  P->ngA = int(ta.g.size());
-  P->ngB = int(tb.g.size());
-  P->nrA = ta.nwarps;
-  P->nrB = tb.nwarps;
+  up(&P->d_pcA, ta.ctas);
+  up(&P->d_pcB, tb.ctas);
+  P->ncA = int(ta.ctas.size());
+  P->ncB = int(tb.ctas.size());
   P->packed = true;
   P->ab_same = false;
 }
@@ -1521,24 +1767,11 @@ static void attach_pack(OzakiPlan* P, ContractPlan* p) {
   attach_pack(P, ta, tb);
 }
 
-// The pack kernel reads a row's K elements with its lanes: coalesced when
-// the last contracted leg (in pair order) is the operand tensor's innermost
-// leg.  Plans whose operands are laid out otherwise gather (block-contiguous
-// reads) and split in two passes.
-bool ozaki_packable(const ContractPlan* p) {
+// Both operands' innermost legs are contracted (in the last pair): the pack
+// reads both with its lanes along k.
+bool ozaki_k_inner(const ContractPlan* p) {
   return !p->va.collegs.empty() && p->va.collegs.back() == p->A->rank - 1 && !p->vb.collegs.empty() &&
          p->vb.collegs.back() == p->B->rank - 1;
-}
-
-// Operands of a plan that is not packed: the gathered sector matrices.
-static void gather_operands(Ctx* ctx, ContractPlan* p, const double* a, const double* b, const double** Am,
-                            const double** Bm, cudaStream_t s) {
-  double* am = (double*)ctx->buf("contract.A", sizeof(double) * std::max<int64_t>(p->amat, 1), s);
-  double* bm = (double*)ctx->buf("contract.B", sizeof(double) * std::max<int64_t>(p->bmat, 1), s);
-  launch_relayout(ctx, p->ra, a, am, 0, 1.0, 0.0, s);
-  launch_relayout(ctx, p->rb, b, bm, 0, 1.0, 0.0, s);
-  *Am = am;
-  *Bm = bm;
 }
 
 void run_gemm_ozaki_scatter(Ctx* ctx, ContractPlan* p, int S, const double* a, const double* b, double* c,
@@ -1546,24 +1779,16 @@ void run_gemm_ozaki_scatter(Ctx* ctx, ContractPlan* p, int S, const double* a, c
   OzakiPlan*& P = p->oz[S == 3 ? 1 : 0][1];
   if (!P) {
     P = prepare_scatter(ctx, p, S);
-    if (ozaki_packable(p)) attach_pack(P, p);
+    attach_pack(P, p);
   }
-  if (!P->packed) gather_operands(ctx, p, a, b, &a, &b, s);
   run_plan(ctx, P, a, b, c, s, true, alpha, beta);
 }
 
-void run_gemm_ozaki(Ctx* ctx, ContractPlan* p, int S, const double* a, const double* b, double* Cmat,
-                    cudaStream_t s, const double* Am, const double* Bm) {
+void run_gemm_ozaki(Ctx* ctx, ContractPlan* p, int S, const double* Am, const double* Bm, double* Cmat,
+                    cudaStream_t s) {
   OzakiPlan*& P = p->oz[S == 3 ? 1 : 0][0];
-  if (!P) {
-    P = build_plan(ctx, p->probs, 0, nullptr, S, ozaki_pick_tn(p->probs));
-    if (ozaki_packable(p)) attach_pack(P, p);
-  }
-  if (!P->packed) {
-    if (Am && Bm) a = Am, b = Bm;
-    else gather_operands(ctx, p, a, b, &a, &b, s);
-  }
-  run_plan(ctx, P, a, b, Cmat, s);
+  if (!P) P = build_plan(ctx, p->probs, 0, nullptr, S, ozaki_pick_tn(p->probs));
+  run_plan(ctx, P, Am, Bm, Cmat, s);
 }
 
 void ozaki_free(OzakiPlan* oz) { delete oz; }
@@ -1575,26 +1800,25 @@ void ozaki_free(OzakiPlan* oz) { delete oz; }
 // output and bbase_src its contraction, and ozaki_batch_bbase turns them
 // into element offsets from c[0] for one set of output pointers.
 OzakiPlan* ozaki_batch_plan(Ctx* ctx, const std::vector<ContractPlan*>& plans, const std::vector<GemmProb>& probs,
-                            int order, int S, int TN, bool pack, std::vector<long long>* bbase_rel,
+                            int order, int S, int TN, std::vector<long long>* bbase_rel,
                             std::vector<int32_t>* bbase_src) {
   ScatterSpec sc;
   bbase_src->clear();
   PackTables ta, tb;
   int ra = 0, rb = 0;
+  bool apart = false;
   for (size_t i = 0; i < plans.size(); ++i) {
     append_scatter(sc, plans[i], bbase_src, int(i));
-    if (pack) {
-      append_pack(ta, plans[i]->A, plans[i]->va, plans[i]->probs, false, ra, int(i));
-      append_pack(tb, plans[i]->B, plans[i]->vb, plans[i]->probs, true, rb, int(i));
-    }
+    append_pack(ta, plans[i]->A, plans[i]->va, plans[i]->probs, false, ra, int(i));
+    append_pack(tb, plans[i]->B, plans[i]->vb, plans[i]->probs, true, rb, int(i));
+    apart = apart || !ozaki_k_inner(plans[i]);
   }
   BST_REQUIRE(sc.rt_off.size() == probs.size(), BST_E_SHAPE, "batch plan: problem count mismatch");
   *bbase_rel = sc.bbase;
   OzakiPlan* P = build_plan(ctx, probs, order, &sc, S, TN == 0 ? ozaki_pick_tn(probs) : TN);
-  if (pack) {
-    BST_REQUIRE(ra == P->rowsA && rb == P->rowsB, BST_E_SHAPE, "batch plan: row count mismatch");
-    attach_pack(P, ta, tb);
-  }
+  BST_REQUIRE(ra == P->rowsA && rb == P->rowsB, BST_E_SHAPE, "batch plan: row count mismatch");
+  attach_pack(P, ta, tb);
+  P->pack_apart = apart;
   return P;
 }
 
@@ -1611,10 +1835,9 @@ void ozaki_batch_bbase(const std::vector<long long>& rel, const std::vector<int3
   for (size_t j = 0; j < rel.size(); ++j) (*out)[j] = rel[j] + delta[src[j]];
 }
 
-void run_ozaki_batch(Ctx* ctx, OzakiPlan* P, double* const* bases, int n, const double* Am, const double* Bm,
-                     double* c0, const long long* bbase, double alpha, double beta, cudaStream_t s) {
-  if (P->packed) run_plan(ctx, P, nullptr, nullptr, c0, s, true, alpha, beta, bases, bases + n, bbase);
-  else run_plan(ctx, P, Am, Bm, c0, s, true, alpha, beta, nullptr, nullptr, bbase);
+void run_ozaki_batch(Ctx* ctx, OzakiPlan* P, double* const* bases, int n, double* c0, const long long* bbase,
+                     double alpha, double beta, cudaStream_t s) {
+  run_plan(ctx, P, nullptr, nullptr, c0, s, true, alpha, beta, bases, bases + n, bbase);
 }
 
 void run_gemm_ozaki_probs(Ctx* ctx, const std::string& tag, const std::vector<GemmProb>& probs, const double* A,

@@ -1025,8 +1025,7 @@ ProjResult svd_projector(Ctx* ctx, Layout* Rt, const double* rt, Layout* Rb, con
   std::iota(cut.begin(), cut.end(), 0);
   ContractPlan* pn = get_contract_plan(ctx, Rt, Rb, cut, cut);
   // Rt and Rb as sector matrices (kept for P and Pt below), and
-  // N = Rt^T Rb (rows: right cut of Rt, cols: right cut of Rb); the
-  // tensor-core product reads Rt's and Rb's blocks itself
+  // N = Rt^T Rb (rows: right cut of Rt, cols: right cut of Rb)
   double* At = (double*)ctx->buf("proj.A", sizeof(double) * std::max<int64_t>(pn->amat, 1), s);  // [beta x alpha]
   double* Bt = (double*)ctx->buf("proj.B", sizeof(double) * std::max<int64_t>(pn->bmat, 1), s);  // [beta' x alpha']
   launch_relayout(ctx, pn->ra, rt, At, 0, 1.0, 0.0, s);
@@ -1034,7 +1033,7 @@ ProjResult svd_projector(Ctx* ctx, Layout* Rt, const double* rt, Layout* Rb, con
   double* Nm = (double*)ctx->buf("contract.Ckeep", sizeof(double) * std::max<int64_t>(pn->cmat, 1), s);
   ctx->work_flops += pn->g.flops;
   if (prec == BST_FP64) launch_gemm_f64(ctx, pn->g, At, Bt, Nm, s);
-  else run_gemm_ozaki(ctx, pn, ozaki_slices(prec), rt, rb, Nm, s, At, Bt);
+  else run_gemm_ozaki(ctx, pn, ozaki_slices(prec), At, Bt, Nm, s);
 
   std::vector<PSec> secs;
   for (auto& cs : pn->vc.secs) {

@@ -1,0 +1,91 @@
+"""The digit arithmetic (digit split or pack, tcgen05 product, output stage)
+at the edges of its tiles and vectors, against the dense product: rows and
+columns around 8, 32, 64 and 128, K around the 32-wide chunks, the 64-wide
+pairs and the register-resident lengths (128, 512), operands with the
+contracted leg innermost or outermost, and interleaved operands through the
+eigensolver's products."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bst():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1808_10804_gb300 import build
+    build.build()
+    from paper_1808_10804_gb300 import bst as b
+    return b
+
+
+@pytest.fixture(scope="module")
+def ctx(bst):
+    c = bst.Context(0)
+    yield c
+    c.close()
+
+
+# Elementwise error of the split products for a K-long sum.  Five digits: each
+# operand is rounded to 44 bits of its row (column) scale 2^e <= 2 max, so an
+# element is off by at most 2^-45 2^e <= 2^-44 max, twice per product; the
+# dropped digit products (i + j >= 5) are at most 4 2^-45 of 2^(ea + eb) <= 4
+# max max, plus as much for the following ones; the diagonals 3 and 4, at most
+# 2^-25 of 2^(ea + eb) per k, round to 24 bits at every step of 16 k.  Their
+# sum stays below 2^-39 per k.  Three digits: 2^-23 per k (26-bit operands and
+# the dropped products).
+BOUND = {"ozaki": 2.0 ** -39, "bf16x3": 2.0 ** -23}
+
+
+def check(got, A, B, prec):
+    ref = A @ B
+    bound = BOUND[prec] * A.shape[1] * np.outer(np.abs(A).max(1), np.abs(B).max(0))
+    assert got.shape == ref.shape
+    assert np.all(np.abs(got - ref) <= bound), (np.abs(got - ref) / bound).max()
+
+
+@pytest.mark.parametrize("prec", ["ozaki", "bf16x3"])
+@pytest.mark.parametrize("inner", ["open", "contracted", "mixed"])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (7, 9, 3), (8, 8, 31), (31, 33, 32), (33, 31, 33), (63, 65, 64),
+                                   (65, 63, 65), (127, 129, 127), (129, 127, 128), (130, 70, 129), (40, 200, 511),
+                                   (200, 40, 513), (257, 96, 700)])
+def test_product_edges(bst, ctx, M, N, K, inner, prec):
+    """Two sectors of sizes (M, K, N) and (N, K + 1, M), entries of very
+    different row scales."""
+    rng = np.random.default_rng([M, N, K])
+    m, k, n = (M, N), (K, K + 1), (N, M)
+    dense = [(rng.standard_normal((m[s], k[s])) * np.exp2(rng.integers(-20, 20, (m[s], 1))),
+              rng.standard_normal((k[s], n[s])) * np.exp2(rng.integers(-20, 20, (1, n[s])))) for s in (0, 1)]
+    at = inner == "open"          # A stored [k, m] (contracted leg outermost), else [m, k]
+    bt = inner == "contracted"    # B stored [n, k], else [k, n]
+    leg = lambda f, d: bst.Leg(f, (0, 2), d)  # noqa: E731
+    A = ctx.layout([leg(-1, k), leg(1, m)] if at else [leg(1, m), leg(-1, k)])
+    B = ctx.layout([leg(-1, n), leg(1, k)] if bt else [leg(1, k), leg(-1, n)])
+    flat = lambda xs, t: torch.tensor(np.concatenate([(x.T if t else x).reshape(-1) for x in xs]),  # noqa: E731
+                                      device="cuda:0")
+    _, c = ctx.contract(A, flat([d[0] for d in dense], at), B, flat([d[1] for d in dense], bt),
+                        (0 if at else 1,), (1 if bt else 0,), prec=prec)
+    ctx.sync()
+    out, pos = c.cpu().numpy(), 0
+    for s in (0, 1):
+        check(out[pos:pos + m[s] * n[s]].reshape(m[s], n[s]), *dense[s], prec)
+        pos += m[s] * n[s]
+    assert pos == out.size
+
+
+@pytest.mark.parametrize("n", [2, 31, 33, 64, 97, 128, 129, 160])
+def test_interleaved_operands(bst, ctx, n):
+    """The eigensolver's products X^T X and H X read columns of row-major
+    blocks; a well separated spectrum comes out to the arithmetic's
+    accuracy (the documented ~1e-12 of the largest value)."""
+    rng = np.random.default_rng(n)
+    q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    lam = np.linspace(1.0, 0.1, n)
+    H = (q * lam) @ q.T
+    X, got = ctx.sym_eig(torch.tensor(0.5 * (H + H.T), device="cuda:0")[None], prec="ozaki")
+    ctx.sync()
+    assert np.abs(got[0].cpu().numpy() - lam).max() <= 1e-11
+    X = X[0].cpu().numpy()
+    assert np.abs(X.T @ X - np.eye(n)).max() <= 1e-10
