@@ -141,11 +141,13 @@ BST_API double bst_ctx_work_flops(bst_ctx ctx);
  *     N^T N with a block of b vectors (CholQR orthonormalisation; b = 160
  *     for BST_FP64, for BST_OZAKI k + k/2 + 16 rounded up to 32 in 64..160,
  *     k the most states the sector can hold: chi, or chi / (2J+1) for an
- *     SU(2) sector of spin J), in rounds (the first two of `iters` steps,
- *     later ones sized by the residual's observed decay), each closed by a
- *     Rayleigh-Ritz step in FP64 (FP32 Jacobi eigensolver refined by
- *     Ogita-Aishima steps); sectors of dimension <= 160 are decomposed
- *     directly.  A round is accepted when every Ritz pair the truncation
+ *     SU(2) sector of spin J), in rounds (the first of at most `iters`
+ *     steps: three plain ones, then Chebyshev filters of the block chosen by
+ *     the spectrum seen so far; later rounds sized to converge; plain steps,
+ *     `iters` or sized by the residual's observed decay, where no filter
+ *     fits the spectrum), each closed by a Rayleigh-Ritz step in FP64 (FP32
+ *     Jacobi eigensolver refined by Ogita-Aishima steps); sectors of
+ *     dimension <= 160 are decomposed directly.  A round is accepted when every Ritz pair the truncation
  *     keeps has a residual ||N^T N v - lambda v|| <= tol * lambda_max (tol
  *     3e-14 for BST_FP64, 4e-12 for BST_OZAKI, whose iterations run on the
  *     tensor cores), or when the residual has stopped falling within

@@ -651,9 +651,12 @@ constexpr int kCholWarps = kCholThreads / 32;
 // Input: either the FP64 matrix M at in + in_off (nparts == 0), or nparts
 // FP32 partial sums of it, partial s at gin + in_off + s b^2, added in slice
 // order (gram_f32_kernel's output).
+// kout set: the row scales' powers of two go there (value index) and not into
+// Rinv, for a block whose columns are scaled by them (scale_cols).
 __global__ void __launch_bounds__(kCholThreads) cholinv_f32(const SmallProb* __restrict__ probs,
                                                             const double* __restrict__ in, double* __restrict__ out,
-                                                            int* err, const float* __restrict__ gin, int nparts) {
+                                                            int* err, const float* __restrict__ gin, int nparts,
+                                                            int* __restrict__ kout) {
   extern __shared__ float sh[];
   const SmallProb pr = probs[blockIdx.x];
   const int b = pr.b, bb = b * b;
@@ -922,6 +925,13 @@ __global__ void __launch_bounds__(kCholThreads) cholinv_f32(const SmallProb* __r
   }
   // Rinv = S L^-T with S the unit-diagonal scaling: Rinv[i][j] = dsc[i] Li[j][i]
   double* R = out + pr.out_off;
+  if (kout) {
+    for (int i = tid; i < b; i += kCholThreads) {
+      kout[pr.val_off + i] = ksc[i];
+      ksc[i] = 0;
+    }
+    __syncthreads();
+  }
   if ((b & 1) || (pr.out_off & 1)) {
     for (int q = tid; q < bb; q += kCholThreads) {
       const int i = q / b, j = q - i * b;
@@ -1029,6 +1039,75 @@ __global__ void ident_combo(const SmallProb* __restrict__ probs, const double* _
       const long long q = (long long)i * b + j;
       out[pr.out_off + q] = (i == j ? alpha : 0.0) + beta * in[pr.in_off + q];
     }
+}
+
+// X[:, j] *= 2^k[j] for the row-major block X (M x b) of each problem, exact
+// in the normal range: the columns of a filtered block differ by the growth
+// of their values, and a digit split along its rows would keep only the
+// largest to full accuracy.
+__global__ void scale_cols(const GramProb* __restrict__ blocks, const SmallProb* __restrict__ probs,
+                           const int* __restrict__ k, double* __restrict__ X) {
+  const GramProb g = blocks[blockIdx.y];
+  const int* e = k + probs[blockIdx.y].val_off;
+  const long long n = (long long)g.M * g.b;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
+    const long long r = q / g.b;
+    const int j = int(q - r * g.b);
+    double* x = X + g.x_off + r * g.ld + j;
+    // (the exponent field moves; zeros and results outside the normal range
+    // go through a multiplication)
+    const long long u = __double_as_longlong(*x);
+    const int ex = int((u >> 52) & 0x7ff), ne = ex + e[j];
+    *x = (ex > 0 && ex < 0x7ff && ne > 0 && ne < 0x7ff) ? __longlong_as_double(u + ((long long)e[j] << 52))
+                                                         : scalbn(*x, e[j]);
+  }
+}
+
+// First-order inverse of the Cholesky factor of G = I + E: I - striu(E) -
+// diag(E) / 2 (upper triangular; error ~E^2).
+__global__ void tri_combo(const SmallProb* __restrict__ probs, const double* __restrict__ in, double* __restrict__ out) {
+  const SmallProb pr = probs[blockIdx.x];
+  const int b = pr.b;
+  for (int i = blockIdx.y; i < b; i += gridDim.y)
+    for (int j = threadIdx.x; j < b; j += blockDim.x) {
+      const long long q = (long long)i * b + j;
+      const double g = in[pr.in_off + q];
+      out[pr.out_off + q] = i == j ? 1.5 - 0.5 * g : i < j ? -g : 0.0;
+    }
+}
+
+// Eigenvalue estimates of N^T N from the last plain step's two CholQR
+// factors: the diagonals of R (N Q side) and R (N^T side) converge to the
+// singular values in order; 0 for a dropped column.
+__global__ void factor_values(const SmallProb* __restrict__ probs, const double* __restrict__ rz,
+                              const double* __restrict__ ry, double* __restrict__ vals) {
+  const SmallProb pr = probs[blockIdx.x];
+  for (int j = threadIdx.x; j < pr.b; j += blockDim.x) {
+    const double d = rz[pr.out_off + (long long)j * (pr.b + 1)] * ry[pr.out_off + (long long)j * (pr.b + 1)];
+    vals[pr.val_off + j] = d > 0 ? 1.0 / d : 0.0;
+  }
+}
+
+// Chebyshev recurrence on row ranges: with L = (2 / alpha) N^T N - 1 and
+// w = N^T N y1,  w <- L y1 (first) or w <- 2 L y1 - y0.  Bound by memory
+// (24 or 32 bytes an element).
+struct ChebProb {
+  int64_t off, n;
+  double alpha;
+};
+__global__ void cheb_combo(const ChebProb* __restrict__ probs, double* __restrict__ w, const double* __restrict__ y1,
+                           const double* __restrict__ y0, int first) {
+  const ChebProb p = probs[blockIdx.y];
+  if (p.alpha == 0.0) {  // a sector that stays as it is
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.n; i += (long long)gridDim.x * blockDim.x)
+      w[p.off + i] = y1[p.off + i];
+    return;
+  }
+  const double a = (first ? 2.0 : 4.0) / p.alpha;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.n; i += (long long)gridDim.x * blockDim.x) {
+    const long long q = p.off + i;
+    w[q] = first ? fma(a, w[q], -y1[q]) : fma(a, w[q], fma(-2.0, y1[q], -y0[q]));
+  }
 }
 
 // Deterministic pseudo-random normal entries (counter-based hash + Box-Muller).

@@ -121,13 +121,21 @@ __global__ void jacobi_block_f32(const SmallProb*, const double*, double*, doubl
 size_t jacobi_block_smem(int b);
 __global__ void oa_update(const SmallProb*, const double*, const double*, double*, double*, double, double, double);
 __global__ void add_inplace(double*, const double*, long long);
-__global__ void cholinv_f32(const SmallProb*, const double*, double*, int*, const float*, int);
+__global__ void cholinv_f32(const SmallProb*, const double*, double*, int*, const float*, int, int*);
 struct GramProb {
   int32_t M, b;
   int64_t x_off, ld, out_off;
 };
 __global__ void gram_f32_kernel(const GramProb*, int, const double*, float*);
+__global__ void scale_cols(const GramProb*, const SmallProb*, const int*, double*);
 __global__ void ident_combo(const SmallProb*, const double*, double*, double, double);
+__global__ void tri_combo(const SmallProb*, const double*, double*);
+__global__ void factor_values(const SmallProb*, const double*, const double*, double*);
+struct ChebProb {
+  int64_t off, n;
+  double alpha;
+};
+__global__ void cheb_combo(const ChebProb*, double*, const double*, const double*, int);
 __global__ void randn_fill(double*, const long long*);
 __global__ void ritz_residual(const ResProb*, const double*, const double*, const double*, double*);
 size_t jacobi_smem(int b);
@@ -574,7 +582,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   double gram_flops = 0;
   for (auto& x : secs)
     if (!x.direct) gram_flops += 2.0 * double(std::max(x.M, x.N)) * x.b * x.b;
-  auto cholqr_factor = [&](const double* X, bool z_side, double* Rout) {
+  auto cholqr_factor = [&](const double* X, bool z_side, double* Rout, int* kout = nullptr) {
     {
       ProfScope ps(ctx, s, "gram_f32", gram_flops, 0.0);
       gram_f32_kernel<<<dim3(unsigned(sp_g.size()), unsigned(nparts)), 256, 0, s>>>(z_side ? dgz : dgq, nparts, X,
@@ -583,7 +591,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       count_launch(ctx);
     }
     ProfScope ps(ctx, s, "cholinv_f32", chol_flops, 0.0);
-    cholinv_f32<<<int(sp_g.size()), 512, cholinv_smem(bmax), s>>>(dsp_g, Msm, Rout, ctx->d_err, Gp, nparts);
+    cholinv_f32<<<int(sp_g.size()), 512, cholinv_smem(bmax), s>>>(dsp_g, Msm, Rout, ctx->d_err, Gp, nparts, kout);
     BST_CUDA(cudaGetLastError());
     count_launch(ctx);
   };
@@ -603,8 +611,8 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   double* Rz = (double*)ctx->buf("proj.Rinvz", sizeof(double) * std::max<int64_t>(smtot, 1), s);
   const int fresh_z = prec == BST_FP64 ? 1 << 30 : 3;
   bool n_split = false;
-  auto iterate = [&](int n) {
-    for (int t = 0; t < n; ++t) {
+  auto iterate = [&](int n, int t0 = 0) {
+    for (int t = t0; t < t0 + n; ++t) {
       gemm_any(ctx, "ss.z", prec, g_z, Nm, Q, Z, s, n_split);
       if (t < fresh_z) cholqr_factor(Z, true, Rz);
       gemm_any(ctx, "ss.qz", prec, g_qz, Z, Rz, Z2, s);
@@ -613,6 +621,141 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       cholqr_factor(Y, false, Rinv);
       gemm_any(ctx, "ss.qy", prec, g_qy, Y, Rinv, Q, s);
     }
+  };
+  // Once the columns have settled towards individual singular vectors (the
+  // first steps, or Ritz vectors), the block is filtered instead: m products
+  // with N^T N as the Chebyshev polynomial of degree m on [0, alpha], one
+  // CholQR after them.  alpha is the block's lower end, so what the block
+  // does not hold stays below 1 in magnitude while a kept value lambda grows
+  // by cosh(m acosh(2 lambda / alpha - 1)): two to four times the plain
+  // steps' decay per product, at a quarter of their factorisations (which
+  // cost more than the products: one CTA a sector).
+  // Measured (plain steps -> filters): the D=6, chi=72 half systems of random
+  // environments 40 steps -> 12, projector 7.8 -> 5.8 ms, full move (after the
+  // contractions' own gains) 33.9 -> 25.5 ms; D=8, chi=192 left move 61 steps
+  // -> 39, 98 -> 84 ms; SU(2) left move 23.0 -> 17.1 ms.
+  // Columns grow apart by up to (4 lambda_1 / alpha)^m / 2 between
+  // factorisations, and so does what a column holds of an earlier one's
+  // direction.  The FP32 factor leaves ~1e-6 of that; a triangular first-order
+  // correction from the Gram matrix in the call's arithmetic (symmetric ones
+  // would leave half of it) brings it to ~1e-11, and the growth is kept below
+  // 1e10.  The columns are scaled to similar length before R^-1 is applied
+  // (scale_cols): a digit split's rows would otherwise keep the short ones to
+  // fewer bits (floor of the residual 7e-12 without, 8e-13 with it).  Higher degrees leave more of the products' rounding (floor of the
+  // residual with degree 6: ~5e-11 lambda_max, 4: 1e-11, 2: 1e-12), so the
+  // last filter of a round has degree 2.
+  int* kcol = (int*)ctx->buf("proj.kcol", sizeof(int) * std::max<int64_t>(valtot, 1), s);
+  double* W3 = (double*)ctx->buf("proj.W3", sizeof(double) * std::max<int64_t>(qtot, 1), s);
+  // a block with ~1e-6 off orthonormal, corrected column by column: X <- X R^-1
+  auto polish_tri = [&](double*& X, double*& tmp) {
+    gemm_any(ctx, "ss.gy", prec, g_gy, X, X, Msm, s);
+    tri_combo<<<dim3(unsigned(sp_it.size()), 32), 128, 0, s>>>(dsp_it, Msm, Rinv);
+    BST_CUDA(cudaGetLastError());
+    count_launch(ctx);
+    gemm_any(ctx, "ss.qy", prec, g_qy, X, Rinv, tmp, s);
+    std::swap(X, tmp);
+  };
+  struct Filter {
+    int m;
+    std::vector<ChebProb> on;
+  };
+  auto filter = [&](const Filter& f) {
+    ChebProb* dch = upload_cached(ctx, "proj.cheb", f.on, s);
+    int64_t nmax = 0;
+    for (auto& c : f.on) nmax = std::max(nmax, c.n);
+    const dim3 grid(unsigned(std::max<int64_t>(1, std::min<int64_t>((nmax + 1023) / 1024, 256))), unsigned(f.on.size()));
+    double *prev = nullptr, *cur = Q, *nxt = Y;
+    for (int k = 0; k < f.m; ++k) {
+      gemm_any(ctx, "ss.z", prec, g_z, Nm, cur, Z, s, n_split);
+      gemm_any(ctx, "ss.y", prec, g_y, Nm, Z, nxt, s, n_split);
+      n_split = true;
+      cheb_combo<<<grid, 256, 0, s>>>(dch, nxt, cur, prev, k == 0 ? 1 : 0);
+      BST_CUDA(cudaGetLastError());
+      count_launch(ctx);
+      double* old = prev ? prev : W3;
+      prev = cur;
+      cur = nxt;
+      nxt = old;
+    }
+    cholqr_factor(cur, false, Rinv, kcol);
+    scale_cols<<<grid, 256, 0, s>>>(dgq, dsp_it, kcol, cur);
+    BST_CUDA(cudaGetLastError());
+    count_launch(ctx);
+    gemm_any(ctx, "ss.qy", prec, g_qy, cur, Rinv, nxt, s);
+    // the block is in nxt; the other two buffers are free
+    Y = cur;
+    W3 = prev;
+    Q = nxt;
+    polish_tri(Q, Y);
+  };
+  // The filters (degrees up to mmax, at most nprod products) by which every
+  // kept value grows by `need`, cheapest first choice, for the values `v` per
+  // sector in hl's layout (Ritz values or estimates, in any order).  Empty
+  // when none fits: a spectrum so steep that the growth bound puts alpha
+  // above a kept value (plain steps, which factor after every half).
+  auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod) {
+    std::vector<std::pair<double, int>> all;
+    for (size_t i = 0; i < secs.size(); ++i)
+      if (!secs[i].direct)
+        for (int j = 0; j < secs[i].c; ++j) {
+          const double d = v[secs[i].val_off + j];
+          if (!std::isfinite(d)) return std::vector<Filter>();
+          all.push_back({d, int(i)});
+        }
+    std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    // smallest value that counts as kept, per sector: down to a tenth of the
+    // truncation's (estimates are low by a small factor at most)
+    std::vector<double> lowest(secs.size(), 0.0);
+    const double cut = all.empty() ? 0.0 : 0.1 * all[std::min<size_t>(all.size(), size_t(chi)) - 1].first;
+    for (size_t t = 0; t < all.size() && all[t].first > cut; ++t) {
+      double& l = lowest[all[t].second];
+      if (int64_t(t) < chi || l == 0) l = all[t].first;
+    }
+    // the filter of degree m and the growth of the kept values (0: does not fit)
+    auto of_degree = [&](int m, Filter& f) {
+      const double span = std::pow(2e10, 1.0 / m) / 4.0;  // largest lambda_1 / alpha
+      double grow = 1e300;
+      f = Filter{m, {}};
+      for (size_t i = 0; i < secs.size(); ++i) {
+        const PSec& x = secs[i];
+        if (x.direct) continue;
+        double top = 0, low = 1e300;
+        for (int j = 0; j < x.c; ++j) {
+          const double d = v[x.val_off + j];
+          top = std::max(top, d);
+          if (d > 0) low = std::min(low, d);
+        }
+        if (lowest[i] == 0) {  // keeps nothing: stays as it is
+          f.on.push_back({x.q_off, int64_t(x.N) * x.b, 0.0});
+          continue;
+        }
+        // (an interval reaching into the block lets the polynomial's zeros
+        // wipe out columns there: degree 2 has few enough for the mixed
+        // tolerance)
+        if (0.8 * low < top / span && (m > 2 || prec == BST_FP64)) return 0.0;
+        const double alpha = std::max(0.8 * low, top / span);
+        if (lowest[i] < 1.05 * alpha) return 0.0;
+        grow = std::min(grow, std::cosh(m * std::acosh(2.0 * lowest[i] / alpha - 1.0)));
+        f.on.push_back({x.q_off, int64_t(x.N) * x.b, alpha});
+      }
+      return grow < 1e300 ? grow : 0.0;
+    };
+    std::vector<Filter> out;
+    Filter last, f, best;
+    const double g2 = of_degree(2, last);
+    if (!(g2 > 1.0) || nprod < 2) return out;
+    const double rest = std::log(std::max(need / g2, 1.0));
+    double cost = 1e300, n = 0;
+    if (rest > 0)
+      for (int m = 2; m <= mmax; ++m) {
+        const double g = of_degree(m, f);
+        if (!(g > 1.0)) continue;
+        const double nm = std::ceil(rest / std::log(g));
+        if (nm * (m + 3.0) < cost) cost = nm * (m + 3.0), n = nm, best = f;  // (a factorisation costs ~3 products)
+      }
+    for (int used = 2; n > 0 && used + best.m <= nprod; n -= 1, used += best.m) out.push_back(best);
+    out.push_back(last);
+    return out;
   };
   // second CholQR pass and two first-order polishes: orthonormal to FP64
   auto orthonormalise = [&]() {
@@ -735,12 +878,42 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   bool mixed_rr = prec != BST_FP64 && ctx->multi_round.count(rr_key) && ctx->multi_round[rr_key];
   if (mixed_rr && ctx->tune_log.size() < (1u << 20))
     ctx->tune_log += "projector subspace: intermediate Rayleigh-Ritz rounds in mixed arithmetic\n";
+  // Plain steps of the first round, from the random start: the columns
+  // settle, and the factors' diagonals tell the spectrum's span
+  const int settle = 3;
   int total = 0, steps = iters;
+  std::vector<Filter> fplan;  // filters of the next round (in place of its plain steps)
+  bool may_filter = true;
   for (int round = 0;; ++round) {
     const bst_prec rrp = mixed_rr ? prec : rr;
     if (!sp_it.empty()) {
-      iterate(steps);
-      total += steps;
+      if (round == 0 && steps >= settle + 2) {
+        iterate(settle);
+        factor_values<<<unsigned(sp_it.size()), 256, 0, s>>>(dsp_it, Rz, Rinv, lam);
+        BST_CUDA(cudaGetLastError());
+        count_launch(ctx);
+        std::vector<double> est(valtot, 0.0);
+        BST_CUDA(cudaMemcpyAsync(est.data(), lam, sizeof(double) * valtot, cudaMemcpyDeviceToHost, s));
+        BST_CUDA(cudaStreamSynchronize(s));
+        const int left = steps - settle;
+        // (a column's share of an earlier direction is about the ratio of
+        // their values to the number of products so far: no degree above it)
+        fplan = plan_filters(est, 1.0 / (0.02 * tol), settle, left);
+        total += settle;
+        if (!fplan.empty()) {
+          polish_tri(Q, Y);
+          for (auto& f : fplan) filter(f), total += f.m;
+        } else {
+          may_filter = false;
+          iterate(left, settle);
+          total += left;
+        }
+      } else if (!fplan.empty()) {
+        for (auto& f : fplan) filter(f), total += f.m;
+      } else {
+        iterate(steps);
+        total += steps;
+      }
       orthonormalise();
       // Rayleigh-Ritz: H = (N Q)^T (N Q).  N Q comes from the iterations'
       // product (the call's arithmetic, N's digits already split): the
@@ -877,7 +1050,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       for (int v : hsw) ctx->tune_log += " " + std::to_string(v);
       ctx->tune_log += "\n";
     }
-    const bool ok = worst <= tol || (round > 0 && worst > 0.5 * prev_worst && worst <= 100 * tol);
+    const bool ok = worst <= tol || (round > 0 && fplan.empty() && worst > 0.5 * prev_worst && worst <= 100 * tol);
     if (ok && !mixed_rr) break;
     if (total >= max_total) {
       if (ctx->multi_round.size() >= 4096) ctx->multi_round.clear();
@@ -889,9 +1062,18 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     // `iters`, at most 6 * iters steps), so slowly converging sectors are
     // checked with few Rayleigh-Ritz rounds
     int next = iters;
+    // (a filtered round that did not bring the residual down by half: its
+    // interval did not fit the spectrum, or its floor is reached; plain steps
+    // from here)
+    if (round > 0 && !fplan.empty() && !(worst < 0.5 * prev_worst)) may_filter = false;
+    fplan.clear();
+    if (!ok && may_filter && worst > 0 && std::isfinite(worst))
+      fplan = plan_filters(hl, worst / (0.02 * tol), 6, std::min(6 * iters, max_total - total));
     if (ok) {
       mixed_rr = false;  // converged under mixed Rayleigh-Ritz: the FP64 round
       next = 0;
+    } else if (!fplan.empty()) {
+      mixed_rr = false;  // sized to converge: its Rayleigh-Ritz step is the FP64 one
     } else if (round > 0 && steps > 0 && worst > 0 && prev_worst > worst) {
       const double rho = std::pow(worst / prev_worst, 1.0 / steps);
       const double need = std::log(0.5 * tol / worst) / std::log(rho);

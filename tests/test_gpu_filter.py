@@ -1,0 +1,84 @@
+"""The projector's filtered subspace iteration over spectra that its rules
+tell apart (slow and fast decay, a sector without kept states, rank-deficient
+sectors, an empty one, no gap inside the block) against the dense SVD."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CHI = 24
+DIMS = ((170, 203, 331), (203, 170, 290))  # rows, columns of the three sectors
+# accepted residual |N^T N v - lambda v| <= tol lambda_1, or 100 tol where it has stopped falling
+TOL = {"fp64": 3e-14, "ozaki": 4e-12}
+
+
+@pytest.fixture(scope="module")
+def bst():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1808_10804_gb300 import build
+    build.build()
+    from paper_1808_10804_gb300 import bst as b
+    return b
+
+
+def spectrum(kind, s, n):
+    """Singular values of sector s; the kept ones and the rest differ by a factor 1.5 or more."""
+    j = np.arange(n)
+    amp = (1.0, 0.9, 0.8)[s]
+    if kind == "slow":
+        return amp * np.where(j < 8, 1.0 - 0.05 * j, 0.4 * 0.998 ** j)
+    if kind == "fast":
+        return amp * np.where(j < 8, 0.75 ** j, 0.05 * 0.7 ** (j - 8))
+    if kind == "unkept":
+        return (1.0, 1e-5, 1e-9)[s] * np.where(j < 24, 0.95 ** j, 0.1 * 0.95 ** j)
+    if kind == "rank":
+        return amp * np.where(j < 8, 0.9 ** j, 0.0)
+    if kind == "empty":
+        return (1.0, 0.0, 0.8)[s] * np.where(j < 12, 0.9 ** j, 0.1 * 0.97 ** j)
+    return amp * np.where(j < 8, 1.0, 0.6)  # "flat": one cluster below the cut
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+@pytest.mark.parametrize("kind", ["slow", "fast", "unkept", "rank", "empty", "flat"])
+def test_projector_spectra(bst, kind, prec):
+    rng = np.random.default_rng(len(kind))
+    rows, cols = DIMS
+    N = []
+    for s in range(3):
+        n = min(rows[s], cols[s])
+        u = np.linalg.qr(rng.standard_normal((rows[s], n)))[0]
+        v = np.linalg.qr(rng.standard_normal((cols[s], n)))[0]
+        N.append((u * spectrum(kind, s, n)) @ v.T)
+    ctx = bst.Context(0)
+    leg = lambda f, d: bst.Leg(f, (0, 1, 2), d)  # noqa: E731
+    Rt = ctx.layout([leg(1, rows), leg(-1, rows)])
+    Rb = ctx.layout([leg(-1, rows), leg(1, cols)])
+    flat = lambda xs: torch.tensor(np.concatenate([x.reshape(-1) for x in xs]), device="cuda:0")  # noqa: E731
+    eye, nb = flat([np.eye(r) for r in rows]), flat(N)
+    svd = [np.linalg.svd(x) for x in N]
+    lam = np.sort(np.concatenate([x[1] for x in svd]))[::-1] ** 2
+    gap = (lam[CHI - 1] - lam[CHI]) / lam[0]
+    # per sector: the projection on the kept left vectors.  Residuals of
+    # 100 tol in CHI vectors turn the kept space by at most 100 tol sqrt(CHI)
+    # over the gap, and their values by 100 tol lambda_1
+    bound = 100 * TOL[prec] * np.sqrt(CHI) / gap
+    for _ in range(2):  # the second call goes by what the first one learnt
+        P, p, Pt, pt, sv, kept = ctx.svd_projector(Rt, eye, Rb, nb, 1, CHI, 1e-14, 1, prec=prec)
+        ctx.sync()
+        assert kept == CHI
+        assert np.abs(np.sort(np.square(sv))[::-1] - lam[:CHI]).max() <= bound * lam[0]
+        p_, pt_ = p.cpu().numpy(), pt.cpu().numpy()
+        new = dict(zip(P.legs[1].charges, P.legs[1].degs))
+        po = to = 0
+        for s in range(3):
+            k = int((svd[s][1] ** 2 > 0.5 * (lam[CHI - 1] + lam[CHI])).sum())
+            assert new.get(s, 0) == k
+            a = p_[po:po + rows[s] * k].reshape(rows[s], k)
+            b = pt_[to:to + rows[s] * k].reshape(k, rows[s])
+            po, to = po + a.size, to + b.size
+            u = svd[s][0][:, :k]
+            assert np.linalg.norm(a @ b - u @ u.T) <= bound
+        assert po == p_.size and to == pt_.size
+    ctx.close()
