@@ -580,12 +580,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // The outputs of problems with no matched block pair (K == 0), written by
-// the last CTAs of the split or pack launch (kZeroCtas per problem): beta * C
-// through the scatter tables, or zeros into the sector matrices of a plain
-// plan.
-constexpr int kZeroCtas = 8;
+// the last CTAs of the split or pack launch: beta * C through the scatter
+// tables, or zeros into the sector matrices of a plain plan.  Single-layer
+// moves leave hundreds of MB of them (charges that the contracted
+// legs do not reach), so a CTA takes whole rows of about 4096
+// elements and their number follows the size: with 8 CTAs a problem the D=8,
+// chi=192 absorption (60 M such elements beside 20 M to pack) took 3.5 ms,
+// now 0.28 ms, and the whole left move 84 -> 66 ms.
+constexpr int kZeroElems = 4096;  // elements of a CTA
+struct ZeroCta {
+  int prob, m0, m1;       // rows [m0, m1) of a problem (an index into zidx or zp)
+};
 struct ZeroJob {
-  int nz;
+  int n;                  // CTAs
+  const ZeroCta* ctas;
   const Prob* probs;      // scatter form: problems listed by zidx
   const int* zidx;
   Scatter sc;
@@ -594,25 +602,29 @@ struct ZeroJob {
 };
 
 __device__ __forceinline__ void zero_part(const ZeroJob& z, int cta) {
-  const int pi = cta / kZeroCtas, part = cta - pi * kZeroCtas;
-  const long long stride = (long long)kZeroCtas * blockDim.x;
+  const ZeroCta zc = z.ctas[cta];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  // lanes along a row; several rows a warp where they are short
+  auto each = [&](int N, auto&& row) {
+    const int lpr = N > 16 ? 32 : N > 8 ? 16 : N > 4 ? 8 : 4;
+    for (int m = zc.m0 + warp * (32 / lpr) + lane / lpr; m < zc.m1; m += nw * (32 / lpr)) row(m, lane % lpr, lpr);
+  };
   if (z.probs) {
-    const Prob p = z.probs[z.zidx[pi]];
-    const long long n = (long long)p.M * p.N;
-    for (long long e = part * (long long)blockDim.x + threadIdx.x; e < n; e += stride) {
-      const int m = int(e / p.N), c = int(e - (long long)m * p.N);
+    const Prob p = z.probs[z.zidx[zc.prob]];
+    each(p.N, [&](int m, int c0, int step) {
       const int2 ri = z.sc.rowtab[p.rt_off + m];
-      const int4 ci = z.sc.coltab[p.ct_off + c];
-      const long long dst = z.sc.bbase[p.bb_off + (long long)ri.x * p.ncc + ci.x] + (long long)ri.y * ci.z + ci.y;
-      z.C[dst] = z.sc.beta == 0.0 ? 0.0 : z.sc.beta * z.C[dst];
-    }
+      const long long* base = z.sc.bbase + p.bb_off + (long long)ri.x * p.ncc;
+      for (int c = c0; c < p.N; c += step) {
+        const int4 ci = z.sc.coltab[p.ct_off + c];
+        const long long dst = base[ci.x] + (long long)ri.y * ci.z + ci.y;
+        z.C[dst] = z.sc.beta == 0.0 ? 0.0 : z.sc.beta * z.C[dst];
+      }
+    });
   } else {
-    const GemmProb p = z.zp[pi];
-    const long long n = (long long)p.M * p.N;
-    for (long long e = part * (long long)blockDim.x + threadIdx.x; e < n; e += stride) {
-      const long long m = e / p.N, c = e - m * p.N;
-      z.C[p.c_off + m * p.c_m + c * p.c_n] = 0.0;
-    }
+    const GemmProb p = z.zp[zc.prob];
+    each(p.N, [&](int m, int c0, int step) {
+      for (int c = c0; c < p.N; c += step) z.C[p.c_off + m * p.c_m + c * p.c_n] = 0.0;
+    });
   }
 }
 
@@ -853,7 +865,7 @@ __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob 
                                                                     int csize, int kpitch, ZeroJob zj) {
   if (int(blockIdx.x) >= gab) {
     const int z = int(blockIdx.x) - gab;
-    if (z < zj.nz * kZeroCtas) zero_part(zj, z);
+    if (z < zj.n) zero_part(zj, z);
     return;
   }
   const bool is_a = int(blockIdx.x) < ga;
@@ -1208,7 +1220,7 @@ __global__ void __launch_bounds__(kSplitThreads, 3) pack_split_kernel(PackJob ja
                                                                       int csize, int kpitch, ZeroJob zj) {
   if (int(blockIdx.x) >= gab) {
     const int z = int(blockIdx.x) - gab;
-    if (z < zj.nz * kZeroCtas) zero_part(zj, z);
+    if (z < zj.n) zero_part(zj, z);
     return;
   }
   const bool is_a = int(blockIdx.x) < ga;
@@ -1283,7 +1295,8 @@ struct OzakiPlan {
   // (its epilogue then always waits for products of that tile, which keeps
   // the CTA's mbarrier phases in step)
   GemmProb* d_zprobs = nullptr;
-  int nzprobs = 0;
+  oz::ZeroCta* d_zctas = nullptr;
+  int nzctas = 0;
   // output scatter into canonical blocks (plans built by
   // ozaki_prepare_scatter): tables on the device, K == 0 problems listed
   // by index for the beta-only pass
@@ -1314,6 +1327,7 @@ struct OzakiPlan {
     cudaFree(d_coltab);
     cudaFree(d_bbase);
     cudaFree(d_zidx);
+    cudaFree(d_zctas);
     cudaFree(d_probs);
     cudaFree(d_tiles);
     cudaFree(d_sa);
@@ -1539,7 +1553,13 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   up(&P->d_probs, hp);
   up(&P->d_tiles, ht);
   up(&P->d_zprobs, zp);
-  P->nzprobs = int(zp.size());
+  std::vector<oz::ZeroCta> zc;
+  for (size_t i = 0; i < zp.size(); ++i) {
+    const int rows = std::max(1, oz::kZeroElems / std::max(zp[i].N, 1));
+    for (int m = 0; m < zp[i].M; m += rows) zc.push_back({int(i), m, std::min(zp[i].M, m + rows)});
+  }
+  up(&P->d_zctas, zc);
+  P->nzctas = int(zc.size());
   up(&P->d_sa, sa);
   up(&P->d_sb, sb);
   up(&P->d_ca, ca);
@@ -1603,9 +1623,9 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
     ProfScope ps(ctx, s, "pack_bf16", 0.0, P->split_bytes);
     const oz::PackJob ja{P->d_pgA, P->d_psA, P->d_pcA, P->rowsA, A, tabA, P->SA, P->eA};
     const oz::PackJob jb{P->d_pgB, P->d_psB, P->d_pcB, P->rowsB, B, tabB, P->SB, P->eB};
-    const oz::ZeroJob zj{P->nzprobs, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
+    const oz::ZeroJob zj{P->nzctas, P->d_zctas, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
     const int cs = P->pack_cluster;
-    const int gz = (P->nzprobs * oz::kZeroCtas + cs - 1) / cs * cs;
+    const int gz = (P->nzctas + cs - 1) / cs * cs;
     auto pack = [&](int ga, int gb, int z) {
       if (ga + gb + z == 0) return;
       launch_clusters(P->S == 5 ? oz::pack_split_kernel<5> : oz::pack_split_kernel<3>, ga + gb + z, oz::kSplitThreads,
@@ -1625,8 +1645,8 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
     ProfScope ps(ctx, s, "split_bf16", 0.0, b_from_a ? 0.5 * P->split_bytes : P->split_bytes);
     const int cs = P->split_cluster;
     const int ga = (split_a && P->ntiles) ? P->split_ca : 0, gb = (b_from_a || !P->ntiles) ? 0 : P->split_cb;
-    const int gz = (P->nzprobs * oz::kZeroCtas + cs - 1) / cs * cs;
-    const oz::ZeroJob zj{P->nzprobs, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
+    const int gz = (P->nzctas + cs - 1) / cs * cs;
+    const oz::ZeroJob zj{P->nzctas, P->d_zctas, P->scatter ? P->d_probs : nullptr, P->d_zidx, sc, P->d_zprobs, C};
     if (ga + gb + gz > 0) {
       const oz::SplitJob ja{P->d_sa, P->d_ca, P->rowsA, A, P->SA, P->eA};
       const oz::SplitJob jb{P->d_sb, P->d_cb, P->rowsB, B, P->SB, P->eB};

@@ -89,3 +89,28 @@ def test_interleaved_operands(bst, ctx, n):
     assert np.abs(got[0].cpu().numpy() - lam).max() <= 1e-11
     X = X[0].cpu().numpy()
     assert np.abs(X.T @ X - np.eye(n)).max() <= 1e-10
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+@pytest.mark.parametrize("M,N", [(1, 1), (3, 4), (70, 5), (9, 16), (33, 17), (1300, 33), (2, 4097), (4100, 63)])
+def test_unmatched_output_sectors(bst, ctx, M, N, beta):
+    """Output sectors no block pair reaches (the contracted leg has no such
+    charge) come out as beta * C, to the bit; two legs a side, so that rows
+    and columns run over several blocks."""
+    rng = np.random.default_rng([M, N])
+    t = lambda n: torch.tensor(rng.standard_normal(n), device="cuda:0")  # noqa: E731
+    A = ctx.layout([bst.Leg(1, (0, 1), (1, 2)), bst.Leg(1, (0, 2), (2, M)), bst.Leg(-1, (0,), (3,))])
+    B = ctx.layout([bst.Leg(1, (0,), (3,)), bst.Leg(-1, (0, 2), (2, N)), bst.Leg(-1, (0, 1), (1, 2))])
+    C = ctx.contract_layout(A, B, (2,), (0,))
+    a, b, c = t(A.nnz), t(B.nnz), t(C.nnz)
+    old = c.cpu().numpy().copy()
+    got = {}
+    for prec in ("ozaki", "fp64"):
+        got[prec] = ctx.contract(A, a, B, b, (2,), (0,), prec=prec, beta=beta, Cl=C, c=c.clone())[1]
+    ctx.sync()
+    ref = got["fp64"].cpu().numpy()
+    out = got["ozaki"].cpu().numpy()
+    zero = ref == beta * old  # entries the plain FP64 path left at beta * C
+    assert zero.sum() >= M * N
+    assert np.array_equal(out[zero], (beta * old)[zero])
+    assert np.abs(out - ref)[~zero].max(initial=0.0) <= 1e-10
