@@ -33,8 +33,13 @@
 // divisions, tile tables that hold all a role needs, one copy per operand and
 // chunk, barriers looked at ahead of time, and no conversion instruction in
 // the epilogue that an addition replaces.  2432 x 2432 x 2432, five digits:
-// 430 -> 375 us (1.15 PFLOP/s of digit products); four of 2048 x 2048 x 512:
-// 347 -> 287 us; 2432^3 with three digits: 292 -> 229 us.
+// 430 -> 352 us (1.23 PFLOP/s of digit products); four of 2048 x 2048 x 512:
+// 347 -> 253 us; 2432^3 with three digits: 292 -> 233 us.  A tile of one or
+// two chunks is bound by the instructions of its output instead (about 100 an
+// element for four warps a scheduler): 200000 x 192 x 16, 307 MB out, 243 ->
+// 199 us with sums that need no shift or sign extension, 32-bit halves in the
+// conversion and four rows side by side.  The launch is programmatic behind
+// the split or pack: 1.6 us less per contraction.
 //
 // Every wait of the pipeline
 // is bounded by the launch's spin limit: on expiry the kernel records
@@ -111,10 +116,12 @@ struct Scatter {
 };
 
 struct Tile {
-  int32_t prob, m0, n0;
+  int32_t prob;
+  int32_t m0, n0;      // first row and column; their low bits (m0: 7, n0: those of TN - 1) hold the
+                       // tile's rows and columns inside the problem, less one
   int32_t nk;          // K chunks of kTK
   int32_t arow, brow;  // the tile's first rows in the split A / B buffers
-  int32_t pad[2];
+  int32_t rt, ct;      // its first entries in the scatter's row and column tables
 };
 
 struct SplitTask {
@@ -216,6 +223,13 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "r"(taddr));
 }
 
+// A grid launched behind another with programmatic serialisation may start
+// when every block of the first has called grid_trigger (or left), and must
+// call grid_wait, which returns when the first has finished and its writes
+// are visible, before it touches what that grid reads or writes.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -223,23 +237,44 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // X 2^e rounded to nearest even, built from the IEEE fields: the FP64 pipe
 // of this part issues about two operations per clock and SM, so a conversion
 // and two products per output cost a 128 x 64 tile ~12000 cycles, more than
-// the products of a K = 128 tile.  Results outside the normal range take the
-// FP64 route.
-__device__ __forceinline__ double scaled_double(long long X, int e) {
-  const unsigned long long u = X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X;
-  const int lz = __clzll((long long)u);
-  const unsigned long long n = u << (lz & 63);
-  const int ex = 1085 - lz + e;  // biased exponent less one of the leading bit's weight 2^(63 - lz + e)
-  // mantissa with its leading bit, plus the round bit (ties to even)
-  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull & ((n & 0x3ffull) || (n & 0x800ull) ? 1ull : 0ull));
-  const unsigned long long bits = ((unsigned long long)(unsigned)ex << 52) + m;
-  if (ex < 1 || ex > 2043 || u == 0) {
-    const int h = max(-1022, min(1023, e >> 1)), l = max(-1022, min(1023, e - (e >> 1)));
-    return double(X) * __longlong_as_double((long long)(h + 1023) << 52) *
-           __longlong_as_double((long long)(l + 1023) << 52);
-  }
-  return __longlong_as_double((long long)(bits | (X < 0 ? 0x8000000000000000ull : 0ull)));
+// the products of a K = 128 tile.  In 32-bit halves (half the instructions of
+// 64-bit shifts and counts).  Results outside the normal range take the FP64
+// route.
+// (out: such a result, the value returned is not it)
+__device__ __forceinline__ double scaled_double(long long X, int e, bool& out) {
+  const long long sg = X >> 63;
+  const unsigned long long u = (unsigned long long)((X ^ sg) - sg);
+  const uint32_t uh = uint32_t(u >> 32), ul = uint32_t(u);
+  const bool narrow = uh == 0;
+  const uint32_t h = narrow ? ul : uh, l = narrow ? 0u : ul;
+  const int lz = __clz(int(h));
+  // normalised: leading bit at bit 63 (X = 0: no matter, 0 is returned)
+  const uint32_t nh = __funnelshift_l(l, h, lz), nl = l << (lz & 31);
+  const int ex = (narrow ? 1053 : 1085) - lz + e;  // biased exponent less one of the leading bit's weight
+  const uint32_t tie = (nl >> 11) & 1u;
+  const uint32_t up = (nl & 0x7ffu) + tie > 0x400u ? 1u : 0u;  // round to nearest, ties to even
+  const unsigned long long m =
+      ((unsigned long long)((uint32_t(ex) << 20) + (nh >> 11)) << 32 | __funnelshift_r(nl, nh, 11)) + up;
+  out = u != 0 && (ex < 1 || ex > 2043);
+  return u == 0 ? 0.0 : __longlong_as_double((long long)(m | ((unsigned long long)sg & 0x8000000000000000ull)));
 }
+
+__device__ __noinline__ double scaled_double_far(long long X, int e) {
+  const int eh = max(-1022, min(1023, e >> 1)), el = max(-1022, min(1023, e - (e >> 1)));
+  return double(X) * __longlong_as_double((long long)(eh + 1023) << 52) *
+         __longlong_as_double((long long)(el + 1023) << 52);
+}
+
+// a b + c, 64 bits wide (modulo 2^64: the accumulators carry the patterns of
+// the rounding constants below until their sum is taken off)
+__device__ __forceinline__ unsigned long long mad_wide(int a, int b, unsigned long long c) {
+  return (unsigned long long)((long long)a * b) + c;
+}
+// Adding 3 2^22 to an FP32 number of magnitude up to 2^22 rounds it to an
+// integer and puts that in the low bits of the pattern: the conversion
+// without the slow conversion instructions.
+constexpr float kMagic = 12582912.0f;
+constexpr int kMagicBits = 0x4B400000;
 
 constexpr int kOutLd = 9;  // 8 columns (odd stride: rows fall on different banks)
 template <int S, int TN>
@@ -299,6 +334,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // everything before this overlaps the end of the split or pack launch
+  grid_wait();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort_flag = &sm.abort_flag;
 
@@ -451,24 +488,48 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int ti = blockIdx.x; ti < ntiles && ok;) {
       ti += gridDim.x;
       const Tile nxt = ti < ntiles ? tiles[ti] : t;
-      const Prob p = probs[t.prob];
       // the tile's rows and columns, loaded while its products run: lane l
       // holds row l's exponent and scatter entry, and those of the columns
-      // that it writes, c0 + (l & 7) (+ 8)
-      const bool row_ok = t.m0 + row < p.M;
-      const int ea = row_ok ? expA[t.arow + row] - CF::kShift : 0;
+      // that it writes, c0 + (l & 7) (+ 8).  Everything hangs on the tile
+      // alone, which came with the one before: of a tile of one chunk the
+      // chain tile - problem - tables was a good part.
+      const int mrows = (t.m0 & (kTM - 1)) + 1 - q * 32, ncols = (t.n0 & (TN - 1)) + 1 - c0;
+      const bool idle = mrows <= 0 || ncols <= 0;  // this warp's part lies past the problem
+      const bool scatter = sc.rowtab != nullptr;
+      const Prob* p = probs + t.prob;
+      const int ea = lane < mrows ? expA[t.arow + row] - CF::kShift : 0;
       int2 ri = make_int2(0, 0);
-      if (p.scatter && row_ok) ri = sc.rowtab[p.rt_off + t.m0 + row];
-      int eb[kCols / 8];
-      int4 ci[kCols / 8];
+      int ncc = 0;
+      long long bb_off = 0;
+      if (scatter) {
+        if (!idle) ri = sc.rowtab[t.rt + q * 32 + min(lane, mrows - 1)];
+        ncc = p->ncc;
+        bb_off = p->bb_off;
+      }
+      // (the output block of this lane's first row in every 8 columns: offset
+      // of the column's first row there, and the block's row length)
+      const bool one_blk = __all_sync(0xffffffffu, ri.x == __shfl_sync(0xffffffffu, ri.x, 0));
+      const int rx0 = __shfl_sync(0xffffffffu, ri.x, lane >> 3);
+      int eb[kCols / 8], cw[kCols / 8];
+      long long cb[kCols / 8];
 #pragma unroll
       for (int h = 0; h < kCols / 8; ++h) {
-        const int gn = t.n0 + c0 + h * 8 + (lane & 7);
-        eb[h] = gn < p.N ? expB[p.brow + gn] : 0;
-        ci[h] = p.scatter && gn < p.N ? sc.coltab[p.ct_off + gn] : make_int4(0, 0, 0, 0);
+        const int col = h * 8 + (lane & 7);
+        eb[h] = cw[h] = 0;
+        cb[h] = 0;
+        if (col < ncols) {
+          eb[h] = expB[t.brow + c0 + col];
+          if (scatter) {
+            const int4 ci = sc.coltab[t.ct + c0 + col];
+            cw[h] = ci.z;
+            cb[h] = sc.bbase[bb_off + (long long)rx0 * ncc + ci.x] + ci.y;
+          }
+        }
       }
-      // T = sum over chunk pairs of (S0 2^18 + S1 2^9 + S2): exact in 64 bits
-      long long T[kCols];
+      // X = sum over chunk pairs of (S0 2^18 + S1 2^9 + S2) 2^(9 if S = 5), plus
+      // S3 + S4 2^-9: integers below 2^63, summed modulo 2^64
+      constexpr int kUp = S == 5 ? 9 : 0;
+      unsigned long long T[kCols];
 #pragma unroll
       for (int j = 0; j < kCols; ++j) T[j] = 0;
       const int npair = (t.nk + 1) >> 1;
@@ -476,6 +537,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         ok = mbar_wait(&sm.acc_full[buf], bph, abort_flag, err, spin);
         if (!ok) break;
         tc_fence_after();
+        if (idle) {
+          mbar_arrive(&sm.acc_empty[buf]);
+          buf ^= 1u;
+          if (buf == 0) bph ^= 1u;
+          continue;
+        }
         // The three diagonals of 8 columns per wait; the buffer goes back
         // to the products as soon as its last load has landed, before the
         // conversions.  |S0| <= 64 2^16 = 2^22: adding 3 2^22 puts it in the
@@ -495,18 +562,27 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            T[h + j] += (long long)__float_as_int(__uint_as_float(v0[j]) + 12582912.0f) * (1 << 18);
-            T[h + j] += (long long)__float2int_rn(__uint_as_float(v1[j])) * (1 << 9);
-            T[h + j] += __float2int_rn(__uint_as_float(v2[j]));
+            T[h + j] = mad_wide(__float_as_int(__uint_as_float(v0[j]) + kMagic), 1 << (18 + kUp), T[h + j]);
+            T[h + j] = mad_wide(__float2int_rn(__uint_as_float(v1[j])), 1 << (9 + kUp), T[h + j]);
+            T[h + j] = mad_wide(__float2int_rn(__uint_as_float(v2[j])), 1 << kUp, T[h + j]);
           }
         }
         buf ^= 1u;
         if (buf == 0) bph ^= 1u;
       }
       if (!ok) break;
-      const long long off0 = ((long long)npair * 0x4B400000ll) << 18;
-      // S = 5: X = T 2^9 + (S3 + S4 2^-9); d3 and d4 go back to the next
-      // tile's products, which wait for them, before any output is written
+      if (idle) {
+        if constexpr (S == 5) mbar_arrive(&sm.acc34_empty);
+        t = nxt;
+        continue;
+      }
+      // d3 and d4 go back to the next tile's products, which wait for them,
+      // before any output is written.  S3 + S4 2^-9 to the nearest integer as
+      // 2^12 H + R, both by the constant (sums up to 2^34, K of 32768: past
+      // that by the 64-bit conversion, which goes through the FP64 pipe)
+      const bool wide = t.nk > 1024;
+      const unsigned long long off0 = ((unsigned long long)npair * kMagicBits) << (18 + kUp);
+      const unsigned long long off = off0 + (S == 5 && !wide ? (unsigned long long)kMagicBits * 4097 : 0);
 #pragma unroll
       for (int h = 0; h < kCols; h += 8) {
         if constexpr (S == 5) {
@@ -516,13 +592,19 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_wait_ld();
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float small = __uint_as_float(w3[j]) + __uint_as_float(w4[j]) * (1.0f / 512.0f);
-            T[h + j] = ((T[h + j] - off0) << 9) + __float2ll_rn(small);
+            const float x = fmaf(__uint_as_float(w4[j]), 1.0f / 512.0f, __uint_as_float(w3[j]));
+            if (wide) {
+              T[h + j] += (unsigned long long)__float2ll_rn(x);
+            } else {
+              const float hc = fmaf(x, 1.0f / 4096.0f, kMagic);
+              const float r = fmaf(hc - kMagic, -4096.0f, x);  // exact, at most 2^11
+              T[h + j] = mad_wide(__float_as_int(hc), 4096, T[h + j]);
+              T[h + j] = mad_wide(__float_as_int(r + kMagic), 1, T[h + j]);
+            }
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) T[h + j] -= off0;
         }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) T[h + j] -= off;
       }
       if constexpr (S == 5) {
         tc_fence_before();
@@ -535,36 +617,69 @@ __global__ void __launch_bounds__(kThreads, 1)
       // blocks, row (ri.x, ri.y) and column (ci.x, ci.y) of the block (ri.x,
       // ci.x) of width ci.z; else the sector matrix.
       long long(*st)[kOutLd] = sm.out[warp - 2];
-      const bool plain = !p.scatter || (sc.alpha == 1.0 && sc.beta == 0.0);
-      const int mrows = p.M - t.m0 - q * 32;
+      const bool plain = !scatter || (sc.alpha == 1.0 && sc.beta == 0.0);
 #pragma unroll
       for (int h = 0; h < kCols / 8; ++h) {
+        if (h * 8 >= ncols) break;
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) st[lane][j] = T[h * 8 + j];
+        for (int j = 0; j < 8; ++j) st[lane][j] = (long long)T[h * 8 + j];
         __syncwarp();
-        const int gn = t.n0 + c0 + h * 8 + (lane & 7);
-        const bool col_ok = gn < p.N;
-        int rblk = -1;
-        long long cbase = 0;
-#pragma unroll 4
-        for (int i = 0; i < 8; ++i) {
-          const int r = 4 * i + (lane >> 3);
-          const double v = scaled_double(st[r][lane & 7], __shfl_sync(0xffffffffu, ea, r) + eb[h]);
-          const bool live = col_ok && r < mrows;
-          if (p.scatter) {
-            const int rx = __shfl_sync(0xffffffffu, ri.x, r), ry = __shfl_sync(0xffffffffu, ri.y, r);
-            if (live) {
-              if (rx != rblk) {
-                rblk = rx;
-                cbase = sc.bbase[p.bb_off + (long long)rx * p.ncc + ci[h].x] + ci[h].y;
-              }
-              double* dst = C + cbase + (long long)ry * ci[h].z;
-              if (plain) *dst = v;
-              else *dst = sc.beta == 0.0 ? sc.alpha * v : fma(sc.alpha, v, sc.beta * *dst);
+        const int col = h * 8 + (lane & 7);
+        const bool col_ok = col < ncols;
+        double* cbase;
+        int rstride;  // between output rows of a block
+        if (scatter) {
+          cbase = C + cb[h];
+          rstride = cw[h];
+        } else {
+          rstride = int(p->c_m);
+          cbase = C + p->c_off + (long long)((t.m0 & ~(kTM - 1)) + q * 32) * rstride +
+                  (long long)((t.n0 & ~(TN - 1)) + c0 + col) * p->c_n;
+        }
+        // (the values of four rows side by side: the shared load, shuffle and
+        // conversion of one are a chain that four warps a scheduler do not
+        // hide)
+        constexpr int kRows = 4;
+#pragma unroll
+        for (int g = 0; g < 8 / kRows; ++g) {
+          if (4 * kRows * g >= mrows) break;
+          const int r0 = 4 * kRows * g + (lane >> 3);  // rows r0, r0 + 4, ..
+          double v[kRows];
+          double* dst[kRows];
+          bool far = false, out[kRows];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            const int r = r0 + 4 * i;
+            dst[i] = cbase + (long long)(scatter ? __shfl_sync(0xffffffffu, ri.y, r) : r) * rstride;
+            v[i] = scaled_double(st[r][lane & 7], __shfl_sync(0xffffffffu, ea, r) + eb[h], out[i]);
+            far = far || out[i];
+          }
+          if (__any_sync(0xffffffffu, far)) {
+#pragma unroll 1
+            for (int i = 0; i < kRows; ++i) {
+              const int r = r0 + 4 * i;
+              const double x = scaled_double_far(st[r][lane & 7], __shfl_sync(0xffffffffu, ea, r) + eb[h]);
+#pragma unroll
+              for (int k = 0; k < kRows; ++k)
+                if (k == i && out[k]) v[k] = x;
             }
-          } else if (live) {
-            C[p.c_off + (long long)(t.m0 + q * 32 + r) * p.c_m + (long long)gn * p.c_n] = v;
+          }
+          if (!one_blk) {  // (rows of several blocks: the columns' table entries again)
+            const int4 ci = col_ok ? sc.coltab[t.ct + c0 + col] : make_int4(0, 0, 0, 0);
+            const long long* bb = sc.bbase + p->bb_off + ci.x;
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+              const int rx = __shfl_sync(0xffffffffu, ri.x, r0 + 4 * i), my = __shfl_sync(0xffffffffu, ri.y, r0 + 4 * i);
+              if (col_ok) dst[i] = C + bb[(long long)rx * p->ncc] + ci.y + (long long)my * rstride;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            if (col_ok && r0 + 4 * i < mrows) {
+              if (plain) *dst[i] = v[i];
+              else *dst[i] = sc.beta == 0.0 ? sc.alpha * v[i] : fma(sc.alpha, v[i], sc.beta * *dst[i]);
+            }
           }
         }
       }
@@ -863,6 +978,7 @@ __device__ __forceinline__ void split_cols(const SplitJob& J, const SplitTask& t
 template <int S>
 __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob ja, SplitJob jb, int ga, int gab,
                                                                     int csize, int kpitch, ZeroJob zj) {
+  grid_trigger();
   if (int(blockIdx.x) >= gab) {
     const int z = int(blockIdx.x) - gab;
     if (z < zj.n) zero_part(zj, z);
@@ -1218,6 +1334,7 @@ __device__ __forceinline__ void pack_cols(PackShared& sm, const PackJob& J, cons
 template <int S>
 __global__ void __launch_bounds__(kSplitThreads, 3) pack_split_kernel(PackJob ja, PackJob jb, int ga, int gab,
                                                                       int csize, int kpitch, ZeroJob zj) {
+  grid_trigger();
   if (int(blockIdx.x) >= gab) {
     const int z = int(blockIdx.x) - gab;
     if (z < zj.n) zero_part(zj, z);
@@ -1501,7 +1618,9 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
     const int pi = int(hp.size());
     hp.push_back(q);
     auto add_tile = [&](int i, const oz::Prob& o, int m0, int n0) {
-      ht.push_back({i, m0, n0, (o.K + oz::kTK - 1) / oz::kTK, o.arow + m0, o.brow + n0, {0, 0}});
+      ht.push_back({i, m0 | (std::min(oz::kTM, o.M - m0) - 1), n0 | (std::min(TN, o.N - n0) - 1),
+                    (o.K + oz::kTK - 1) / oz::kTK, o.arow + m0, o.brow + n0, int32_t(o.rt_off + m0),
+                    int32_t(o.ct_off + n0)});
     };
     if (g.K == 0) {
       zp.push_back(g);
@@ -1662,8 +1781,19 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
   const CUtensorMap& mB = b_from_a ? P->mapBA : P->mapB;
   const int* eB = b_from_a ? P->eA : P->eB;
   auto launch = [&](auto kern, size_t smem) {
-    kern<<<grid, oz::kThreads, smem, s>>>(P->mapA, mB, P->d_probs, P->d_tiles, P->ntiles, P->eA, eB, C, sc,
-                                         ctx->d_err, spin);
+    // (behind the split or pack, whose last blocks its prologue overlaps)
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(oz::kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    BST_CUDA(cudaLaunchKernelEx(&cfg, kern, P->mapA, mB, (const oz::Prob*)P->d_probs, (const oz::Tile*)P->d_tiles,
+                                P->ntiles, (const int*)P->eA, eB, C, sc, ctx->d_err, spin));
   };
   if (P->S == 5 && P->TN == 64) {
     set_kernel_attrs<5, 64>();
