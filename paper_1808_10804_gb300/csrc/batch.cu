@@ -36,6 +36,7 @@ struct BatchTask {
 
 struct BatchRel {
   BatchTask* tasks = nullptr;
+  RelBox* boxes = nullptr;
   int2* chunks = nullptr;
   int nchunks = 0;
   int chunk = 2048;  // elements per CTA
@@ -43,8 +44,10 @@ struct BatchRel {
   std::vector<BatchTask> host;
   void free_all() {
     cudaFree(tasks);
+    cudaFree(boxes);
     cudaFree(chunks);
     tasks = nullptr;
+    boxes = nullptr;
     chunks = nullptr;
   }
 };
@@ -98,15 +101,17 @@ struct BatchPlan {
 constexpr int kBatchThreads = 256;
 constexpr int kChunkChoices[] = {1024, 2048, 4096, 8192};
 
-// Same element mapping as relayout_kernel, with a per-task base pointer.
+// Same copies as relayout_legs_kernel, with a per-task base pointer.
 __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const BatchTask* __restrict__ tasks,
+                                                                       const RelBox* __restrict__ boxes,
                                                                        const int2* __restrict__ chunks,
                                                                        double* const* __restrict__ bases,
                                                                        double* mat, int dir, double alpha,
                                                                        double beta, int chunk) {
   const int2 c = chunks[blockIdx.x];
+  __shared__ RelLegs sh;
   const BatchTask& bt = tasks[c.x];
-  relayout_range<kBatchThreads>(bt.t, c.y, min(bt.t.n, c.y + chunk), bases[bt.src], mat, dir, alpha, beta);
+  relayout_legs<kBatchThreads>(sh, boxes[c.x], c.y, min(bt.t.n, c.y + chunk), bases[bt.src], mat, dir, alpha, beta);
 }
 
 // (Re)build the chunk table of a relayout for `chunk` elements per CTA.
@@ -123,6 +128,10 @@ static void upload_rel(BatchRel& r, int chunk) {
   if (!r.host.empty()) {
     BST_CUDA(cudaMalloc(&r.tasks, sizeof(BatchTask) * r.host.size()));
     BST_CUDA(cudaMemcpy(r.tasks, r.host.data(), sizeof(BatchTask) * r.host.size(), cudaMemcpyHostToDevice));
+    std::vector<RelBox> hb(r.host.size());
+    for (size_t i = 0; i < hb.size(); ++i) rel_make_box(r.host[i].t, hb[i]);
+    BST_CUDA(cudaMalloc(&r.boxes, sizeof(RelBox) * hb.size()));
+    BST_CUDA(cudaMemcpy(r.boxes, hb.data(), sizeof(RelBox) * hb.size(), cudaMemcpyHostToDevice));
   }
   if (!ch.empty()) {
     BST_CUDA(cudaMalloc(&r.chunks, sizeof(int2) * ch.size()));
@@ -134,7 +143,7 @@ static void launch_rel(Ctx* ctx, const BatchRel& r, double* const* bases, double
                        double beta, cudaStream_t s) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  relayout_batch_kernel<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.chunks, bases, mat, dir, alpha, beta,
+  relayout_batch_kernel<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, bases, mat, dir, alpha, beta,
                                                             r.chunk);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);

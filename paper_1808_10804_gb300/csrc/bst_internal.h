@@ -125,12 +125,17 @@ struct MatView {
   }
 };
 
-// A relayout ready to launch: tasks and chunk table on the device.
+struct RelBox;
+
+// A relayout ready to launch: tasks and chunk table on the device, and the
+// tasks' boxes (null in contract_noalloc's fixed scratch: a slower kernel).
 struct DevRelayout {
   RelTask* tasks = nullptr;
+  RelBox* boxes = nullptr;
   int2* chunks = nullptr;
   int nchunks = 0;
   int ntasks = 0;
+  bool transposes = false;  // copied by boxes through shared memory
   double elems = 0;
   void upload(const std::vector<RelTask>& t);
   void free_all();

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "bst_internal.h"
+#include "relayout_dev.cuh"
 
 namespace bst {
 
@@ -313,11 +314,18 @@ static void build_view(Ctx* ctx, const Layout* L, const std::vector<int>& rowleg
   BST_CUDA(cudaMalloc(&out->secs, sizeof(DevSector) * std::max<long long>(v.cn, 1)));
   BST_CUDA(cudaMalloc(&out->rel.tasks, sizeof(RelTask) * std::max<long long>(nb, 1)));
   BST_CUDA(cudaMalloc(&out->rel.chunks, sizeof(int2) * std::max<long long>(nchunk_max, 1)));
+  const bool boxes = nb > 0 && L->nnz < (int64_t(1) << 31);  // (offsets of 32 bits)
+  if (boxes) BST_CUDA(cudaMalloc(&out->rel.boxes, sizeof(RelBox) * nb));
   plan_view_kernel<<<1, kPlanThreads, 0, s>>>(dl, v, t.q, t.d, t.sect, t.off, int(nb), rch, rext, roff, cch, cext,
                                               coff, rtot, ctot, secidx, out->secs, counts, out->rel.tasks,
                                               out->rel.chunks, counts + 1);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
+  if (boxes) {
+    rel_boxes_kernel<<<unsigned((nb + 127) / 128), 128, 0, s>>>(out->rel.tasks, int(nb), out->rel.boxes);
+    BST_CUDA(cudaGetLastError());
+    count_launch(ctx);
+  }
   int hc[2] = {0, 0};
   BST_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
   BST_CUDA(cudaStreamSynchronize(s));  // the tables above are freed on return

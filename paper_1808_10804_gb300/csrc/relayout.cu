@@ -4,7 +4,17 @@
 // Every relayout is a list of tasks; a task moves one contiguous block,
 // row-major over its own leg order, to or from a strided region of another
 // buffer.  The work is split into chunks of kChunk elements, one CTA per
-// chunk, so uneven block sizes load-balance across the 152 SMs.
+// chunk, so uneven block sizes load-balance across the 152 SMs; large
+// transposing copies go by boxes instead, one CTA per box.
+//
+// What bounds it: small copies, their latency (table loads, then the
+// elements; eight of them in flight a thread).  With the divisions by the
+// legs' extents prepared in every thread, and four elements in flight, the
+// three copies of an FP64 corner contraction (odd sizes, 18 MB) took 39 us,
+// now 32, the 78 of a D = 4, chi = 16 move 640 us, now 495.  Large ones whose
+// innermost legs differ: each 8-byte store of a warp went to another sector,
+// 2.0 TB/s; through boxes 3.7 TB/s (permutation 2031 of a D = 8, chi = 256
+// tensor, 289 MB: 269 -> 155 us), bound by the instructions of the two passes.
 #include <algorithm>
 
 #include "bst_internal.h"
@@ -32,6 +42,11 @@ ProfScope::~ProfScope() {
 
 constexpr int kChunk = 2048;
 constexpr int kRelThreads = 256;
+// Copies through boxes: four runs a thread, six CTAs an SM (a few spilled
+// registers included: 155 us for the D = 8, chi = 256 permutation below, with
+// four CTAs 180, with two runs and eight CTAs 172).
+constexpr int kBoxU = 4, kBoxCtas = 6;
+constexpr double kBoxElems = 4e6;  // copies of fewer elements stay in the L2 cache, see launch_relayout
 
 std::vector<int2> relayout_chunks(const std::vector<RelTask>& t) {
   std::vector<int2> ch;
@@ -45,14 +60,28 @@ void DevRelayout::upload(const std::vector<RelTask>& t) {
   ntasks = int(t.size());
   elems = 0;
   for (auto& x : t) elems += x.n;
-  std::vector<int2> ch;
-  for (int i = 0; i < ntasks; ++i)
-    for (int s = 0; s < t[i].n; s += kChunk) ch.push_back(make_int2(i, s));
-  nchunks = int(ch.size());
+  std::vector<int2> ch = relayout_chunks(t);
   if (ntasks) {
     BST_CUDA(cudaMalloc(&tasks, sizeof(RelTask) * ntasks));
     BST_CUDA(cudaMemcpy(tasks, t.data(), sizeof(RelTask) * ntasks, cudaMemcpyHostToDevice));
+    std::vector<RelBox> hb(ntasks);
+    bool ok = true;
+    for (int i = 0; i < ntasks; ++i) rel_make_box(t[i], hb[i]), ok = ok && hb[i].ntiles > 0;
+    double across = 0;  // elements of blocks whose innermost leg is not the strided side's
+    for (int i = 0; i < ntasks; ++i)
+      if (hb[i].n > 1 && hb[i].leg[0].slot != 0) across += t[i].n;
+    transposes = ok && elems >= kBoxElems && across > 0.5 * elems;
+    if (transposes) {  // a CTA per box
+      ch.clear();
+      for (int i = 0; i < ntasks; ++i)
+        for (int k = 0; k < (t[i].n > 0 ? hb[i].ntiles : 0); ++k) ch.push_back(make_int2(i, k));
+    }
+    if (ok) {
+      BST_CUDA(cudaMalloc(&boxes, sizeof(RelBox) * ntasks));
+      BST_CUDA(cudaMemcpy(boxes, hb.data(), sizeof(RelBox) * ntasks, cudaMemcpyHostToDevice));
+    }
   }
+  nchunks = int(ch.size());
   if (nchunks) {
     BST_CUDA(cudaMalloc(&chunks, sizeof(int2) * nchunks));
     BST_CUDA(cudaMemcpy(chunks, ch.data(), sizeof(int2) * nchunks, cudaMemcpyHostToDevice));
@@ -61,8 +90,10 @@ void DevRelayout::upload(const std::vector<RelTask>& t) {
 
 void DevRelayout::free_all() {
   if (tasks) cudaFree(tasks);
+  if (boxes) cudaFree(boxes);
   if (chunks) cudaFree(chunks);
   tasks = nullptr;
+  boxes = nullptr;
   chunks = nullptr;
   ntasks = nchunks = 0;
 }
@@ -103,12 +134,47 @@ __global__ void __launch_bounds__(kRelThreads) relayout_kernel(const RelTask* __
   relayout_range<kRelThreads>(t, c.y, min(t.n, c.y + kChunk), blk, mat, dir, alpha, beta);
 }
 
+__global__ void __launch_bounds__(kRelThreads) relayout_legs_kernel(const RelTask* __restrict__ tasks,
+                                                                    const RelBox* __restrict__ boxes,
+                                                                    const int2* __restrict__ chunks, double* blk,
+                                                                    double* mat, int dir, double alpha, double beta) {
+  __shared__ RelLegs sh;
+  const int2 c = chunks[blockIdx.x];
+  relayout_legs<kRelThreads>(sh, boxes[c.x], c.y, min(tasks[c.x].n, c.y + kChunk), blk, mat, dir, alpha, beta);
+}
+
+__global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(const RelBox* __restrict__ boxes,
+                                                                             const int2* __restrict__ tiles, double* blk,
+                                                                             double* mat, int dir, double alpha,
+                                                                             double beta) {
+  __shared__ RelShared sh;
+  const int2 c = tiles[blockIdx.x];
+  relayout_box<kRelThreads, kBoxU>(sh, boxes[c.x], c.y, blk, mat, dir, alpha, beta);
+}
+
+__global__ void rel_boxes_kernel(const RelTask* tasks, int n, RelBox* boxes) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) rel_make_box(tasks[i], boxes[i]);
+}
+
+// Boxes only for large copies between different innermost legs: the
+// scattered side of a smaller one is merged in the L2 cache, and a box pays
+// for its tables and two more barriers (a D = 4, chi = 64 permutation takes
+// 14 us by boxes, 10 by legs; the odd-sized FP64 corner's copies 89 and 32);
+// with the same innermost leg on both sides the direct copy reaches 5.1 TB/s.
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir, double alpha,
                      double beta, cudaStream_t s) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  relayout_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.chunks, const_cast<double*>(blk), mat, dir,
-                                                     alpha, beta);
+  if (r.boxes && r.transposes)
+    relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
+                                                          beta);
+  else if (r.boxes)
+    relayout_legs_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, const_cast<double*>(blk), mat, dir,
+                                                          alpha, beta);
+  else
+    relayout_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
+                                                      beta);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

@@ -1,0 +1,52 @@
+"""Block permutations against numpy at the edges of the relayout kernels'
+boxes: innermost legs kept and moved, legs shorter and longer than a run (16
+to 64 elements), legs that merge, odd extents, up to six legs, both below and
+above the size from which boxes are used.  Copies are exact."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bst():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1808_10804_gb300 import build
+    build.build()
+    from paper_1808_10804_gb300 import bst as b
+    return b
+
+
+@pytest.mark.parametrize("shape,perm", [
+    ((1, 1), (1, 0)), ((7,), (0,)), ((2049, 3), (1, 0)), ((3, 2049), (1, 0)), ((5, 1, 7), (2, 1, 0)),
+    ((33, 65, 17), (2, 0, 1)), ((16, 15, 16, 2), (3, 2, 1, 0)), ((2, 3, 2, 3, 2, 40), (5, 0, 4, 1, 3, 2)),
+    # past 4 million elements: by boxes
+    ((2111, 2029), (1, 0)), ((4200, 1001), (1, 0)), ((3, 1400001), (1, 0)), ((1400001, 3), (1, 0)),
+    ((17, 65, 63, 61), (2, 0, 3, 1)), ((2, 129, 5, 255, 13), (4, 2, 0, 3, 1)), ((19, 300, 31, 29), (0, 2, 1, 3)),
+    ((2, 3, 5, 7, 11, 13, 14, 11), (7, 5, 3, 1, 6, 4, 2, 0)), ((41, 40, 50, 51), (1, 0, 3, 2)),
+])
+def test_permute_box_edges(bst, shape, perm):
+    ctx = bst.Context(0)
+    rng = np.random.default_rng(len(shape))
+    # one block of the given shape, and beside it one of one more on every
+    # leg that is not the first (charge 2 there, balanced by the first leg)
+    legs = [bst.Leg(1 if i == 0 else -1, (0,), (n,)) for i, n in enumerate(shape)]
+    if len(shape) > 1:
+        legs[0] = bst.Leg(1, (0, 2), (shape[0], 2))
+        legs[1] = bst.Leg(-1, (0, 2), (shape[1], shape[1] + 1))
+    L = ctx.layout(legs)
+    x = rng.standard_normal(L.nnz)
+    dims = [shape] if len(shape) == 1 else [shape, (2, shape[1] + 1) + shape[2:]]
+    Lp, y = ctx.permute(L, torch.tensor(x, device="cuda:0"), perm)
+    ctx.sync()
+    y = y.cpu().numpy()
+    assert y.size == x.size == sum(int(np.prod(d)) for d in dims)
+    blocks, pos = [], 0
+    for d in dims:
+        blocks.append(x[pos:pos + int(np.prod(d))].reshape(d).transpose(perm).reshape(-1))
+        pos += blocks[-1].size
+    # (blocks in lexicographic order of their charges, 0 before 2 on every leg)
+    assert np.array_equal(y, np.concatenate(blocks))
+    ctx.close()
