@@ -564,10 +564,14 @@ __global__ void oa_update(const SmallProb* __restrict__ probs, const double* __r
   }
 }
 
-// X <- X + XE (in place; XE computed by a GEMM)
-__global__ void add_inplace(double* __restrict__ X, const double* __restrict__ XE, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    X[i] += XE[i];
+// out <- a + t, problem by problem (t computed by a GEMM; a and out may be the
+// same)
+__global__ void add_blocks(const SmallProb* __restrict__ probs, const double* a, const double* __restrict__ t,
+                           double* out) {
+  const SmallProb p = probs[blockIdx.x];
+  const long long n = (long long)p.b * p.b;
+  for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.y * blockDim.x)
+    out[p.in_off + i] = a[p.in_off + i] + t[p.in_off + i];
 }
 
 // Conversions between FP64 and FP32 with a power-of-two scale, built from

@@ -120,7 +120,7 @@ __global__ void jacobi_block_f32(const SmallProb*, const double*, double*, doubl
                                  int*);
 size_t jacobi_block_smem(int b);
 __global__ void oa_update(const SmallProb*, const double*, const double*, double*, double*, double, double, double);
-__global__ void add_inplace(double*, const double*, long long);
+__global__ void add_blocks(const SmallProb*, const double*, const double*, double*);
 __global__ void cholinv_f32(const SmallProb*, const double*, double*, int*, const float*, int, int*);
 struct GramProb {
   int32_t M, b;
@@ -333,6 +333,9 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
   double* T = (double*)ctx->buf(pre + "eig.t", sizeof(double) * smtot, s);
   double* S = (double*)ctx->buf(pre + "eig.s", sizeof(double) * smtot, s);
   double* E = (double*)ctx->buf(pre + "eig.e", sizeof(double) * smtot, s);
+  // (not graded: X and T = H X side by side, see the refinement)
+  double* XC = gr ? nullptr : (double*)ctx->buf(pre + "eig.xc", sizeof(double) * 2 * smtot, s);
+  double* X0 = gr ? X : XC;
   const std::string wsname = pre + "gemm_f64.splitk";
   const char* ws = wsname.c_str();
   std::vector<GemmProb> g_xtx, g_hx, g_s, g_xe;
@@ -380,7 +383,7 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
       BST_CUDA(cudaGetLastError());
       count_launch(ctx);
     }
-    gemm_any(ctx, pre + "oa.xe", prec, g_xe, X1, T, X, s, false, ws);  // X = X1 X2
+    gemm_any(ctx, pre + "oa.xe", prec, g_xe, X1, T, X0, s, false, ws);  // X = X1 X2
   } else if (near_diag) {
     ProfScope ps(ctx, s, "jacobi_f32", jac_flops, 0.0);
     // values below 1e-6 of the largest are not resolved by this FP32 pass
@@ -391,7 +394,7 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
     // there to far below FP64 rounding.  Rotations by less than ~3e-5 are
     // left to the refinement as well (sweeps after the first find most
     // pairs there, and skip their updates).
-    jacobi(dsp, H, X, lam, 10, 1e-5f, 1e-6f, 1e-8f, 1e-10f);
+    jacobi(dsp, H, X0, lam, 10, 1e-5f, 1e-6f, 1e-8f, 1e-10f);
     BST_CUDA(cudaGetLastError());
     count_launch(ctx);
   } else {
@@ -409,7 +412,7 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
       BST_CUDA(cudaGetLastError());
       count_launch(ctx);
     }
-    gemm_any(ctx, pre + "oa.xe", prec, g_xe, X1, T, X, s, false, ws);  // X = X1 X2
+    gemm_any(ctx, pre + "oa.xe", prec, g_xe, X1, T, X0, s, false, ws);  // X = X1 X2
   }
   // three refinement steps: quadratic from the FP32 stage's angles, which
   // for a pair of values closer than ~1e-6 relative are limited by FP32
@@ -417,7 +420,7 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
   // (not graded) X and T = H X side by side in one buffer XC, so that
   // X^T X and X^T T are one launch: X^T [X | T]
   std::vector<GemmProb> g_hx2, g_xs;
-  double *XC = nullptr, *XS = nullptr;
+  double* XS = nullptr;
   if (!gr) {
     for (auto& p : sp) {
       const int b = p.b;
@@ -430,9 +433,7 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
       const int64_t o = p.in_off;
       g_xs.push_back(gp(b, b, b, o, 1, b, smtot + o, 1, b, smtot + o, b, 1));  // X^T T
     }
-    XC = (double*)ctx->buf(pre + "eig.xc", sizeof(double) * 2 * smtot, s);
     XS = (double*)ctx->buf(pre + "eig.xs", sizeof(double) * 2 * smtot, s);
-    BST_CUDA(cudaMemcpyAsync(XC, X, sizeof(double) * smtot, cudaMemcpyDeviceToDevice, s));
   }
   for (int it = 0; it < 3; ++it) {
     const double* xtx = XtX;
@@ -455,13 +456,13 @@ static void small_eig(Ctx* ctx, bst_prec prec, const std::vector<SmallProb>& sp,
     // largest; S is accurate to ~eps sigma_1 (sigma_i + sigma_j)
     oa_update<<<dim3(unsigned(sp.size()), unsigned(slices)), 256, 0, s>>>(dsp, xtx, sm, E, lam, 1e-9,
                                                                           gr ? 1e-12 : 1e-6, gr ? 1e-13 : 0.0);
-    double* Xi = gr ? X : XC;
-    gemm_any(ctx, pre + "oa.xe", prec, g_xe, Xi, E, T, s, false, ws);
-    add_inplace<<<std::max<int64_t>(1, std::min<int64_t>((smtot + 255) / 256, 1216)), 256, 0, s>>>(Xi, T, smtot);
+    gemm_any(ctx, pre + "oa.xe", prec, g_xe, X0, E, T, s, false, ws);
+    // (this call's problems only: the rest of X belongs to a solve on another
+    // stream)
+    add_blocks<<<dim3(unsigned(sp.size()), unsigned(slices)), 256, 0, s>>>(dsp, X0, T, it == 2 ? X : X0);
     BST_CUDA(cudaGetLastError());
     count_launch(ctx, 2);
   }
-  if (!gr) BST_CUDA(cudaMemcpyAsync(X, XC, sizeof(double) * smtot, cudaMemcpyDeviceToDevice, s));
 }
 
 // Sum of squares of each listed block of x (one CTA per block, fixed order).

@@ -82,3 +82,39 @@ def test_projector_spectra(bst, kind, prec):
             assert np.linalg.norm(a @ b - u @ u.T) <= bound
         assert po == p_.size and to == pt_.size
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+def test_solves_side_by_side(bst, prec):
+    """Sectors that are decomposed directly (on the second stream) beside
+    iterated ones, several matrices through one context: neither solve
+    touches the other's vectors, nor takes up what an earlier call left."""
+    rows = (60, 128, 260, 33)
+    ctx = bst.Context(0)
+    leg = lambda f: bst.Leg(f, (0, 1, 2, 3), rows)  # noqa: E731
+    Rt, Rb = ctx.layout([leg(1), leg(-1)]), ctx.layout([leg(-1), leg(1)])
+    flat = lambda xs: torch.tensor(np.concatenate([x.reshape(-1) for x in xs]), device="cuda:0")  # noqa: E731
+    eye = flat([np.eye(r) for r in rows])
+    for seed in range(6):
+        rng = np.random.default_rng(seed)
+        N = []
+        for s, r in enumerate(rows):
+            u, v = (np.linalg.qr(rng.standard_normal((r, r)))[0] for _ in range(2))
+            amp = rng.uniform(0.5, 1.0)
+            j = np.arange(r)
+            N.append((u * (amp * np.where(j < 6, 0.95 ** j, 0.2 * 0.97 ** j))) @ v.T)
+        svd = [np.linalg.svd(x) for x in N]
+        lam = np.sort(np.concatenate([x[1] for x in svd]))[::-1] ** 2
+        # (24 kept values, six a sector, above the gap)
+        bound = 100 * TOL[prec] * np.sqrt(CHI) / ((lam[CHI - 1] - lam[CHI]) / lam[0])
+        P, p, Pt, pt, sv, kept = ctx.svd_projector(Rt, eye, Rb, flat(N), 1, CHI, 1e-14, 1, prec=prec)
+        ctx.sync()
+        assert kept == CHI and tuple(P.legs[1].degs) == (6, 6, 6, 6)
+        assert np.abs(np.sort(np.square(sv))[::-1] - lam[:CHI]).max() <= bound * lam[0]
+        p_, pt_, pos = p.cpu().numpy(), pt.cpu().numpy(), 0
+        for s, r in enumerate(rows):
+            a, b = p_[pos:pos + 6 * r].reshape(r, 6), pt_[pos:pos + 6 * r].reshape(6, r)
+            pos += 6 * r
+            u = svd[s][0][:, :6]
+            assert np.linalg.norm(a @ b - u @ u.T) <= bound
+    ctx.close()
