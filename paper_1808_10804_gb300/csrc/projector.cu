@@ -694,6 +694,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   // sector in hl's layout (Ritz values or estimates, in any order).  Empty
   // when none fits: a spectrum so steep that the growth bound puts alpha
   // above a kept value (plain steps, which factor after every half).
+  double gain = 1.0;  // growth that the plan gives every kept value
   auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod) {
     std::vector<std::pair<double, int>> all;
     for (size_t i = 0; i < secs.size(); ++i)
@@ -730,11 +731,16 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
           f.on.push_back({x.q_off, int64_t(x.N) * x.b, 0.0});
           continue;
         }
-        // (an interval reaching into the block lets the polynomial's zeros
-        // wipe out columns there: degree 2 has few enough for the mixed
-        // tolerance)
-        if (0.8 * low < top / span && (m > 2 || prec == BST_FP64)) return 0.0;
         const double alpha = std::max(0.8 * low, top / span);
+        // an interval reaching into the block lets the polynomial's zeros
+        // wipe out columns there, and the rest of those columns drown in the
+        // growth of the others: degree 2 with few of them does for the mixed
+        // tolerance
+        if (0.8 * low < top / span) {
+          int inside = 0;
+          for (int j = 0; j < x.c; ++j) inside += v[x.val_off + j] < alpha;
+          if (m > 2 || prec == BST_FP64 || 8 * inside > x.c) return 0.0;
+        }
         if (lowest[i] < 1.05 * alpha) return 0.0;
         grow = std::min(grow, std::cosh(m * std::acosh(2.0 * lowest[i] / alpha - 1.0)));
         f.on.push_back({x.q_off, int64_t(x.N) * x.b, alpha});
@@ -754,7 +760,9 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
         const double nm = std::ceil(rest / std::log(g));
         if (nm * (m + 3.0) < cost) cost = nm * (m + 3.0), n = nm, best = f;  // (a factorisation costs ~3 products)
       }
-    for (int used = 2; n > 0 && used + best.m <= nprod; n -= 1, used += best.m) out.push_back(best);
+    gain = g2;
+    const double gb = n > 0 ? of_degree(best.m, f) : 1.0;
+    for (int used = 2; n > 0 && used + best.m <= nprod; n -= 1, used += best.m) out.push_back(best), gain *= gb;
     out.push_back(last);
     return out;
   };
@@ -772,9 +780,10 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     }
     std::swap(Q, Y);  // the polished block is in Y
   };
-  if (!sp_it.empty()) {
+  std::vector<long long> rng;
+  auto random_start = [&]() {
     // deterministic random start (a seed per sector, one launch)
-    std::vector<long long> rng;
+    rng.clear();
     int64_t nmax = 0;
     for (auto& x : secs)
       if (!x.direct) {
@@ -789,7 +798,8 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
         Q, drng);
     BST_CUDA(cudaGetLastError());
     count_launch(ctx);
-  }
+  };
+  if (!sp_it.empty()) random_start();
   // Rounds of `iters` iterations, each closed by a Rayleigh-Ritz step.  A
   // round is accepted when every Ritz pair that the truncation would keep
   // (plus a few below it) has a residual ||N^T N v - lambda v|| at most
@@ -1067,6 +1077,11 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     // interval did not fit the spectrum, or its floor is reached; plain steps
     // from here)
     if (round > 0 && !fplan.empty() && !(worst < 0.5 * prev_worst)) may_filter = false;
+    // (a first round that is nowhere near what its filters promised, as over
+    // a spectrum whose estimates were of no use: most of its block's columns
+    // are lost, and plain steps start afresh)
+    const bool lost = round == 0 && !fplan.empty() && !(worst <= 1e-4) && !(worst * gain <= 1e4);
+    if (lost) may_filter = false;
     fplan.clear();
     if (!ok && may_filter && worst > 0 && std::isfinite(worst))
       fplan = plan_filters(hl, worst / (0.02 * tol), 6, std::min(6 * iters, max_total - total));
@@ -1083,8 +1098,9 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     steps = next == 0 ? 0 : std::min(next, std::max(1, max_total - total));
     prev_worst = worst;
     // resume from the Ritz vectors
+    if (lost) random_start();
     for (auto& x : secs)
-      if (!x.direct)
+      if (!x.direct && !lost)
         BST_CUDA(cudaMemcpyAsync(Q + x.q_off, dV + x.v_off, sizeof(double) * int64_t(x.N) * x.b,
                                  cudaMemcpyDeviceToDevice, s));
   }
