@@ -1080,8 +1080,13 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     // (a first round that is nowhere near what its filters promised, as over
     // a spectrum whose estimates were of no use: most of its block's columns
     // are lost, and plain steps start afresh)
-    const bool lost = round == 0 && !fplan.empty() && !(worst <= 1e-4) && !(worst * gain <= 1e4);
-    if (lost) may_filter = false;
+    // A residual above lambda_max: the refinement of the Ritz vectors
+    // diverged (a cluster of many values ~1e-9 apart), they are no basis to
+    // go on from; plain steps resume from the block before it, or from a new
+    // one if it had been filtered.
+    const bool diverged = !(worst <= 1.0);
+    const bool lost = !fplan.empty() && (diverged || (round == 0 && !(worst <= 1e-4) && !(worst * gain <= 1e4)));
+    if (lost || diverged) may_filter = false;
     fplan.clear();
     if (!ok && may_filter && worst > 0 && std::isfinite(worst))
       fplan = plan_filters(hl, worst / (0.02 * tol), 6, std::min(6 * iters, max_total - total));
@@ -1100,7 +1105,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     // resume from the Ritz vectors
     if (lost) random_start();
     for (auto& x : secs)
-      if (!x.direct && !lost)
+      if (!x.direct && !lost && !diverged)
         BST_CUDA(cudaMemcpyAsync(Q + x.q_off, dV + x.v_off, sizeof(double) * int64_t(x.N) * x.b,
                                  cudaMemcpyDeviceToDevice, s));
   }
