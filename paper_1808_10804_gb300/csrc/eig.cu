@@ -224,9 +224,13 @@ __global__ void __launch_bounds__(1024) jacobi_eig_f32(const SmallProb* __restri
 // with the indices in blocks of 16.  A sweep is nb - 1 rounds (nb blocks,
 // round-robin pairing of blocks); in a round every block pair P = I u J is
 // one 32 x 32 subproblem: a warp runs one cyclic sweep of 2 x 2 rotations
-// on A[P, P] (in its own shared buffer), accumulating Q^T in registers
-// (lane i holds row i), then all threads apply A[P, :] <- Q^T A[P, :],
-// A[:, P] <- A[:, P] Q and V[:, P] <- V[:, P] Q.  Per sweep this moves
+// on A[P, P], both it and Q^T in registers (lane i holds row i), then all
+// threads apply A[P, :] <- Q^T A[P, :], A[:, P] <- A[:, P] Q and
+// V[:, P] <- V[:, P] Q.  The sweep's 31 steps are a serial chain of one warp,
+// and shared memory was its bound (224 accesses a step): the rows of a pair
+// are exchanged by shuffles, the columns by keeping them in tournament order
+// in the registers (a step moves 31 of them on by one place, which costs
+// moves instead of accesses), so 64 shuffles and 9 accesses are left.  Per sweep this moves
 // the matrix through shared memory nb - 1 times instead of b - 1 (the
 // scalar kernel's rounds are bound by those passes), at the same
 // arithmetic.  bp = b rounded up to 32 (zero padding, decoupled).
@@ -325,28 +329,41 @@ __global__ void __launch_bounds__(kBjThreads) jacobi_block_f32(const SmallProb* 
         // index map of the pair: local 0..15 -> block bi, 16..31 -> block bj
         float* S = Sub + warp * 32 * kQt;
         const int gl = (lane < 16 ? bi * 16 + lane : bj * 16 + lane - 16);
-        for (int k = 0; k < 32; ++k) {
-          const int gk = (k < 16 ? bi * 16 + k : bj * 16 + k - 16);
-          S[lane * 33 + k] = A[gl * ld + gk];
+        // Lane i holds row i of S, the columns by their place in the
+        // tournament: in step rr the pairs are (T[k], B[k]), T[0] column 31,
+        // T[k] column (rr + k) mod 31, B[k] column (rr - k) mod 31
+        auto at = [&](int k) { return A[gl * ld + (k < 16 ? bi * 16 + k : bj * 16 + k - 16)]; };
+        float T[16], B[16], qt[32];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          T[k] = at(k == 0 ? 31 : k);
+          B[k] = at(k == 0 ? 0 : 31 - k);
         }
-        float qt[32];
+        float diag = at(lane);
 #pragma unroll
         for (int k = 0; k < 32; ++k) qt[k] = (k == lane) ? 1.f : 0.f;
-        __syncwarp();
         // one cyclic sweep: 31 rounds of 16 disjoint rotations
         bool any_rot = false;
+        int d = lane;  // (lane - rr) mod 31
+#pragma unroll 1
         for (int rr = 0; rr < 31; ++rr) {
-          // lane's partner in round rr (index 31 fixed, others rotate)
-          int mate;
-          if (lane == 31) mate = rr;
-          else if (lane == rr) mate = 31;
-          else {
-            mate = 2 * rr - lane;
-            mate %= 31;
-            if (mate < 0) mate += 31;
-          }
+          // this lane's place: T[k] or B[k], and its partner in the other
+          const bool top = lane == 31 || (d >= 1 && d <= 15);
+          const int k = lane == 31 || d == 0 ? 0 : d <= 15 ? d : 31 - d;
+          int mate = top ? rr - k : rr + k;
+          mate = lane == 31 ? rr : d == 0 ? 31 : mate < 0 ? mate + 31 : mate >= 31 ? mate - 31 : mate;
+          // S[lane][mate], out of the other half's registers
+          float x[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) x[i] = top ? B[i] : T[i];
+#pragma unroll
+          for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+            for (int i = 0; i < w; ++i) x[i] = (k & w) ? x[i + w] : x[i];
           const int p = min(lane, mate), q = max(lane, mate);
-          const float apq = S[p * 33 + q], app = S[p * 33 + p], aqq = S[q * 33 + q];
+          // (both lanes of a pair from the same entry)
+          const float apq = __shfl_sync(0xffffffffu, x[0], p);
+          const float app = __shfl_sync(0xffffffffu, diag, p), aqq = __shfl_sync(0xffffffffu, diag, q);
           float c = 1.f, sn = 0.f;
           const float dd = fmaxf(fabsf(app), kTau) * fmaxf(fabsf(aqq), kTau);
           // (skip_ang > 0: rotations whose angle test 0.1 a^2 / gap^2 is
@@ -354,55 +371,54 @@ __global__ void __launch_bounds__(kBjThreads) jacobi_block_f32(const SmallProb* 
           const float gq = aqq - app;
           const bool rot = fabsf(apq) > 1e-30f && apq * apq > 1e-15f * dd &&
                            !(skip_ang > 0.f && 0.1f * (apq * apq) <= skip_ang * fmaxf(gq * gq, 1e-37f));
+          const bool lo = lane == p;
           if (rot) {
             const float tau = gq / (2.f * apq);
             const float t = copysignf(1.f, tau) / (fabsf(tau) + sqrtf(1.f + tau * tau));
             c = rsqrtf(1.f + t * t);
             sn = t * c;
+            diag += lo ? -t * apq : t * apq;
           }
           // a step without any rotation leaves S and Q^T as they are
-          if (!__any_sync(0xffffffffu, rot)) continue;
-          any_rot = true;
-          // row of this lane: S'[lane] = c S[lane] -/+ s S[mate], then the
-          // columns likewise (S' is no longer symmetric); in halves of 16
-          // (reads of a half before anyone writes it)
-          const bool lo = lane == p;
+          if (__any_sync(0xffffffffu, rot)) {
+            any_rot = true;
+            const float m = lo ? -sn : sn;  // row <- c row + m partner's row
+            if (top) *reinterpret_cast<float2*>(S + 2 * k) = make_float2(c, m);
+            __syncwarp();
 #pragma unroll
-          for (int h = 0; h < 32; h += 16) {
-            float rl[16], rm[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              rl[k] = S[lane * 33 + h + k];
-              rm[k] = S[mate * 33 + h + k];
+            for (int i = 0; i < 16; ++i) {
+              const float u = __shfl_sync(0xffffffffu, T[i], mate), v = __shfl_sync(0xffffffffu, B[i], mate);
+              T[i] = fmaf(m, u, c * T[i]);
+              B[i] = fmaf(m, v, c * B[i]);
             }
-            __syncwarp();
+            // the columns: T[i] <- c T[i] + m B[i], B[i] <- c B[i] - m T[i]
 #pragma unroll
-            for (int k = 0; k < 16; ++k) S[lane * 33 + h + k] = lo ? (c * rl[k] - sn * rm[k]) : (sn * rm[k] + c * rl[k]);
-            __syncwarp();
-          }
-#pragma unroll
-          for (int h = 0; h < 32; h += 16) {
-            float rl[16], rm[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              rl[k] = S[(h + k) * 33 + lane];
-              rm[k] = S[(h + k) * 33 + mate];
+            for (int i = 0; i < 16; i += 2) {
+              const float4 g = *reinterpret_cast<const float4*>(S + 2 * i);
+              const float t0 = T[i], t1 = T[i + 1];
+              T[i] = fmaf(g.y, B[i], g.x * t0);
+              B[i] = fmaf(-g.y, t0, g.x * B[i]);
+              T[i + 1] = fmaf(g.w, B[i + 1], g.z * t1);
+              B[i + 1] = fmaf(-g.w, t1, g.z * B[i + 1]);
             }
-            __syncwarp();
+            // Q^T rows: row lane of Q^T = column lane of Q
 #pragma unroll
-            for (int k = 0; k < 16; ++k) S[(h + k) * 33 + lane] = lo ? (c * rl[k] - sn * rm[k]) : (sn * rm[k] + c * rl[k]);
+            for (int i = 0; i < 32; ++i) qt[i] = fmaf(m, __shfl_sync(0xffffffffu, qt[i], mate), c * qt[i]);
             __syncwarp();
           }
-          // Q^T rows: row lane of Q^T = column lane of Q
+          // the next step's places
+          const float t1 = T[1];
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const float m = __shfl_sync(0xffffffffu, qt[k], mate);
-            qt[k] = lo ? (c * qt[k] - sn * m) : (sn * m + c * qt[k]);
-          }
+          for (int i = 1; i < 15; ++i) T[i] = T[i + 1];
+          T[15] = B[15];
+#pragma unroll
+          for (int i = 15; i > 0; --i) B[i] = B[i - 1];
+          B[0] = t1;
+          d = d == 0 ? 30 : d - 1;
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) S[lane * kQt + k] = qt[k];
+        for (int i = 0; i < 32; ++i) S[lane * kQt + i] = qt[i];
         if (lane == 0) moved[warp] = int(any_rot);
       }
       __syncthreads();
