@@ -230,7 +230,12 @@ __global__ void __launch_bounds__(1024) jacobi_eig_f32(const SmallProb* __restri
 // and shared memory was its bound (224 accesses a step): the rows of a pair
 // are exchanged by shuffles, the columns by keeping them in tournament order
 // in the registers (a step moves 31 of them on by one place, which costs
-// moves instead of accesses), so 64 shuffles and 9 accesses are left.  Per sweep this moves
+// moves instead of accesses), so 64 shuffles and 9 accesses are left.
+// The updates are bound by their FP32 arithmetic (1024 multiply-adds a task,
+// 512 threads): A's blocks are updated once for both triangles, and V's rows
+// fill up the threads of the two passes (three rounds of tasks for b = 160
+// instead of six).  Two direct FP64 solves of up to 133 values: 3.34 ms with
+// the sweep in shared memory, 2.69 in registers, 2.46 with half the updates.  Per sweep this moves
 // the matrix through shared memory nb - 1 times instead of b - 1 (the
 // scalar kernel's rounds are bound by those passes), at the same
 // arithmetic.  bp = b rounded up to 32 (zero padding, decoupled).
@@ -420,26 +425,36 @@ __global__ void __launch_bounds__(kBjThreads) jacobi_block_f32(const SmallProb* 
 #pragma unroll
         for (int i = 0; i < 32; ++i) S[lane * kQt + i] = qt[i];
         if (lane == 0) moved[warp] = int(any_rot);
+        // (after 31 steps the columns are back at their first places)
+        if (any_rot) {
+          auto put = [&](int k, float x) { A[gl * ld + (k < 16 ? bi * 16 + k : bj * 16 + k - 16)] = x; };
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            put(k == 0 ? 31 : k, T[k]);
+            put(k == 0 ? 0 : 31 - k, B[k]);
+          }
+        }
       }
       __syncthreads();
-      // ---- A[P, :] <- Q^T A[P, :]: task (pair, column) ----
-      for (int t = tid; t < npair * bp; t += nt) {
-        const int pp = t / bp, col = t - pp * bp;
-        int bi, bj;
-        if (pp == 0) {
-          bi = nb - 1;
-          bj = r;
-        } else {
-          bi = r + pp;
-          if (bi >= nb - 1) bi -= nb - 1;
-          bj = r - pp;
-          if (bj < 0) bj += nb - 1;
-        }
-        if (!moved[pp]) continue;  // Q = I: A[P, :] unchanged
-        const float* QT = Sub + pp * 32 * kQt;
-        float a[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) a[k] = A[(k < 16 ? bi * 16 + k : bj * 16 + k - 16) * ld + col];
+      // A is symmetric: blocks A[P, P'] of different pairs once, their mirror
+      // images written along (A[P, P] came out of the sweep).  Threads take a
+      // column of A[P, P'] for A[P, P'] <- Q_P^T A[P, P'], after a barrier a
+      // row for A[P, P'] <- A[P, P'] Q_P', and rows of V[:, P] <- V[:, P] Q_P
+      // fill up the threads of either pass.
+      auto index = [&](int pp, int k) {
+        int bi = r + pp, bj = r - pp;
+        if (pp == 0) bi = nb - 1;
+        else if (bi >= nb - 1) bi -= nb - 1;
+        if (bj < 0) bj += nb - 1;
+        return k < 16 ? bi * 16 + k : bj * 16 + k - 16;
+      };
+      auto pairs = [&](int u, int& p1, int& p2) {  // the u-th p1 < p2
+        p1 = 0;
+        while (u >= npair - 1 - p1) u -= npair - 1 - p1++;
+        p2 = p1 + 1 + u;
+      };
+      // out_i = sum_k QT[i][k] a_k
+      auto apply = [&](const float* QT, const float(&a)[32], auto&& put) {
 #pragma unroll 4
         for (int i = 0; i < 32; ++i) {
           float acc0 = 0.f, acc1 = 0.f;
@@ -452,44 +467,61 @@ __global__ void __launch_bounds__(kBjThreads) jacobi_block_f32(const SmallProb* 
             acc0 = fmaf(q.z, a[k + 2], acc0);
             acc1 = fmaf(q.w, a[k + 3], acc1);
           }
-          A[(i < 16 ? bi * 16 + i : bj * 16 + i - 16) * ld + col] = acc0 + acc1;
+          put(i, acc0 + acc1);
         }
-      }
-      __syncthreads();
-      // ---- A[:, P] <- A[:, P] Q and V[:, P] <- V[:, P] Q: task (matrix, pair, row) ----
-      for (int t = tid; t < 2 * npair * bp; t += nt) {
-        const int which = t / (npair * bp);
-        const int rem = t - which * npair * bp;
-        const int pp = rem / bp, row = rem - pp * bp;
-        int bi, bj;
-        if (pp == 0) {
-          bi = nb - 1;
-          bj = r;
-        } else {
-          bi = r + pp;
-          if (bi >= nb - 1) bi -= nb - 1;
-          bj = r - pp;
-          if (bj < 0) bj += nb - 1;
+      };
+      auto v_row = [&](int t) {  // task t of V
+        const int pp = t / bp, row = t - pp * bp;
+        if (!moved[pp]) return;  // Q = I
+        float* Vr = V + row * ld;
+        float a[32];
+        const int i0 = index(pp, 0), i1 = index(pp, 16);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) a[k] = Vr[k < 16 ? i0 + k : i1 + k - 16];
+        apply(Sub + pp * 32 * kQt, a, [&](int i, float x) { Vr[i < 16 ? i0 + i : i1 + i - 16] = x; });
+      };
+      const int na = npair * (npair - 1) / 2 * 32, nv = npair * bp;
+      const int v1 = min(nv, max(0, (na + nv) / nt * nt - na));  // rows of V in the first pass
+      for (int t = tid; t < na + v1; t += nt) {
+        if (t >= na) {
+          v_row(t - na);
+          continue;
         }
-        if (!moved[pp]) continue;  // Q = I
-        float* M = which ? V : A;
-        const float* QT = Sub + pp * 32 * kQt;
+        int p1, p2;
+        pairs(t >> 5, p1, p2);
+        if (!moved[p1]) continue;
+        float* Ac = A + index(p2, lane);
+        const int i0 = index(p1, 0), i1 = index(p1, 16);
         float a[32];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) a[k] = M[row * ld + (k < 16 ? bi * 16 + k : bj * 16 + k - 16)];
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) {
-          float acc0 = 0.f, acc1 = 0.f;
-          const float4* q4 = reinterpret_cast<const float4*>(QT + j * kQt);
+        for (int k = 0; k < 32; ++k) a[k] = Ac[(k < 16 ? i0 + k : i1 + k - 16) * ld];
+        apply(Sub + p1 * 32 * kQt, a, [&](int i, float x) { Ac[(i < 16 ? i0 + i : i1 + i - 16) * ld] = x; });
+      }
+      __syncthreads();
+      for (int t = tid; t < na + nv - v1; t += nt) {
+        if (t >= na) {
+          v_row(t - na + v1);
+          continue;
+        }
+        int p1, p2;
+        pairs(t >> 5, p1, p2);
+        if (!moved[p1] && !moved[p2]) continue;
+        const int row = index(p1, lane);
+        float* Ar = A + row * ld;
+        float* Am = A + row;
+        const int i0 = index(p2, 0), i1 = index(p2, 16);
+        float a[32];
 #pragma unroll
-          for (int k = 0; k < 32; k += 4) {
-            const float4 q = q4[k >> 2];
-            acc0 = fmaf(a[k], q.x, acc0);
-            acc1 = fmaf(a[k + 1], q.y, acc1);
-            acc0 = fmaf(a[k + 2], q.z, acc0);
-            acc1 = fmaf(a[k + 3], q.w, acc1);
-          }
-          M[row * ld + (j < 16 ? bi * 16 + j : bj * 16 + j - 16)] = acc0 + acc1;
+        for (int k = 0; k < 32; ++k) a[k] = Ar[k < 16 ? i0 + k : i1 + k - 16];
+        if (moved[p2]) {
+          apply(Sub + p2 * 32 * kQt, a, [&](int i, float x) {
+            const int j = i < 16 ? i0 + i : i1 + i - 16;
+            Ar[j] = x;
+            Am[j * ld] = x;
+          });
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) Am[(i < 16 ? i0 + i : i1 + i - 16) * ld] = a[i];
         }
       }
       __syncthreads();
