@@ -295,12 +295,12 @@ int64_t plan_check(Ctx* ctx, Layout* A, Layout* B, const std::vector<int>& la, c
 // relayout.cu
 std::vector<int2> relayout_chunks(const std::vector<RelTask>& t);  // chunk table of a task list
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir,
-                     double alpha, double beta, cudaStream_t s);
+                     double alpha, double beta, cudaStream_t s, int order = 0);
 
 // gemm_f64.cu
 DevGemm* get_dev_gemm(Ctx* ctx, const std::string& key, const std::vector<GemmProb>& probs);
 void launch_gemm_f64(Ctx* ctx, const DevGemm& g, const double* A, const double* B, double* C,
-                     cudaStream_t s);
+                     cudaStream_t s, bool behind = false);
 // the same product with K split into ksplit slices reduced in a fixed order
 // (more CTAs for small, deep products)
 // C[prob] = sum over the ksplit slices of W (slice stride g.wtot, problem

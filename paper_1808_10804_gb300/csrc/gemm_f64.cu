@@ -6,6 +6,7 @@
 #include <algorithm>
 
 #include "bst_internal.h"
+#include "relayout_dev.cuh"
 
 namespace bst {
 
@@ -83,23 +84,47 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 }
 
 // One 64x64 output tile of problem p over the K range [kb, ke), written to
-// out[m * om + n * on].  128 threads = 4 warps in a 2x2 arrangement, each warp
-// a 32x32 sub-tile made of 4x4 DMMA tiles of 8x8.  The operand tiles are
-// double-buffered in shared memory: the next K block's loads are in flight
-// (in registers) while the current block is multiplied.
+// out[m * om + n * on].  128 threads = 4 warps, up to 4x4 DMMA tiles of 8x8
+// each.  The operand tiles are double-buffered in shared memory: the next K
+// block's loads are in flight (in registers) while the current block is
+// multiplied.
+//
+// What bounds it: the DMMA units, one a scheduler (an 8x8x4 product takes one
+// about 570 cycles), so a product is issued only where it counts, and the
+// 8x8 tiles are dealt to the warps one by one:
+//   * none past M or N (an odd-sized FP64 corner, 0.33 GFLOP: 594 -> 428 us, with
+//     two CTAs an SM so that nothing spills: three took 512);
+//   * of a Gram matrix (both operands the same) only those on and above its
+//     diagonal; the sums below are the same products in the same order, so
+//     they are mirrored.
 constexpr int kLd = (kF64TileM * kBK) / 128;  // elements of a 64 x 16 tile per thread
 __device__ __forceinline__ void f64_tile(const GemmProb& p, int m0, int n0, int kb, int ke,
                                          const double* __restrict__ A, const double* __restrict__ B,
                                          double* __restrict__ out, long long om, long long on,
-                                         double (*sA)[kBK][kF64TileM + kPad], double (*sB)[kBK][kF64TileN + kPad]) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+                                         double (*sA)[kBK][kF64TileM + kPad], double (*sB)[kBK][kF64TileN + kPad],
+                                         int turn) {
+  const int tid = threadIdx.x, lane = tid & 31, part = ((tid >> 5) + turn) & 3;
   const int g = lane >> 2, tg = lane & 3;
-  double acc[4][4][2];
+  const bool sym = A == B && p.a_off == p.b_off && p.M == p.N && p.a_m == p.b_n && p.a_k == p.b_k;
+  if (sym && m0 > n0) return;  // (uniform) below the diagonal
+  // this warp's 8x8 tiles: every fourth of the tile's, row by row (in a Gram
+  // matrix's diagonal tile the columns from the row's own on)
+  const int r8 = min(8, (p.M - m0 + 7) >> 3), c8 = min(8, (p.N - n0 + 7) >> 3);
+  const bool tri = sym && m0 == n0;
+  const int total = tri ? r8 * (r8 + 1) / 2 : r8 * c8, cnt = (total - part + 3) >> 2;
+  int at[16];  // row and column of the t-th (in 8s: row << 8 | column)
+  {
+    int i = 0, j = part;  // (counted in a row that starts at column 0, then moved)
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int t = 0; t < 16; ++t) {
+      while (i < r8 && j >= c8) ++i, j -= c8 - (tri ? i : 0);
+      at[t] = i << 8 | j;
+      j += 4;
+    }
+  }
+  double acc[16][2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+  for (int t = 0; t < 16; ++t) acc[t][0] = acc[t][1] = 0.0;
   const double* Ap = A + p.a_off;
   const double* Bp = B + p.b_off;
   double ra[kLd], rb[kLd];
@@ -129,47 +154,57 @@ __device__ __forceinline__ void f64_tile(const GemmProb& p, int m0, int n0, int 
 #pragma unroll
     for (int kk = 0; kk < kBK; kk += 4) {
       if (kk >= kn) break;
-      double af[4], bf[4];
+      const double* a = &sA[buf][kk + tg][g];
+      const double* b = &sB[buf][kk + tg][g];
+      if (cnt == 16) {  // (without a branch per tile the loads run ahead)
+        double af[16], bf[16];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) af[i] = sA[buf][kk + tg][wm + i * 8 + g];
+        for (int t = 0; t < 16; ++t) af[t] = a[(at[t] >> 8) * 8], bf[t] = b[(at[t] & 255) * 8];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bf[j] = sB[buf][kk + tg][wn + j * 8 + g];
+        for (int t = 0; t < 16; ++t) dmma(acc[t][0], acc[t][1], af[t], bf[t]);
+      } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dmma(acc[i][j][0], acc[i][j][1], af[i], bf[j]);
+        for (int t = 0; t < 16; ++t) {
+          if (t >= cnt) break;
+          dmma(acc[t][0], acc[t][1], a[(at[t] >> 8) * 8], b[(at[t] & 255) * 8]);
+        }
+      }
     }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int t = 0; t < 16; ++t) {
+    if (t >= cnt) break;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int gm = m0 + wm + i * 8 + g;
-        const int gn = n0 + wn + j * 8 + tg * 2 + h;
-        if (gm < p.M && gn < p.N) out[(long long)gm * om + (long long)gn * on] = acc[i][j][h];
-      }
+    for (int h = 0; h < 2; ++h) {
+      const int gm = m0 + (at[t] >> 8) * 8 + g;
+      const int gn = n0 + (at[t] & 255) * 8 + tg * 2 + h;
+      if (gm >= p.M || gn >= p.N) continue;
+      out[(long long)gm * om + (long long)gn * on] = acc[t][h];
+      if (sym && (at[t] >> 8) * 8 + m0 < (at[t] & 255) * 8 + n0) out[(long long)gn * om + (long long)gm * on] = acc[t][h];
+    }
+  }
 }
 
-__global__ void __launch_bounds__(128, 3) gemm_f64_kernel(const GemmProb* __restrict__ probs,
+__global__ void __launch_bounds__(128, 2) gemm_f64_kernel(const GemmProb* __restrict__ probs,
                                                        const int32_t* __restrict__ tile_prob,
                                                        const int32_t* __restrict__ tile_idx,
                                                        const double* __restrict__ A,
                                                        const double* __restrict__ B, double* __restrict__ C) {
   __shared__ double sA[2][kBK][kF64TileM + kPad];
   __shared__ double sB[2][kBK][kF64TileN + kPad];
+  grid_trigger();
   const GemmProb p = probs[tile_prob[blockIdx.x]];
   const int nt = (p.N + kF64TileN - 1) / kF64TileN;
   const int m0 = (tile_idx[blockIdx.x] / nt) * kF64TileM;
   const int n0 = (tile_idx[blockIdx.x] % nt) * kF64TileN;
-  f64_tile(p, m0, n0, 0, p.K, A, B, C + p.c_off, p.c_m, p.c_n, sA, sB);
+  grid_wait();
+  f64_tile(p, m0, n0, 0, p.K, A, B, C + p.c_off, p.c_m, p.c_n, sA, sB, int(blockIdx.x));
 }
 
 // Split-K: CTA (tile, s) computes the partial product over the s-th K slice
 // (slices of a multiple of 16) into W[s][problem][m][n]; the reduction adds
 // the slices in a fixed order (deterministic result).
-__global__ void __launch_bounds__(128, 3) gemm_f64_splitk_kernel(const GemmProb* __restrict__ probs,
+__global__ void __launch_bounds__(128, 2) gemm_f64_splitk_kernel(const GemmProb* __restrict__ probs,
                                                               const int32_t* __restrict__ tile_prob,
                                                               const int32_t* __restrict__ tile_idx,
                                                               const double* __restrict__ A,
@@ -185,7 +220,8 @@ __global__ void __launch_bounds__(128, 3) gemm_f64_splitk_kernel(const GemmProb*
   const int n0 = (tile_idx[blockIdx.x] % nt) * kF64TileN;
   const int kc = ((p.K + ksplit - 1) / ksplit + kBK - 1) / kBK * kBK;
   const int kb = min(p.K, int(blockIdx.y) * kc), ke = min(p.K, kb + kc);
-  f64_tile(p, m0, n0, kb, ke, A, B, W + blockIdx.y * wtot + w_off[pi], p.N, 1, sA, sB);
+  f64_tile(p, m0, n0, kb, ke, A, B, W + blockIdx.y * wtot + w_off[pi], p.N, 1, sA, sB,
+           int(blockIdx.x + blockIdx.y));
 }
 
 __global__ void gemm_f64_reduce_kernel(const GemmProb* __restrict__ probs, const double* __restrict__ W,
@@ -236,10 +272,12 @@ void launch_ksplit_reduce(Ctx* ctx, const DevGemm& g, const double* W, int kspli
   count_launch(ctx);
 }
 
-void launch_gemm_f64(Ctx* ctx, const DevGemm& g, const double* A, const double* B, double* C, cudaStream_t s) {
+void launch_gemm_f64(Ctx* ctx, const DevGemm& g, const double* A, const double* B, double* C, cudaStream_t s,
+                     bool behind) {
   if (g.ntiles == 0) return;
   ProfScope ps(ctx, s, "gemm_f64", g.flops, 0.0);
-  gemm_f64_kernel<<<g.ntiles, 128, 0, s>>>(g.probs, g.tile_prob, g.tile_idx, A, B, C);
+  launch_behind(behind, gemm_f64_kernel, dim3(unsigned(g.ntiles)), 128, 0, s, (const GemmProb*)g.probs,
+                (const int32_t*)g.tile_prob, (const int32_t*)g.tile_idx, A, B, C);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

@@ -223,13 +223,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "r"(taddr));
 }
 
-// A grid launched behind another with programmatic serialisation may start
-// when every block of the first has called grid_trigger (or left), and must
-// call grid_wait, which returns when the first has finished and its writes
-// are visible, before it touches what that grid reads or writes.
-__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -1782,18 +1775,8 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
   const int* eB = b_from_a ? P->eA : P->eB;
   auto launch = [&](auto kern, size_t smem) {
     // (behind the split or pack, whose last blocks its prologue overlaps)
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(oz::kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    BST_CUDA(cudaLaunchKernelEx(&cfg, kern, P->mapA, mB, (const oz::Prob*)P->d_probs, (const oz::Tile*)P->d_tiles,
-                                P->ntiles, (const int*)P->eA, eB, C, sc, ctx->d_err, spin));
+    launch_behind(true, kern, dim3(unsigned(grid)), oz::kThreads, smem, s, P->mapA, mB, (const oz::Prob*)P->d_probs,
+                  (const oz::Tile*)P->d_tiles, P->ntiles, (const int*)P->eA, eB, C, sc, ctx->d_err, spin);
   };
   if (P->S == 5 && P->TN == 64) {
     set_kernel_attrs<5, 64>();

@@ -137,10 +137,15 @@ __global__ void __launch_bounds__(kRelThreads) relayout_kernel(const RelTask* __
 __global__ void __launch_bounds__(kRelThreads) relayout_legs_kernel(const RelTask* __restrict__ tasks,
                                                                     const RelBox* __restrict__ boxes,
                                                                     const int2* __restrict__ chunks, double* blk,
-                                                                    double* mat, int dir, double alpha, double beta) {
+                                                                    double* mat, int dir, double alpha, double beta,
+                                                                    bool beside) {
   __shared__ RelLegs sh;
+  grid_trigger();
   const int2 c = chunks[blockIdx.x];
-  relayout_legs<kRelThreads>(sh, boxes[c.x], c.y, min(tasks[c.x].n, c.y + kChunk), blk, mat, dir, alpha, beta);
+  const int end = min(tasks[c.x].n, c.y + kChunk);
+  if (!beside) grid_wait();
+  relayout_legs<kRelThreads>(sh, boxes[c.x], c.y, end, blk, mat, dir, alpha, beta);
+  if (beside) grid_wait();
 }
 
 __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(const RelBox* __restrict__ boxes,
@@ -162,16 +167,19 @@ __global__ void rel_boxes_kernel(const RelTask* tasks, int n, RelBox* boxes) {
 // for its tables and two more barriers (a D = 4, chi = 64 permutation takes
 // 14 us by boxes, 10 by legs; the odd-sized FP64 corner's copies 89 and 32);
 // with the same innermost leg on both sides the direct copy reaches 5.1 TB/s.
+// order 1: behind this call's previous kernel, 2: beside it (neither touches
+// what the other writes).
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir, double alpha,
-                     double beta, cudaStream_t s) {
+                     double beta, cudaStream_t s, int order) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
   if (r.boxes && r.transposes)
     relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                           beta);
   else if (r.boxes)
-    relayout_legs_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, const_cast<double*>(blk), mat, dir,
-                                                          alpha, beta);
+    launch_behind(order != 0, relayout_legs_kernel, dim3(unsigned(r.nchunks)), kRelThreads, 0, s, (const RelTask*)r.tasks,
+                  (const RelBox*)r.boxes, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta,
+                  order == 2);
   else
     relayout_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                       beta);

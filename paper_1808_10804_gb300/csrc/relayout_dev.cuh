@@ -5,6 +5,32 @@
 
 namespace bst {
 
+// A grid launched behind another (launch_behind) may start when every block
+// of the first has called grid_trigger (or left), and must call grid_wait,
+// which returns when the first has finished and its writes are visible,
+// before it touches what that grid reads or writes, and in every block before
+// it ends (so that a third grid that waits for it waits for both).
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch with programmatic serialisation behind the previous kernel of the
+// stream (behind: that kernel is this library's, launched by the same call),
+// else an ordinary one.
+template <class... P, class... A>
+void launch_behind(bool behind, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = behind ? 1 : 0;
+  BST_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+}
+
 // Division by a runtime constant d >= 1 for numerators below 2^31 with one
 // high multiply, an add and a shift (Granlund and Montgomery's round-up
 // method): l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1,

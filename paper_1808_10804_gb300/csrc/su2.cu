@@ -715,7 +715,7 @@ void su2_contract(Ctx* ctx, Layout* A, const double* a, Layout* B, const double*
   BST_REQUIRE((A->nnz == 0 || a) && (B->nnz == 0 || b) && (C->nnz == 0 || c), BST_E_ARG, "data pointer is NULL");
   if (C->nnz == 0) return;
   launch_relayout(ctx, p->ra, a, p->Am, 0, 1.0, 0.0, s);
-  launch_relayout(ctx, p->rb, b, p->Bm, 0, 1.0, 0.0, s);
+  launch_relayout(ctx, p->rb, b, p->Bm, 0, 1.0, 0.0, s, p->ra.nchunks ? 2 : 0);
   ctx->work_flops += p->g.flops;
   if (!p->probs.empty()) {
     if (prec == BST_FP64) {
