@@ -295,7 +295,10 @@ int64_t plan_check(Ctx* ctx, Layout* A, Layout* B, const std::vector<int>& la, c
 // relayout.cu
 std::vector<int2> relayout_chunks(const std::vector<RelTask>& t);  // chunk table of a task list
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir,
-                     double alpha, double beta, cudaStream_t s, int order = 0);
+                     double alpha, double beta, cudaStream_t s, bool behind = false);
+// the gathers of both operands of a contraction, in one launch where they can be
+void launch_gathers(Ctx* ctx, const DevRelayout& ra, const double* a, double* Am, const DevRelayout& rb,
+                    const double* b, double* Bm, cudaStream_t s);
 
 // gemm_f64.cu
 DevGemm* get_dev_gemm(Ctx* ctx, const std::string& key, const std::vector<GemmProb>& probs);

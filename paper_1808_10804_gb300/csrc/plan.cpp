@@ -212,16 +212,15 @@ void run_contract(Ctx* ctx, ContractPlan* p, const double* a, const double* b, b
   double* Cm = (double*)ctx->buf("contract.C", sizeof(double) * std::max<int64_t>(p->cmat, 1), s);
   double* Am = (double*)ctx->buf("contract.A", sizeof(double) * std::max<int64_t>(p->amat, 1), s);
   double* Bm = (double*)ctx->buf("contract.B", sizeof(double) * std::max<int64_t>(p->bmat, 1), s);
-  launch_relayout(ctx, p->ra, a, Am, 0, 1.0, 0.0, s);
-  // The first kernel starts when everything before the call is done; the
-  // others' launches overlap the one before, and B's copy all of A's (a D = 4,
-  // chi = 16 edge by itself 53 -> 41 us).  The GEMM only while it is as short
+  // The gathers start when everything before the call is done; the other
+  // launches overlap the one before (a D = 4, chi = 16 edge by itself 53 ->
+  // 41 us).  The GEMM only while it is as short
   // as a launch: blocks that start on the SMs that the copies leave first end
   // up two on one and none on another (an odd-sized corner of 0.33 GFLOP
   // 447 -> 509 us).
-  launch_relayout(ctx, p->rb, b, Bm, 0, 1.0, 0.0, s, p->ra.nchunks ? 2 : 0);
+  launch_gathers(ctx, p->ra, a, Am, p->rb, b, Bm, s);
   launch_gemm_f64(ctx, p->g, Am, Bm, Cm, s, p->g.flops < 1.5e7 && (p->ra.nchunks || p->rb.nchunks));
-  launch_relayout(ctx, p->rc, c, Cm, 1, alpha, beta, s, p->g.ntiles ? 1 : 0);
+  launch_relayout(ctx, p->rc, c, Cm, 1, alpha, beta, s, p->g.ntiles > 0);
 }
 
 // ---- permute -------------------------------------------------------------------

@@ -137,15 +137,29 @@ __global__ void __launch_bounds__(kRelThreads) relayout_kernel(const RelTask* __
 __global__ void __launch_bounds__(kRelThreads) relayout_legs_kernel(const RelTask* __restrict__ tasks,
                                                                     const RelBox* __restrict__ boxes,
                                                                     const int2* __restrict__ chunks, double* blk,
-                                                                    double* mat, int dir, double alpha, double beta,
-                                                                    bool beside) {
+                                                                    double* mat, int dir, double alpha, double beta) {
   __shared__ RelLegs sh;
   grid_trigger();
   const int2 c = chunks[blockIdx.x];
   const int end = min(tasks[c.x].n, c.y + kChunk);
-  if (!beside) grid_wait();
+  grid_wait();
   relayout_legs<kRelThreads>(sh, boxes[c.x], c.y, end, blk, mat, dir, alpha, beta);
-  if (beside) grid_wait();
+}
+
+// Both operands' gathers of a contraction in one launch.
+struct RelPart {
+  const RelTask* tasks;
+  const RelBox* boxes;
+  const int2* chunks;
+  double *blk, *mat;
+};
+__global__ void __launch_bounds__(kRelThreads) relayout_pair_kernel(RelPart a, RelPart b, int na) {
+  __shared__ RelLegs sh;
+  grid_trigger();
+  const bool first = int(blockIdx.x) < na;
+  const RelPart p = first ? a : b;
+  const int2 c = p.chunks[int(blockIdx.x) - (first ? 0 : na)];
+  relayout_legs<kRelThreads>(sh, p.boxes[c.x], c.y, min(p.tasks[c.x].n, c.y + kChunk), p.blk, p.mat, 0, 1.0, 0.0);
 }
 
 __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(const RelBox* __restrict__ boxes,
@@ -167,22 +181,35 @@ __global__ void rel_boxes_kernel(const RelTask* tasks, int n, RelBox* boxes) {
 // for its tables and two more barriers (a D = 4, chi = 64 permutation takes
 // 14 us by boxes, 10 by legs; the odd-sized FP64 corner's copies 89 and 32);
 // with the same innermost leg on both sides the direct copy reaches 5.1 TB/s.
-// order 1: behind this call's previous kernel, 2: beside it (neither touches
-// what the other writes).
+// behind: the previous kernel of the stream is this call's, launch_behind.
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir, double alpha,
-                     double beta, cudaStream_t s, int order) {
+                     double beta, cudaStream_t s, bool behind) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
   if (r.boxes && r.transposes)
     relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                           beta);
   else if (r.boxes)
-    launch_behind(order != 0, relayout_legs_kernel, dim3(unsigned(r.nchunks)), kRelThreads, 0, s, (const RelTask*)r.tasks,
-                  (const RelBox*)r.boxes, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta,
-                  order == 2);
+    launch_behind(behind, relayout_legs_kernel, dim3(unsigned(r.nchunks)), kRelThreads, 0, s, (const RelTask*)r.tasks,
+                  (const RelBox*)r.boxes, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta);
   else
     relayout_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                       beta);
+  BST_CUDA(cudaGetLastError());
+  count_launch(ctx);
+}
+
+void launch_gathers(Ctx* ctx, const DevRelayout& ra, const double* a, double* Am, const DevRelayout& rb,
+                    const double* b, double* Bm, cudaStream_t s) {
+  if (ra.nchunks == 0 || rb.nchunks == 0 || !ra.boxes || !rb.boxes || ra.transposes || rb.transposes) {
+    launch_relayout(ctx, ra, a, Am, 0, 1.0, 0.0, s);
+    launch_relayout(ctx, rb, b, Bm, 0, 1.0, 0.0, s);
+    return;
+  }
+  ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * (ra.elems + rb.elems));
+  relayout_pair_kernel<<<ra.nchunks + rb.nchunks, kRelThreads, 0, s>>>(
+      RelPart{ra.tasks, ra.boxes, ra.chunks, const_cast<double*>(a), Am},
+      RelPart{rb.tasks, rb.boxes, rb.chunks, const_cast<double*>(b), Bm}, ra.nchunks);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

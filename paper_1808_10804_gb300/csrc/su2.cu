@@ -714,8 +714,7 @@ void su2_contract(Ctx* ctx, Layout* A, const double* a, Layout* B, const double*
   BST_REQUIRE(p->C == C, BST_E_SHAPE, "C is not the layout of this contraction");
   BST_REQUIRE((A->nnz == 0 || a) && (B->nnz == 0 || b) && (C->nnz == 0 || c), BST_E_ARG, "data pointer is NULL");
   if (C->nnz == 0) return;
-  launch_relayout(ctx, p->ra, a, p->Am, 0, 1.0, 0.0, s);
-  launch_relayout(ctx, p->rb, b, p->Bm, 0, 1.0, 0.0, s, p->ra.nchunks ? 2 : 0);
+  launch_gathers(ctx, p->ra, a, p->Am, p->rb, b, p->Bm, s);
   ctx->work_flops += p->g.flops;
   if (!p->probs.empty()) {
     if (prec == BST_FP64) {
