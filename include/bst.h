@@ -141,7 +141,7 @@ BST_API double bst_ctx_work_flops(bst_ctx ctx);
  *     N^T N with a block of b vectors (CholQR orthonormalisation; b = 160
  *     for BST_FP64, for BST_OZAKI k + k/2 + 16 rounded up to 32 in 64..160,
  *     k the most states the sector can hold: chi, or chi / (2J+1) for an
- *     SU(2) sector of spin J), in rounds (the first of at most `iters`
+ *     SU(2) sector of spin J), in rounds (the first of at most 2 `iters`
  *     steps: three plain ones, then Chebyshev filters of the block chosen by
  *     the spectrum seen so far; later rounds sized to converge; plain steps,
  *     `iters` or sized by the residual's observed decay, where no filter

@@ -695,7 +695,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   // when none fits: a spectrum so steep that the growth bound puts alpha
   // above a kept value (plain steps, which factor after every half).
   double gain = 1.0;  // growth that the plan gives every kept value
-  auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod) {
+  auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod, int settled = 0) {
     std::vector<std::pair<double, int>> all;
     for (size_t i = 0; i < secs.size(); ++i)
       if (!secs[i].direct)
@@ -713,6 +713,19 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       double& l = lowest[all[t].second];
       if (int64_t(t) < chi || l == 0) l = all[t].first;
     }
+    // (plain steps before: the kept values have grown by their ratio to the
+    // block's lower end in each)
+    double ratio = 1e300;
+    for (size_t i = 0; i < secs.size(); ++i)
+      if (lowest[i] > 0) {
+        double low = lowest[i];
+        for (int j = 0; j < secs[i].c; ++j) {
+          const double d = v[secs[i].val_off + j];
+          if (d > 0) low = std::min(low, d);
+        }
+        ratio = std::min(ratio, lowest[i] / low);
+      }
+    if (settled > 0 && ratio < 1e300) need /= std::pow(ratio, settled);
     // the filter of degree m and the growth of the kept values (0: does not fit)
     auto of_degree = [&](int m, Filter& f) {
       const double span = std::pow(2e10, 1.0 / m) / 4.0;  // largest lambda_1 / alpha
@@ -895,8 +908,10 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   int total = 0, steps = iters;
   std::vector<Filter> fplan;  // filters of the next round (in place of its plain steps)
   bool may_filter = true;
+  int worked = 0;  // rounds that iterated
   for (int round = 0;; ++round) {
     const bst_prec rrp = mixed_rr ? prec : rr;
+    worked += steps > 0;
     if (!sp_it.empty()) {
       if (round == 0 && steps >= settle + 2) {
         iterate(settle);
@@ -908,8 +923,13 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
         BST_CUDA(cudaStreamSynchronize(s));
         const int left = steps - settle;
         // (a column's share of an earlier direction is about the ratio of
-        // their values to the number of products so far: no degree above it)
-        fplan = plan_filters(est, 1.0 / (0.02 * tol), settle, left);
+        // their values to the number of products so far: no degree above it.
+        // Sized to converge with a margin of ~200, the residual being about a
+        // tenth of the growth's inverse: up to twice the plain steps cost less
+        // than a Rayleigh-Ritz step more.  Twelve D = 6, chi = 72 projectors:
+        // 5.00 ms with at most 9 steps in the round, 4.80 without a margin,
+        // 4.38 so.)
+        fplan = plan_filters(est, 20.0 / tol, settle, left + iters, settle);
         total += settle;
         if (!fplan.empty()) {
           polish_tri(Q, Y);
@@ -1111,7 +1131,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   }
   if (prec != BST_FP64) {
     if (ctx->multi_round.size() >= 4096) ctx->multi_round.clear();
-    ctx->multi_round[rr_key] = total > iters;
+    ctx->multi_round[rr_key] = worked > 1;
   }
   hSig.assign(valtot, 0.0);
   for (auto& x : secs) {
