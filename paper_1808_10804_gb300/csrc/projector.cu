@@ -631,10 +631,10 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   // by cosh(m acosh(2 lambda / alpha - 1)): two to four times the plain
   // steps' decay per product, at a quarter of their factorisations (which
   // cost more than the products: one CTA a sector).
-  // Measured (plain steps -> filters): the D=6, chi=72 half systems of random
-  // environments 40 steps -> 12, projector 7.8 -> 5.8 ms, full move (after the
-  // contractions' own gains) 33.9 -> 25.5 ms; D=8, chi=192 left move 61 steps
-  // -> 39, 98 -> 84 ms; SU(2) left move 23.0 -> 17.1 ms.
+  // Measured (plain steps -> filters, with the kernels of that time): the D=6,
+  // chi=72 half systems of random environments 40 steps -> 12, projector 7.8 ->
+  // 5.8 ms, full move 33.9 -> 25.5 ms; D=8, chi=192 left move 61 steps -> 39,
+  // 98 -> 84 ms; SU(2) left move 23.0 -> 17.1 ms.
   // Columns grow apart by up to (4 lambda_1 / alpha)^m / 2 between
   // factorisations, and so does what a column holds of an earlier one's
   // direction.  The FP32 factor leaves ~1e-6 of that; a triangular first-order
