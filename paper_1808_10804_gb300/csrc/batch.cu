@@ -101,7 +101,9 @@ struct BatchPlan {
 constexpr int kBatchThreads = 256;
 constexpr int kChunkChoices[] = {1024, 2048, 4096, 8192};
 
-// Same copies as relayout_legs_kernel, with a per-task base pointer.
+// Same copies as relayout_legs_kernel (or, without boxes, relayout_kernel),
+// with a per-task base pointer.
+template <bool kBoxes>
 __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const BatchTask* __restrict__ tasks,
                                                                        const RelBox* __restrict__ boxes,
                                                                        const int2* __restrict__ chunks,
@@ -111,7 +113,11 @@ __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const Bat
   const int2 c = chunks[blockIdx.x];
   __shared__ RelLegs sh;
   const BatchTask& bt = tasks[c.x];
-  relayout_legs<kBatchThreads>(sh, boxes[c.x], c.y, min(bt.t.n, c.y + chunk), bases[bt.src], mat, dir, alpha, beta);
+  const int end = min(bt.t.n, c.y + chunk);
+  if constexpr (kBoxes)
+    relayout_legs<kBatchThreads>(sh, boxes[c.x], c.y, end, bases[bt.src], mat, dir, alpha, beta);
+  else
+    relayout_range<kBatchThreads>(bt.t, c.y, end, bases[bt.src], mat, dir, alpha, beta);
 }
 
 // (Re)build the chunk table of a relayout for `chunk` elements per CTA.
@@ -129,9 +135,12 @@ static void upload_rel(BatchRel& r, int chunk) {
     BST_CUDA(cudaMalloc(&r.tasks, sizeof(BatchTask) * r.host.size()));
     BST_CUDA(cudaMemcpy(r.tasks, r.host.data(), sizeof(BatchTask) * r.host.size(), cudaMemcpyHostToDevice));
     std::vector<RelBox> hb(r.host.size());
-    for (size_t i = 0; i < hb.size(); ++i) rel_make_box(r.host[i].t, hb[i]);
-    BST_CUDA(cudaMalloc(&r.boxes, sizeof(RelBox) * hb.size()));
-    BST_CUDA(cudaMemcpy(r.boxes, hb.data(), sizeof(RelBox) * hb.size(), cudaMemcpyHostToDevice));
+    bool ok = true;  // (no boxes past 32-bit offsets)
+    for (size_t i = 0; i < hb.size(); ++i) rel_make_box(r.host[i].t, hb[i]), ok = ok && hb[i].ntiles > 0;
+    if (ok) {
+      BST_CUDA(cudaMalloc(&r.boxes, sizeof(RelBox) * hb.size()));
+      BST_CUDA(cudaMemcpy(r.boxes, hb.data(), sizeof(RelBox) * hb.size(), cudaMemcpyHostToDevice));
+    }
   }
   if (!ch.empty()) {
     BST_CUDA(cudaMalloc(&r.chunks, sizeof(int2) * ch.size()));
@@ -143,8 +152,8 @@ static void launch_rel(Ctx* ctx, const BatchRel& r, double* const* bases, double
                        double beta, cudaStream_t s) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  relayout_batch_kernel<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, bases, mat, dir, alpha, beta,
-                                                            r.chunk);
+  auto kern = r.boxes ? relayout_batch_kernel<true> : relayout_batch_kernel<false>;
+  kern<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, bases, mat, dir, alpha, beta, r.chunk);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }
