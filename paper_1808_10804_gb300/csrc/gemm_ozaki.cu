@@ -41,11 +41,11 @@
 // conversion and four rows side by side.  The launch is programmatic behind
 // the split or pack: 1.6 us less per contraction.
 //
-// Every wait of the pipeline
-// is bounded by the launch's spin limit: on expiry the kernel records
-// BST_E_TIMEOUT in the context's error word and every role leaves its loop;
-// before tensor memory is freed and the CTA exits, the TMA copies it has
-// issued and the products it has issued are waited for (they always
+// Every wait of the pipeline is bounded by the launch's spin limit: on expiry
+// the kernel records BST_E_TIMEOUT in the context's error word, the copying
+// and the issuing role leave their loops, and the output stage stores nothing
+// more; before tensor memory is freed and the CTA exits, the TMA copies it
+// has issued and the products it has issued are waited for (they always
 // complete; those waits carry a separate, much larger bound).
 #include <cuda.h>
 #include <cooperative_groups.h>
@@ -476,9 +476,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int row = q * 32 + lane;
     const uint32_t lane_base = tmem + (uint32_t(q * 32) << 16);
     uint32_t buf = 0, bph = 0;
+    // Each lane polls for itself, so when a wait expires, or another role has
+    // aborted, some lanes of a warp may have seen the phase complete and
+    // others not.  A lane that gave up does not leave its warp, whose loads,
+    // shuffles and barriers need it: it walks on to the last tile, with no
+    // more waits and nothing stored (a vote per wait instead cost an SU(2)
+    // corner 2 %, 607 -> 620 us).
     bool ok = true;
     Tile t = tiles[blockIdx.x];
-    for (int ti = blockIdx.x; ti < ntiles && ok;) {
+    for (int ti = blockIdx.x; ti < ntiles;) {
       ti += gridDim.x;
       const Tile nxt = ti < ntiles ? tiles[ti] : t;
       // the tile's rows and columns, loaded while its products run: lane l
@@ -527,8 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kCols; ++j) T[j] = 0;
       const int npair = (t.nk + 1) >> 1;
       for (int pp = 0; pp < npair; ++pp) {
-        ok = mbar_wait(&sm.acc_full[buf], bph, abort_flag, err, spin);
-        if (!ok) break;
+        if (ok) ok = mbar_wait(&sm.acc_full[buf], bph, abort_flag, err, spin);
         tc_fence_after();
         if (idle) {
           mbar_arrive(&sm.acc_empty[buf]);
@@ -563,7 +568,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         buf ^= 1u;
         if (buf == 0) bph ^= 1u;
       }
-      if (!ok) break;
       if (idle) {
         if constexpr (S == 5) mbar_arrive(&sm.acc34_empty);
         t = nxt;
@@ -619,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < 8; ++j) st[lane][j] = (long long)T[h * 8 + j];
         __syncwarp();
         const int col = h * 8 + (lane & 7);
-        const bool col_ok = col < ncols;
+        const bool col_ok = col < ncols && ok;
         double* cbase;
         int rstride;  // between output rows of a block
         if (scatter) {

@@ -52,3 +52,43 @@ def test_pipeline_wait_timeout_is_reported_and_recovered(bst):
         assert torch.equal(out2, ref)     # same bits as before the timeout
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["ozaki", "bf16x3"])
+def test_any_wait_limit_ends(bst, prec):
+    """Limits between one poll and enough of them: the roles of a CTA, and
+    the lanes of a warp, give up at different points of the pipeline.  Every
+    launch ends, with the timeout reported or with the right bits, and the
+    next unlimited call gives them."""
+    ctx = bst.Context(0)
+    try:
+        rng = np.random.default_rng(22)
+        # several tiles a CTA, of one to seven chunk pairs, some with idle warps
+        r = u1.Leg(1, (-2, 0, 2), (1300, 2000, 700))
+        k = u1.Leg(-1, (-2, 0, 2), (24, 400, 200))
+        c = u1.Leg(-1, (-2, 0, 2), (530, 2100, 1050))
+        A = ctx.layout([to_bst_leg(bst, l) for l in (r, k)])
+        B = ctx.layout([to_bst_leg(bst, l) for l in (k.dual(), c)])
+        a = torch.tensor(rng.standard_normal(A.nnz), dtype=torch.float64, device="cuda:0")
+        b = torch.tensor(rng.standard_normal(B.nnz), dtype=torch.float64, device="cuda:0")
+        CL, ref = ctx.contract(A, a, B, b, [1], [0], prec=prec)
+        ctx.sync()
+        out = torch.zeros_like(ref)
+        expired = 0
+        for limit in (1, 2, 3, 4, 6, 8, 12, 16, 32, 64, 128, 1024, 1 << 16):
+            ctx.set_wait_limit(limit)
+            out.zero_()
+            ctx.contract(A, a, B, b, [1], [0], prec=prec, Cl=CL, c=out)
+            try:
+                ctx.sync()
+                assert torch.equal(out, ref), limit
+            except bst.BstError as e:
+                assert e.code == 6        # BST_E_TIMEOUT
+                expired += 1
+        assert expired >= 1
+        ctx.set_wait_limit(0)
+        ctx.contract(A, a, B, b, [1], [0], prec=prec, Cl=CL, c=out)
+        ctx.sync()
+        assert torch.equal(out, ref)
+    finally:
+        ctx.close()
