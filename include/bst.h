@@ -293,7 +293,8 @@ BST_API bst_status bst_plan_check(bst_ctx ctx, bst_layout A, bst_layout B, int32
  * charge through the cut, so every group is one dense GEMM whose result is
  * already reduced (Sec. 2, grouping by output quantum numbers so the
  * unreduced result never exists).  `prec` selects the GEMM arithmetic.
- * beta == 0 ignores the previous contents of c (NaN-safe).
+ * beta == 0 ignores the previous contents of c (NaN-safe).  c may overlap a
+ * and b: both have been read before any of c is written.
  * SU(2) tensors (both A and B BST_SU2): every pair of blocks that agree on
  * the contracted legs contributes m_A . m_B, expanded into the output's
  * canonical blocks with X = <c_C, c_A . c_B> / (2 J_C + 1) (Sec. 2: the CGC

@@ -1723,11 +1723,13 @@ static void launch_clusters(void (*kern)(P...), int grid, int threads, int csize
 }
 
 // A, B: the operands' sector matrices, or for a packed plan the operand
-// tensors themselves (tabA / tabB: per-segment tensor tables of a batch)
+// tensors themselves (tabA / tabB: per-segment tensor tables of a batch).
+// zeros_last: C overlaps an operand, so no output is written before a packed
+// plan has read both.
 static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, double* C, cudaStream_t s,
                      bool split_a = true, double alpha = 1.0, double beta = 0.0,
                      const double* const* tabA = nullptr, const double* const* tabB = nullptr,
-                     const long long* bbase = nullptr) {
+                     const long long* bbase = nullptr, bool zeros_last = false) {
   const oz::Scatter sc{P->d_rowtab, P->d_coltab, bbase ? bbase : P->d_bbase, alpha, beta};
   const bool b_from_a = P->ab_same && A == B && split_a;
   if (P->packed) {
@@ -1735,7 +1737,7 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
     // 512 once more from cache), S digits written; the byte count is that of
     // the split of gathered rows without the FP64 row write and read of a
     // separate gather.  The K == 0 problems' outputs are written by the same
-    // launch.
+    // launch, or by one behind it.
     ProfScope ps(ctx, s, "pack_bf16", 0.0, P->split_bytes);
     const oz::PackJob ja{P->d_pgA, P->d_psA, P->d_pcA, P->rowsA, A, tabA, P->SA, P->eA};
     const oz::PackJob jb{P->d_pgB, P->d_psB, P->d_pcB, P->rowsB, B, tabB, P->SB, P->eB};
@@ -1748,12 +1750,14 @@ static void run_plan(Ctx* ctx, OzakiPlan* P, const double* A, const double* B, d
                       cs, s, ja, jb, ga, ga + gb, cs, P->kpitch, zj);
       count_launch(ctx);
     };
+    const int gz0 = zeros_last ? 0 : gz;
     if (P->pack_apart) {
       pack(P->ncA, 0, 0);
-      pack(0, P->ncB, gz);
+      pack(0, P->ncB, gz0);
     } else {
-      pack(P->ncA, P->ncB, gz);
+      pack(P->ncA, P->ncB, gz0);
     }
+    if (zeros_last) pack(0, 0, gz);
     if (P->ntiles == 0) return;
   } else {
     // the split of both operands; the K == 0 problems' outputs are written
@@ -1918,7 +1922,11 @@ void run_gemm_ozaki_scatter(Ctx* ctx, ContractPlan* p, int S, const double* a, c
     P = prepare_scatter(ctx, p, S);
     attach_pack(P, p);
   }
-  run_plan(ctx, P, a, b, c, s, true, alpha, beta);
+  auto meets = [&](const double* x, const Layout* X) {
+    const uintptr_t x0 = uintptr_t(x), c0 = uintptr_t(c);
+    return x0 < c0 + sizeof(double) * p->C->nnz && c0 < x0 + sizeof(double) * X->nnz;
+  };
+  run_plan(ctx, P, a, b, c, s, true, alpha, beta, nullptr, nullptr, nullptr, meets(a, p->A) || meets(b, p->B));
 }
 
 void run_gemm_ozaki(Ctx* ctx, ContractPlan* p, int S, const double* Am, const double* Bm, double* Cmat,

@@ -114,3 +114,34 @@ def test_unmatched_output_sectors(bst, ctx, M, N, beta):
     assert zero.sum() >= M * N
     assert np.array_equal(out[zero], (beta * old)[zero])
     assert np.abs(out - ref)[~zero].max(initial=0.0) <= 1e-10
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+@pytest.mark.parametrize("over", ["a", "b", "both"])
+@pytest.mark.parametrize("inner", ["open", "contracted"])
+def test_output_over_an_operand(bst, ctx, inner, over, beta):
+    """The output laid over an operand, so that its last sector, which has no
+    match, covers blocks that do count: the bits of a call with buffers of
+    their own."""
+    rng = np.random.default_rng(7)
+    open_a, open_b, k = bst.Leg(1, (0, 1, 2), (300, 411, 257)), bst.Leg(-1, (0, 1, 2), (190, 333, 222)), (0, 1)
+    ka, kb = bst.Leg(-1, k, (65, 130)), bst.Leg(1, k, (65, 130))
+    A = ctx.layout([ka, open_a] if inner == "open" else [open_a, ka])
+    B = ctx.layout([kb, open_b] if inner == "open" else [open_b, kb])
+    pairs = ((0,), (0,)) if inner == "open" else ((1,), (1,))
+    C = ctx.contract_layout(A, B, *pairs)
+    n = A.nnz + B.nnz + C.nnz
+    data = torch.tensor(rng.standard_normal(n), device="cuda:0")
+    end = C.nnz - 257 * 222 // 2  # in the middle of that sector
+    off = {"a": (end - A.nnz // 2, 0, end + A.nnz), "b": (end + B.nnz, 0, end - B.nnz // 2),
+           "both": (end - A.nnz // 2, 0, end - B.nnz // 2)}[over]
+    part = lambda x, o, L: x[o:o + L.nnz]  # noqa: E731
+    assert max(o + L.nnz for o, L in zip(off, (A, C, B))) <= n
+    a0, c0, b0 = (part(data, o, L).clone() for o, L in zip(off, (A, C, B)))
+    for prec in ("ozaki", "bf16x3", "fp64"):
+        ref = ctx.contract(A, a0, B, b0, *pairs, prec=prec, beta=beta, Cl=C, c=c0.clone())[1]
+        x = data.clone()
+        a, c, b = (part(x, o, L) for o, L in zip(off, (A, C, B)))
+        ctx.contract(A, a, B, b, *pairs, prec=prec, beta=beta, Cl=C, c=c)
+        ctx.sync()
+        assert torch.equal(c, ref), prec
