@@ -20,6 +20,7 @@
 #include <numeric>
 
 #include "bst_internal.h"
+#include "residual.h"
 
 namespace bst {
 
@@ -976,7 +977,7 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       std::vector<double> rv;
       for (auto& x : secs)
         if (!x.direct)
-          for (int j = 0; j < x.c; ++j) rv.push_back(hl[x.val_off + j]);
+          for (int j = 0; j < x.c; ++j) rv.push_back(std::isfinite(hl[x.val_off + j]) ? hl[x.val_off + j] : 0.0);
       double cut = 0;
       if (int64_t(rv.size()) >= chi && chi > 0) {
         std::nth_element(rv.begin(), rv.begin() + (chi - 1), rv.end(), std::greater<double>());
@@ -1031,7 +1032,8 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     std::vector<std::pair<double, int>> all;
     for (size_t i = 0; i < secs.size(); ++i)
       for (int j = 0; j < secs[i].c; ++j) {
-        const double v = hl[secs[i].val_off + j];
+        // (a value that is not finite has no place in the order)
+        const double v = std::isfinite(hl[secs[i].val_off + j]) ? hl[secs[i].val_off + j] : 0.0;
         lmax = std::max(lmax, v);
         all.push_back({v, int(i)});
       }
@@ -1066,9 +1068,19 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       count_launch(ctx);
       BST_CUDA(cudaMemcpyAsync(hres.data(), res, sizeof(double) * valtot, cudaMemcpyDeviceToHost, s));
       BST_CUDA(cudaStreamSynchronize(s));
-      for (auto& r : rp)
-        for (int j = 0; j < r.k; ++j) worst = std::max(worst, hres[r.val_off + j]);
-      worst = lmax > 0 ? worst / lmax : 0.0;
+      for (auto& r : rp) worst = raise_worst(worst, &hres[r.val_off], size_t(r.k));
+      if (std::isfinite(worst)) worst = lmax > 0 ? worst / lmax : 0.0;
+    }
+    for (auto& x : secs)
+      if (!x.direct && !std::isfinite(raise_worst(0.0, &hl[x.val_off], size_t(x.c))))
+        worst = std::numeric_limits<double>::infinity();
+    if (!std::isfinite(worst)) {
+      // N itself not finite (its norm tells): no step can help, the caller
+      // refuses it
+      double nss = 0;
+      BST_CUDA(cudaMemcpyAsync(&nss, ctx->buf("proj.nss", sizeof(double), s), sizeof(double), cudaMemcpyDeviceToHost, s));
+      BST_CUDA(cudaStreamSynchronize(s));
+      if (!std::isfinite(nss)) break;
     }
     if (ctx->tune_log.size() < (1u << 20)) {
       char line[160];
@@ -1103,9 +1115,17 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     // A residual above lambda_max: the refinement of the Ritz vectors
     // diverged (a cluster of many values ~1e-9 apart), they are no basis to
     // go on from; plain steps resume from the block before it, or from a new
-    // one if it had been filtered.
+    // one if it had been filtered or is not finite itself.
     const bool diverged = !(worst <= 1.0);
-    const bool lost = !fplan.empty() && (diverged || (round == 0 && !(worst <= 1e-4) && !(worst * gain <= 1e4)));
+    bool lost = !fplan.empty() && (diverged || (round == 0 && !(worst <= 1e-4) && !(worst * gain <= 1e4)));
+    if (!std::isfinite(worst) && !lost) {
+      double* qss = (double*)ctx->buf("proj.qss", sizeof(double), s);
+      double h = 0;
+      launch_sumsq(ctx, Q, qtot, qss, s);
+      BST_CUDA(cudaMemcpyAsync(&h, qss, sizeof(double), cudaMemcpyDeviceToHost, s));
+      BST_CUDA(cudaStreamSynchronize(s));
+      lost = !std::isfinite(h);
+    }
     if (lost || diverged) may_filter = false;
     fplan.clear();
     if (!ok && may_filter && worst > 0 && std::isfinite(worst))

@@ -118,3 +118,27 @@ def test_solves_side_by_side(bst, prec):
             u = svd[s][0][:, :6]
             assert np.linalg.norm(a @ b - u @ u.T) <= bound
     ctx.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+def test_operand_not_finite_is_refused(bst, prec, bad):
+    """One entry that is not finite: refused at once, whatever an earlier call
+    with the same sectors learnt, and the next call is as good as the first."""
+    rows = (170, 203)
+    ctx = bst.Context(0)
+    leg = lambda f: bst.Leg(f, (0, 1), rows)  # noqa: E731
+    Rt, Rb = ctx.layout([leg(1), leg(-1)]), ctx.layout([leg(-1), leg(1)])
+    rng = np.random.default_rng(5)
+    flat = lambda xs: torch.tensor(np.concatenate([x.reshape(-1) for x in xs]), device="cuda:0")  # noqa: E731
+    eye, good = flat([np.eye(r) for r in rows]), flat([rng.standard_normal((r, r)) / r for r in rows])
+    sv = []
+    for call in range(3):
+        sv.append(np.sort(ctx.svd_projector(Rt, eye, Rb, good, 1, CHI, 1e-14, 1, prec=prec)[4]))
+        x = good.clone()
+        x[(5, 170 * 170 + 77, 40000)[call]] = bad
+        with pytest.raises(bst.BstError) as e:
+            ctx.svd_projector(Rt, eye, Rb, x, 1, CHI, 1e-14, 1, prec=prec)
+        assert e.value.code == 7  # BST_E_NUMERIC
+        assert np.abs(sv[-1] - sv[0]).max() <= 1e-9 * sv[0].max()
+    ctx.close()
