@@ -36,7 +36,7 @@ struct BatchTask {
 
 struct BatchRel {
   BatchTask* tasks = nullptr;
-  RelBox* boxes = nullptr;
+  RelLegTab* legs = nullptr;
   int2* chunks = nullptr;
   int nchunks = 0;
   int chunk = 2048;  // elements per CTA
@@ -44,10 +44,10 @@ struct BatchRel {
   std::vector<BatchTask> host;
   void free_all() {
     cudaFree(tasks);
-    cudaFree(boxes);
+    cudaFree(legs);
     cudaFree(chunks);
     tasks = nullptr;
-    boxes = nullptr;
+    legs = nullptr;
     chunks = nullptr;
   }
 };
@@ -101,11 +101,11 @@ struct BatchPlan {
 constexpr int kBatchThreads = 256;
 constexpr int kChunkChoices[] = {1024, 2048, 4096, 8192};
 
-// Same copies as relayout_legs_kernel (or, without boxes, relayout_kernel),
+// Same copies as relayout_legs_kernel (or, without tables, relayout_kernel),
 // with a per-task base pointer.
-template <bool kBoxes>
+template <bool kLegs>
 __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const BatchTask* __restrict__ tasks,
-                                                                       const RelBox* __restrict__ boxes,
+                                                                       const RelLegTab* __restrict__ legs,
                                                                        const int2* __restrict__ chunks,
                                                                        double* const* __restrict__ bases,
                                                                        double* mat, int dir, double alpha,
@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const Bat
   __shared__ RelLegs sh;
   const BatchTask& bt = tasks[c.x];
   const int end = min(bt.t.n, c.y + chunk);
-  if constexpr (kBoxes)
-    relayout_legs<kBatchThreads>(sh, boxes[c.x], c.y, end, bases[bt.src], mat, dir, alpha, beta);
+  if constexpr (kLegs)
+    relayout_legs<kBatchThreads>(sh, legs[c.x], c.y, end, bases[bt.src], mat, dir, alpha, beta);
   else
     relayout_range<kBatchThreads>(bt.t, c.y, end, bases[bt.src], mat, dir, alpha, beta);
 }
@@ -134,12 +134,12 @@ static void upload_rel(BatchRel& r, int chunk) {
   if (!r.host.empty()) {
     BST_CUDA(cudaMalloc(&r.tasks, sizeof(BatchTask) * r.host.size()));
     BST_CUDA(cudaMemcpy(r.tasks, r.host.data(), sizeof(BatchTask) * r.host.size(), cudaMemcpyHostToDevice));
-    std::vector<RelBox> hb(r.host.size());
-    bool ok = true;  // (no boxes past 32-bit offsets)
-    for (size_t i = 0; i < hb.size(); ++i) rel_make_box(r.host[i].t, hb[i]), ok = ok && hb[i].ntiles > 0;
+    std::vector<RelLegTab> hl(r.host.size());
+    bool ok = true;  // (no tables past 32-bit offsets)
+    for (size_t i = 0; i < hl.size(); ++i) rel_make_legs(r.host[i].t, hl[i]), ok = ok && rel_narrow(r.host[i].t);
     if (ok) {
-      BST_CUDA(cudaMalloc(&r.boxes, sizeof(RelBox) * hb.size()));
-      BST_CUDA(cudaMemcpy(r.boxes, hb.data(), sizeof(RelBox) * hb.size(), cudaMemcpyHostToDevice));
+      BST_CUDA(cudaMalloc(&r.legs, sizeof(RelLegTab) * hl.size()));
+      BST_CUDA(cudaMemcpy(r.legs, hl.data(), sizeof(RelLegTab) * hl.size(), cudaMemcpyHostToDevice));
     }
   }
   if (!ch.empty()) {
@@ -152,8 +152,8 @@ static void launch_rel(Ctx* ctx, const BatchRel& r, double* const* bases, double
                        double beta, cudaStream_t s) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  auto kern = r.boxes ? relayout_batch_kernel<true> : relayout_batch_kernel<false>;
-  kern<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.boxes, r.chunks, bases, mat, dir, alpha, beta, r.chunk);
+  auto kern = r.legs ? relayout_batch_kernel<true> : relayout_batch_kernel<false>;
+  kern<<<r.nchunks, kBatchThreads, 0, s>>>(r.tasks, r.legs, r.chunks, bases, mat, dir, alpha, beta, r.chunk);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

@@ -7,6 +7,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <initializer_list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -126,18 +127,27 @@ struct MatView {
 };
 
 struct RelBox;
+struct RelLegTab;
+struct Ctx;
 
-// A relayout ready to launch: tasks and chunk table on the device, and the
-// tasks' boxes (null in contract_noalloc's fixed scratch: a slower kernel).
+// A relayout ready to launch: tasks and chunk table on the device, with room
+// for the tasks' leg tables, which are made with an uploaded list, and before
+// its first launch for a contraction's views (prepare_legs; tensor-core
+// contractions never read theirs).  Without them (contract_noalloc's fixed
+// scratch, offsets past 32 bits) a slower kernel copies.
 struct DevRelayout {
+  void* mem = nullptr;  // holds tasks, legs and chunks
   RelTask* tasks = nullptr;
-  RelBox* boxes = nullptr;
+  RelLegTab* legs = nullptr;
   int2* chunks = nullptr;
+  RelBox* boxes = nullptr;  // set: copied by boxes through shared memory
   int nchunks = 0;
   int ntasks = 0;
-  bool transposes = false;  // copied by boxes through shared memory
+  bool narrow = false;      // offsets of 32 bits
+  bool legs_made = false;
   double elems = 0;
-  void upload(const std::vector<RelTask>& t);
+  void alloc(int64_t max_tasks, int64_t max_chunks);
+  void upload(Ctx* ctx, const std::vector<RelTask>& t);
   void free_all();
 };
 
@@ -294,6 +304,8 @@ int64_t plan_check(Ctx* ctx, Layout* A, Layout* B, const std::vector<int>& la, c
 
 // relayout.cu
 std::vector<int2> relayout_chunks(const std::vector<RelTask>& t);  // chunk table of a task list
+// makes the leg tables that are still missing (of up to three lists), on the device
+void prepare_legs(Ctx* ctx, std::initializer_list<DevRelayout*> rels, cudaStream_t s);
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir,
                      double alpha, double beta, cudaStream_t s, bool behind = false);
 // the gathers of both operands of a contraction, in one launch where they can be

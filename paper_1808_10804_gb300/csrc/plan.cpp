@@ -218,6 +218,7 @@ void run_contract(Ctx* ctx, ContractPlan* p, const double* a, const double* b, b
   // as a launch: blocks that start on the SMs that the copies leave first end
   // up two on one and none on another (an odd-sized corner of 0.33 GFLOP
   // 447 -> 509 us).
+  prepare_legs(ctx, {&p->ra, &p->rb, &p->rc}, s);
   launch_gathers(ctx, p->ra, a, Am, p->rb, b, Bm, s);
   launch_gemm_f64(ctx, p->g, Am, Bm, Cm, s, p->g.flops < 1.5e7 && (p->ra.nchunks || p->rb.nchunks));
   launch_relayout(ctx, p->rc, c, Cm, 1, alpha, beta, s, p->g.ntiles > 0);
@@ -267,7 +268,7 @@ DevRelayout* get_permute_plan(Ctx* ctx, Layout* src, const std::vector<int>& per
     if (n) tasks.push_back(t);
   }
   auto rp = std::make_unique<DevRelayout>();
-  if (ctx->device >= 0) rp->upload(tasks);
+  if (ctx->device >= 0) rp->upload(ctx, tasks);
   DevRelayout* raw = rp.get();
   ctx->rplans[key] = std::move(rp);
   return raw;
@@ -355,7 +356,7 @@ DevRelayout* get_fuse_plan(Ctx* ctx, Layout* src, const std::vector<int>& groups
     if (n) tasks.push_back(t);
   }
   auto rp = std::make_unique<DevRelayout>();
-  if (ctx->device >= 0) rp->upload(tasks);
+  if (ctx->device >= 0) rp->upload(ctx, tasks);
   DevRelayout* raw = rp.get();
   ctx->rplans[key] = std::move(rp);
   return raw;

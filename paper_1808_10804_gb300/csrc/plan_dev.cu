@@ -20,7 +20,6 @@
 #include <algorithm>
 
 #include "bst_internal.h"
-#include "relayout_dev.cuh"
 
 namespace bst {
 
@@ -312,26 +311,19 @@ static void build_view(Ctx* ctx, const Layout* L, const std::vector<int>& rowleg
   int* secidx = reinterpret_cast<int*>(ctot + v.cn);
   int* counts = secidx + v.cn;  // nsec, nchunks
   BST_CUDA(cudaMalloc(&out->secs, sizeof(DevSector) * std::max<long long>(v.cn, 1)));
-  BST_CUDA(cudaMalloc(&out->rel.tasks, sizeof(RelTask) * std::max<long long>(nb, 1)));
-  BST_CUDA(cudaMalloc(&out->rel.chunks, sizeof(int2) * std::max<long long>(nchunk_max, 1)));
-  const bool boxes = nb > 0 && L->nnz < (int64_t(1) << 31);  // (offsets of 32 bits)
-  if (boxes) BST_CUDA(cudaMalloc(&out->rel.boxes, sizeof(RelBox) * nb));
+  out->rel.alloc(nb, nchunk_max);
   plan_view_kernel<<<1, kPlanThreads, 0, s>>>(dl, v, t.q, t.d, t.sect, t.off, int(nb), rch, rext, roff, cch, cext,
                                               coff, rtot, ctot, secidx, out->secs, counts, out->rel.tasks,
                                               out->rel.chunks, counts + 1);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
-  if (boxes) {
-    rel_boxes_kernel<<<unsigned((nb + 127) / 128), 128, 0, s>>>(out->rel.tasks, int(nb), out->rel.boxes);
-    BST_CUDA(cudaGetLastError());
-    count_launch(ctx);
-  }
   int hc[2] = {0, 0};
   BST_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
   BST_CUDA(cudaStreamSynchronize(s));  // the tables above are freed on return
   out->nsec = hc[0];
   out->rel.ntasks = int(nb);
   out->rel.nchunks = hc[1];
+  out->rel.narrow = L->nnz < (int64_t(1) << 31);
   double e = 0;
   for (int64_t b = 0; b < nb; ++b) {
     int64_t n = 1;

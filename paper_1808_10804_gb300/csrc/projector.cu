@@ -99,7 +99,7 @@ static ProjView* get_projview(Ctx* ctx, Layout* L, const std::vector<int>& rows,
   }
   auto pv = std::make_shared<ProjView>();
   pv->mv = make_matview(L, rows, cols);
-  pv->rel.upload(pv->mv.tasks);
+  pv->rel.upload(ctx, pv->mv.tasks);
   ProjView* raw = pv.get();
   std::lock_guard<std::mutex> g(ctx->mu);
   ctx->projviews[key] = std::move(pv);
@@ -1272,6 +1272,7 @@ ProjResult svd_projector(Ctx* ctx, Layout* Rt, const double* rt, Layout* Rb, con
   // N = Rt^T Rb (rows: right cut of Rt, cols: right cut of Rb)
   double* At = (double*)ctx->buf("proj.A", sizeof(double) * std::max<int64_t>(pn->amat, 1), s);  // [beta x alpha]
   double* Bt = (double*)ctx->buf("proj.B", sizeof(double) * std::max<int64_t>(pn->bmat, 1), s);  // [beta' x alpha']
+  prepare_legs(ctx, {&pn->ra, &pn->rb}, s);
   launch_relayout(ctx, pn->ra, rt, At, 0, 1.0, 0.0, s);
   launch_relayout(ctx, pn->rb, rb, Bt, 0, 1.0, 0.0, s);
   double* Nm = (double*)ctx->buf("contract.Ckeep", sizeof(double) * std::max<int64_t>(pn->cmat, 1), s);
@@ -1649,7 +1650,7 @@ ProjResult su2_projector(Ctx* ctx, Layout* Rt, const double* rt, Layout* Rb, con
       if (n > 0) tasks.push_back(t);
     }
     auto r = std::make_unique<DevRelayout>();
-    r->upload(tasks);
+    r->upload(ctx, tasks);
     rel = r.get();
     std::lock_guard<std::mutex> g(ctx->mu);
     ctx->rplans[rkey] = std::move(r);
@@ -1883,12 +1884,12 @@ ProjResult su2_projector(Ctx* ctx, Layout* Rt, const double* rt, Layout* Rb, con
     auto& slotv = ctx->rplans["su2p/V/" + std::to_string(LV->id) + "/" + std::to_string(LN->id)];
     if (!slotv) {
       slotv = std::make_unique<DevRelayout>();
-      slotv->upload(tv);
+      slotv->upload(ctx, tv);
     }
     auto& slotu = ctx->rplans["su2p/U/" + std::to_string(LU->id) + "/" + std::to_string(LN->id)];
     if (!slotu) {
       slotu = std::make_unique<DevRelayout>();
-      slotu->upload(tu);
+      slotu->upload(ctx, tu);
     }
     launch_relayout(ctx, *slotv, vd, Vs, 1, 1.0, 0.0, s);
     launch_relayout(ctx, *slotu, ud, Us, 1, 1.0, 0.0, s);

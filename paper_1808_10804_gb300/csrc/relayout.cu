@@ -55,47 +55,82 @@ std::vector<int2> relayout_chunks(const std::vector<RelTask>& t) {
   return ch;
 }
 
-void DevRelayout::upload(const std::vector<RelTask>& t) {
+void DevRelayout::alloc(int64_t max_tasks, int64_t max_chunks) {
+  const size_t nt = size_t(std::max<int64_t>(max_tasks, 1)), nc = size_t(std::max<int64_t>(max_chunks, 1));
+  const size_t olegs = (sizeof(RelTask) * nt + 255) / 256 * 256, ochunks = olegs + sizeof(RelLegTab) * nt;
+  BST_CUDA(cudaMalloc(&mem, ochunks + sizeof(int2) * nc));
+  tasks = reinterpret_cast<RelTask*>(mem);
+  legs = reinterpret_cast<RelLegTab*>(static_cast<char*>(mem) + olegs);
+  chunks = reinterpret_cast<int2*>(static_cast<char*>(mem) + ochunks);
+}
+
+struct RelLists {
+  const RelTask* tasks[3];
+  RelLegTab* legs[3];
+  int n[3];
+};
+__global__ void rel_legs_kernel(RelLists l) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (i < l.n[r]) rel_make_legs(l.tasks[r][i], l.legs[r][i]);
+}
+
+// A stream that is being captured makes none (its graph keeps the kernel
+// without).
+void prepare_legs(Ctx* ctx, std::initializer_list<DevRelayout*> rels, cudaStream_t s) {
+  DevRelayout* todo[3];
+  int k = 0, longest = 0;
+  for (DevRelayout* r : rels)
+    if (r->narrow && !r->legs_made && r->ntasks > 0) todo[k++] = r, longest = std::max(longest, r->ntasks);
+  if (k == 0) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  BST_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return;
+  RelLists l{};
+  for (int i = 0; i < k; ++i) l.tasks[i] = todo[i]->tasks, l.legs[i] = todo[i]->legs, l.n[i] = todo[i]->ntasks;
+  rel_legs_kernel<<<dim3(unsigned((longest + 63) / 64), unsigned(k)), 64, 0, s>>>(l);
+  BST_CUDA(cudaGetLastError());
+  count_launch(ctx);
+  BST_CUDA(cudaStreamSynchronize(s));  // (the next launch may be on another stream)
+  for (int i = 0; i < k; ++i) todo[i]->legs_made = true;
+}
+
+void DevRelayout::upload(Ctx* ctx, const std::vector<RelTask>& t) {
   free_all();
   ntasks = int(t.size());
   elems = 0;
-  for (auto& x : t) elems += x.n;
-  std::vector<int2> ch = relayout_chunks(t);
-  if (ntasks) {
-    BST_CUDA(cudaMalloc(&tasks, sizeof(RelTask) * ntasks));
-    BST_CUDA(cudaMemcpy(tasks, t.data(), sizeof(RelTask) * ntasks, cudaMemcpyHostToDevice));
-    std::vector<RelBox> hb(ntasks);
-    bool ok = true;
-    for (int i = 0; i < ntasks; ++i) rel_make_box(t[i], hb[i]), ok = ok && hb[i].ntiles > 0;
+  narrow = true;
+  for (auto& x : t) elems += x.n, narrow = narrow && rel_narrow(x);
+  std::vector<int2> ch;
+  std::vector<RelBox> hb;
+  if (narrow && elems >= kBoxElems) {
+    hb.resize(ntasks);
     double across = 0;  // elements of blocks whose innermost leg is not the strided side's
-    for (int i = 0; i < ntasks; ++i)
+    for (int i = 0; i < ntasks; ++i) {
+      rel_make_box(t[i], hb[i]);
       if (hb[i].n > 1 && hb[i].leg[0].slot != 0) across += t[i].n;
-    transposes = ok && elems >= kBoxElems && across > 0.5 * elems;
-    if (transposes) {  // a CTA per box
-      ch.clear();
-      for (int i = 0; i < ntasks; ++i)
-        for (int k = 0; k < (t[i].n > 0 ? hb[i].ntiles : 0); ++k) ch.push_back(make_int2(i, k));
     }
-    if (ok) {
-      BST_CUDA(cudaMalloc(&boxes, sizeof(RelBox) * ntasks));
-      BST_CUDA(cudaMemcpy(boxes, hb.data(), sizeof(RelBox) * ntasks, cudaMemcpyHostToDevice));
-    }
+    if (!(across > 0.5 * elems)) hb.clear();
+  }
+  if (!hb.empty()) {  // a CTA per box
+    for (int i = 0; i < ntasks; ++i)
+      for (int k = 0; k < (t[i].n > 0 ? hb[i].ntiles : 0); ++k) ch.push_back(make_int2(i, k));
+    BST_CUDA(cudaMalloc(&boxes, sizeof(RelBox) * ntasks));
+    BST_CUDA(cudaMemcpy(boxes, hb.data(), sizeof(RelBox) * ntasks, cudaMemcpyHostToDevice));
+  } else {
+    ch = relayout_chunks(t);
   }
   nchunks = int(ch.size());
-  if (nchunks) {
-    BST_CUDA(cudaMalloc(&chunks, sizeof(int2) * nchunks));
-    BST_CUDA(cudaMemcpy(chunks, ch.data(), sizeof(int2) * nchunks, cudaMemcpyHostToDevice));
-  }
+  if (nchunks == 0) return;
+  alloc(ntasks, nchunks);
+  BST_CUDA(cudaMemcpy(tasks, t.data(), sizeof(RelTask) * ntasks, cudaMemcpyHostToDevice));
+  BST_CUDA(cudaMemcpy(chunks, ch.data(), sizeof(int2) * nchunks, cudaMemcpyHostToDevice));
+  if (!boxes) prepare_legs(ctx, {this}, 0);
 }
 
 void DevRelayout::free_all() {
-  if (tasks) cudaFree(tasks);
+  if (mem) cudaFree(mem);
   if (boxes) cudaFree(boxes);
-  if (chunks) cudaFree(chunks);
-  tasks = nullptr;
-  boxes = nullptr;
-  chunks = nullptr;
-  ntasks = nchunks = 0;
+  *this = DevRelayout{};
 }
 
 void* DevBuf::get(size_t need, cudaStream_t s) {
@@ -135,7 +170,7 @@ __global__ void __launch_bounds__(kRelThreads) relayout_kernel(const RelTask* __
 }
 
 __global__ void __launch_bounds__(kRelThreads) relayout_legs_kernel(const RelTask* __restrict__ tasks,
-                                                                    const RelBox* __restrict__ boxes,
+                                                                    const RelLegTab* __restrict__ legs,
                                                                     const int2* __restrict__ chunks, double* blk,
                                                                     double* mat, int dir, double alpha, double beta) {
   __shared__ RelLegs sh;
@@ -143,13 +178,13 @@ __global__ void __launch_bounds__(kRelThreads) relayout_legs_kernel(const RelTas
   const int2 c = chunks[blockIdx.x];
   const int end = min(tasks[c.x].n, c.y + kChunk);
   grid_wait();
-  relayout_legs<kRelThreads>(sh, boxes[c.x], c.y, end, blk, mat, dir, alpha, beta);
+  relayout_legs<kRelThreads>(sh, legs[c.x], c.y, end, blk, mat, dir, alpha, beta);
 }
 
 // Both operands' gathers of a contraction in one launch.
 struct RelPart {
   const RelTask* tasks;
-  const RelBox* boxes;
+  const RelLegTab* legs;
   const int2* chunks;
   double *blk, *mat;
 };
@@ -159,7 +194,7 @@ __global__ void __launch_bounds__(kRelThreads) relayout_pair_kernel(RelPart a, R
   const bool first = int(blockIdx.x) < na;
   const RelPart p = first ? a : b;
   const int2 c = p.chunks[int(blockIdx.x) - (first ? 0 : na)];
-  relayout_legs<kRelThreads>(sh, p.boxes[c.x], c.y, min(p.tasks[c.x].n, c.y + kChunk), p.blk, p.mat, 0, 1.0, 0.0);
+  relayout_legs<kRelThreads>(sh, p.legs[c.x], c.y, min(p.tasks[c.x].n, c.y + kChunk), p.blk, p.mat, 0, 1.0, 0.0);
 }
 
 __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(const RelBox* __restrict__ boxes,
@@ -169,11 +204,6 @@ __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(con
   __shared__ RelShared sh;
   const int2 c = tiles[blockIdx.x];
   relayout_box<kRelThreads, kBoxU>(sh, boxes[c.x], c.y, blk, mat, dir, alpha, beta);
-}
-
-__global__ void rel_boxes_kernel(const RelTask* tasks, int n, RelBox* boxes) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) rel_make_box(tasks[i], boxes[i]);
 }
 
 // Boxes only for large copies between different innermost legs: the
@@ -186,12 +216,12 @@ void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* 
                      double beta, cudaStream_t s, bool behind) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  if (r.boxes && r.transposes)
+  if (r.boxes)
     relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                           beta);
-  else if (r.boxes)
+  else if (r.legs_made)
     launch_behind(behind, relayout_legs_kernel, dim3(unsigned(r.nchunks)), kRelThreads, 0, s, (const RelTask*)r.tasks,
-                  (const RelBox*)r.boxes, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta);
+                  (const RelLegTab*)r.legs, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta);
   else
     relayout_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.tasks, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
                                                       beta);
@@ -201,15 +231,15 @@ void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* 
 
 void launch_gathers(Ctx* ctx, const DevRelayout& ra, const double* a, double* Am, const DevRelayout& rb,
                     const double* b, double* Bm, cudaStream_t s) {
-  if (ra.nchunks == 0 || rb.nchunks == 0 || !ra.boxes || !rb.boxes || ra.transposes || rb.transposes) {
+  if (ra.nchunks == 0 || rb.nchunks == 0 || !ra.legs_made || !rb.legs_made) {
     launch_relayout(ctx, ra, a, Am, 0, 1.0, 0.0, s);
     launch_relayout(ctx, rb, b, Bm, 0, 1.0, 0.0, s);
     return;
   }
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * (ra.elems + rb.elems));
   relayout_pair_kernel<<<ra.nchunks + rb.nchunks, kRelThreads, 0, s>>>(
-      RelPart{ra.tasks, ra.boxes, ra.chunks, const_cast<double*>(a), Am},
-      RelPart{rb.tasks, rb.boxes, rb.chunks, const_cast<double*>(b), Bm}, ra.nchunks);
+      RelPart{ra.tasks, ra.legs, ra.chunks, const_cast<double*>(a), Am},
+      RelPart{rb.tasks, rb.legs, rb.chunks, const_cast<double*>(b), Bm}, ra.nchunks);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

@@ -137,7 +137,6 @@ __host__ __device__ constexpr int rel_pos(int i) { return i + (i >> 4); }
 struct alignas(16) RelBoxLeg {
   FastDiv outer, nt;   // boxes along the legs outside this one; along this one
   FastDiv full, last;  // extent in a box, in the last box along the leg
-  FastDiv whole;       // extent of the leg
   int32_t lin;         // stride inside a box, row-major in the contiguous side's order
   int32_t slot;        // its place (innermost first) in the strided side's order
   int32_t sb, sm;      // element strides of the two sides
@@ -151,10 +150,11 @@ struct alignas(16) RelBox {
   RelBoxLeg leg[kMaxRank];  // contiguous side's order, innermost first
 };
 
-__host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
+// The legs of a task of more than one element, contiguous side's order,
+// innermost first (those that follow each other on both sides as one):
+// extents and strides of the contiguous and the strided side; their number.
+__host__ __device__ inline int rel_task_legs(const RelTask& t, int* L, long long* sb, long long* sm) {
   int n = 0;
-  int L[kMaxRank];
-  long long sb[kMaxRank], sm[kMaxRank], inm[kMaxRank];
   long long bs = 1;
   for (int k = t.rank - 1; k >= 0; --k) {
     if (t.shape[k] > 1) {
@@ -169,6 +169,13 @@ __host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
     }
     bs *= t.shape[k];
   }
+  return n;
+}
+
+__host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
+  int L[kMaxRank];
+  long long sb[kMaxRank], sm[kMaxRank], inm[kMaxRank];
+  const int n = rel_task_legs(t, L, sb, sm);
   b.blk_off = t.blk_off;
   b.mat_base = t.mat_base;
   b.n = n;
@@ -188,7 +195,6 @@ __host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
     b.leg[j].sb = int32_t(sb[j]);
     b.leg[j].sm = int32_t(sm[j]);
     b.leg[j].run = (sb[j] < 16 ? 1 : 0) | (inm[j] < 16 ? 2 : 0);
-    b.leg[j].whole.init(uint32_t(L[j]));
     b.nrun[0] += sb[j] < 16;
     b.nrun[1] += inm[j] < 16;
   }
@@ -249,10 +255,6 @@ __host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
 struct alignas(16) RelLeg {
   uint32_t d, m, l;  // extent and its FastDiv
   int32_t lin, st, pad[3];
-};
-
-struct RelLegs {
-  int4 leg[kMaxRank];  // extent and its FastDiv, stride of the strided side
 };
 
 struct RelShared {
@@ -378,17 +380,48 @@ __device__ __forceinline__ void relayout_box(RelShared& sh, const RelBox& b, int
   });
 }
 
+// ---- copies by leg tables --------------------------------------------------------
+
+// A task's legs with their divisions prepared: extent, its FastDiv's m and l,
+// stride of the strided side.
+struct alignas(16) RelLegTab {
+  long long blk_off, mat_base;
+  int32_t n, pad[3];
+  int4 leg[kMaxRank];  // contiguous side's order, innermost first
+};
+
+__host__ __device__ inline void rel_make_legs(const RelTask& t, RelLegTab& b) {
+  int L[kMaxRank];
+  long long sb[kMaxRank], sm[kMaxRank];
+  b.blk_off = t.blk_off;
+  b.mat_base = t.mat_base;
+  b.n = rel_task_legs(t, L, sb, sm);
+  for (int j = 0; j < b.n; ++j) {
+    FastDiv f;
+    f.init(uint32_t(L[j]));
+    b.leg[j] = make_int4(int(f.d), int(f.m), int(f.l), int(sm[j]));
+  }
+}
+
+// Whether a task's offsets on the strided side fit 32 bits.
+inline bool rel_narrow(const RelTask& t) {
+  long long span = 0;
+  for (int i = 0; i < t.rank; ++i) span += (t.shape[i] - 1) * (long long)t.mstride[i];
+  return span < (1ll << 31);
+}
+
+struct RelLegs {
+  int4 leg[kMaxRank];
+};
+
 // Elements [begin, end) of one task by the leg table (32-bit offsets), eight
 // a thread: a chunk of 2048 in one pass, the loads of all before the stores.
 template <int kThreads>
-__device__ __forceinline__ void relayout_legs(RelLegs& sh, const RelBox& b, int begin, int end, double* blk, double* mat,
-                                              int dir, double alpha, double beta) {
+__device__ __forceinline__ void relayout_legs(RelLegs& sh, const RelLegTab& b, int begin, int end, double* blk,
+                                              double* mat, int dir, double alpha, double beta) {
   constexpr int kU = 8;
   const int n = b.n;
-  if (int(threadIdx.x) < n) {
-    const RelBoxLeg& g = b.leg[threadIdx.x];
-    sh.leg[threadIdx.x] = make_int4(int(g.whole.d), int(g.whole.m), int(g.whole.l), g.sm);
-  }
+  if (int(threadIdx.x) < n) sh.leg[threadIdx.x] = b.leg[threadIdx.x];
   blk += b.blk_off;
   mat += b.mat_base;
   __syncthreads();
@@ -437,8 +470,5 @@ __device__ __forceinline__ void relayout_legs(RelLegs& sh, const RelBox& b, int 
     }
   }
 }
-
-// box list of a task list, one thread a task
-__global__ void rel_boxes_kernel(const RelTask* tasks, int n, RelBox* boxes);
 
 }  // namespace bst

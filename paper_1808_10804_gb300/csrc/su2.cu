@@ -658,8 +658,8 @@ static Su2Plan* build_su2_plan(Ctx* ctx, Layout* A, Layout* B, const std::vector
 
   // device side (a host-only context keeps the host plan only)
   if (ctx->device < 0) return plan.release();
-  p->ra.upload(ta);
-  p->rb.upload(tb);
+  p->ra.upload(ctx, ta);
+  p->rb.upload(ctx, tb);
   p->g.upload(p->probs, kF64TileM, kF64TileN);
   auto up = [](auto** dst, const auto& v) {
     using T = typename std::remove_reference<decltype(v)>::type::value_type;

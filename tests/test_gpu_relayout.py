@@ -50,3 +50,43 @@ def test_permute_box_edges(bst, shape, perm):
     # (blocks in lexicographic order of their charges, 0 before 2 on every leg)
     assert np.array_equal(y, np.concatenate(blocks))
     ctx.close()
+
+
+def test_tables_made_where_they_are_read(bst):
+    """The first tensor-core contraction of new layouts launches the three
+    views of the planner, its pack and its product, and nothing for copies
+    that only FP64 makes; FP64 calls after it are right from the first on, by
+    the same bits on any stream and in a captured graph."""
+    ctx = bst.Context(0)
+    rng = np.random.default_rng(3)
+    legs = [bst.Leg(1, (-1, 0, 1), (3, 7, 4)), bst.Leg(-1, (-1, 0, 1), (5, 2, 6)), bst.Leg(-1, (0, 1), (9, 8))]
+    A = ctx.layout(legs)
+    B = ctx.layout([bst.Leg(-leg.flow, leg.charges, leg.degs) for leg in legs])
+    a, b = (torch.tensor(rng.standard_normal(L.nnz), device="cuda:0") for L in (A, B))
+    n0 = ctx.launches
+    Cl, c = ctx.contract(A, a, B, b, (2,), (2,), prec="ozaki")
+    ctx.sync()
+    assert ctx.launches - n0 == 5  # (the planner's views, pack, product)
+    other = torch.cuda.Stream()
+    other.wait_stream(torch.cuda.current_stream())
+    first = ctx.contract(A, a, B, b, (2,), (2,), Cl=Cl, stream=other)[1]
+    other.synchronize()
+    again = ctx.contract(A, a, B, b, (2,), (2,), Cl=Cl)[1]
+    ctx.sync()
+    assert torch.equal(first, again)
+    assert (first - c).abs().max() <= 1e-10
+    # a graph of an FP64 call whose layouts have only seen tensor-core calls
+    ctx.contract(A, a, B, b, (0,), (0,))  # (workspace for the next one)
+    Cg, cg = ctx.contract(A, a, B, b, (1, 2), (1, 2), prec="ozaki")
+    out = torch.zeros_like(cg)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        ctx.contract(A, a, B, b, (1, 2), (1, 2), Cl=Cg, c=out, stream=s)
+    g.replay()
+    torch.cuda.synchronize()
+    ref = ctx.contract(A, a, B, b, (1, 2), (1, 2), Cl=Cg)[1]
+    ctx.sync()
+    assert torch.equal(out, ref)
+    ctx.close()
