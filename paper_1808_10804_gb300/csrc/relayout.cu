@@ -103,13 +103,18 @@ void DevRelayout::upload(Ctx* ctx, const std::vector<RelTask>& t) {
   std::vector<int2> ch;
   std::vector<RelBox> hb;
   if (narrow && elems >= kBoxElems) {
-    hb.resize(ntasks);
-    double across = 0;  // elements of blocks whose innermost leg is not the strided side's
-    for (int i = 0; i < ntasks; ++i) {
-      rel_make_box(t[i], hb[i]);
-      if (hb[i].n > 1 && hb[i].leg[0].slot != 0) across += t[i].n;
+    // a sample of the blocks decides: up to 64, by their elements
+    double in = 0, of = 0;
+    for (int i = 0; i < ntasks; i += (ntasks + 63) / 64) {
+      RelBox b;
+      rel_make_box(t[i], b);
+      of += t[i].n;
+      if (rel_box_pays(t[i], b)) in += t[i].n;
     }
-    if (!(across > 0.5 * elems)) hb.clear();
+    if (in > 0.5 * of) {
+      hb.resize(ntasks);
+      for (int i = 0; i < ntasks; ++i) rel_make_box(t[i], hb[i]);
+    }
   }
   if (!hb.empty()) {  // a CTA per box
     for (int i = 0; i < ntasks; ++i)
@@ -206,11 +211,22 @@ __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(con
   relayout_box<kRelThreads, kBoxU>(sh, boxes[c.x], c.y, blk, mat, dir, alpha, beta);
 }
 
-// Boxes only for large copies between different innermost legs: the
-// scattered side of a smaller one is merged in the L2 cache, and a box pays
-// for its tables and two more barriers (a D = 4, chi = 64 permutation takes
-// 14 us by boxes, 10 by legs; the odd-sized FP64 corner's copies 89 and 32);
-// with the same innermost leg on both sides the direct copy reaches 5.1 TB/s.
+// Boxes only where rel_box_pays.  A straight copy reaches 5.8 TB/s when a
+// warp's elements stay on a few lines of the strided side, and what it
+// scatters is merged in the L2 cache while both sides fit there; a box pays
+// for its tables and two more barriers, and more when few runs, or a small
+// block, leave its threads idle.  Microseconds straight / by boxes:
+//   by the lines of a warp, blocks (n, a, b) -> (n, b, a) of 40 M elements:
+//     b a = 16 x 2 (2 lines) 107 / 132, 5 x 16 (5) 111 / 186, 6 x 16 (6)
+//     111 / 148, 16 x 16 (16) 188 / 132; rank 6, legs of 5 to 9, 15.5 M
+//     elements: 7 or 8 lines 62 / 83, 32 lines 135 / 75 and 91 / 81;
+//   by the runs, (m, n) -> (n, m): 5 M elements, m = 2 (4 lines) 29 / 50, 5
+//     (10) 42 / 48, 12 (24, one run) 49 / 41, 16 (32, 16 runs) 55 / 31; 40 M
+//     elements 240 / 321, 432 / 299, 603 / 244, 722 / 179;
+//   by the size, 18.8 M elements in blocks of 900: 145 / 136, 5.1 M in blocks
+//     of 73 k 43 / 30, 60 M in blocks of 0.7 M 429 / 221.
+// Below 4 M elements: a D = 4, chi = 64 permutation takes 14 us by boxes, 10
+// straight, the odd-sized FP64 corner's copies 89 and 32.
 // behind: the previous kernel of the stream is this call's, launch_behind.
 void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* mat, int dir, double alpha,
                      double beta, cudaStream_t s, bool behind) {

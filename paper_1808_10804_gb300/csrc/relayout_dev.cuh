@@ -1,6 +1,8 @@
 // Device helpers of the relayout kernels (block <-> strided region copies).
 #pragma once
 
+#include <algorithm>
+
 #include "bst_internal.h"
 
 namespace bst {
@@ -251,6 +253,36 @@ __host__ __device__ inline void rel_make_box(const RelTask& t, RelBox& b) {
   b.ntiles = int32_t(inner);
 }
 
+// Whether a task is copied faster by boxes than straight, 2048 elements a CTA
+// (see launch_relayout): a warp's 32 elements lie on 12 or more 128-byte lines
+// of the strided side, and the box has at least eight runs on either side for
+// the threads, or the elements lie on 24 or more sectors of 32 bytes and the
+// block is so large that the parts of a sector no longer meet in the cache.
+// b: its box.
+inline bool rel_box_pays(const RelTask& t, const RelBox& b) {
+  if (t.n < 1024 || b.n < 2 || b.leg[0].slot == 0) return false;
+  int L[kMaxRank], at[kMaxRank] = {}, count[2] = {0, 0};
+  long long sb[kMaxRank], sm[kMaxRank], seen[2][32], off = 0;
+  const int n = rel_task_legs(t, L, sb, sm);
+  for (int e = 0; e < 32; ++e) {
+    for (int u = 0; u < 2; ++u) {  // lines, sectors
+      const long long at_u = off / (u ? 4 : 16);
+      if (std::find(seen[u], seen[u] + count[u], at_u) == seen[u] + count[u]) seen[u][count[u]++] = at_u;
+    }
+    for (int j = 0; j < n; ++j) {
+      off += sm[j];
+      if (++at[j] < L[j]) break;
+      off -= sm[j] * L[j];
+      at[j] = 0;
+    }
+  }
+  int rows[2] = {1, 1};
+  for (int j = 0; j < n; ++j)
+    for (int side = 0; side < 2; ++side)
+      if (!(b.leg[j].run >> side & 1)) rows[side] *= int(b.leg[j].full.d);
+  return count[0] >= 12 && ((rows[0] >= 8 && rows[1] >= 8) || (count[1] >= 24 && t.n >= 1 << 24));
+}
+
 // A leg of the box at hand, on one side's list.
 struct alignas(16) RelLeg {
   uint32_t d, m, l;  // extent and its FastDiv
@@ -329,7 +361,8 @@ __device__ __forceinline__ void relayout_box(RelShared& sh, const RelBox& b, int
   // one side's runs, threads along a run, kU runs at a time
   auto each = [&](int side, auto&& body) {
     const int run = sh.run[side], rows = sh.rows[side];
-    const int sl = run > 32 ? 6 : run > 16 ? 5 : run > 8 ? 4 : run > 4 ? 3 : 2;
+    int sl = run > 32 ? 6 : run > 16 ? 5 : run > 8 ? 4 : run > 4 ? 3 : 2;
+    while ((kThreads >> sl) > rows && (1 << sl) < run) ++sl;  // (few long runs: all threads along them)
     const int step = kThreads >> sl;
     for (int x = int(threadIdx.x) & ((1 << sl) - 1); x < run; x += 1 << sl) {
       const int2 t = place(side, 0, b.nrun[side], x);

@@ -26,6 +26,10 @@ def bst():
     ((2111, 2029), (1, 0)), ((4200, 1001), (1, 0)), ((3, 1400001), (1, 0)), ((1400001, 3), (1, 0)),
     ((17, 65, 63, 61), (2, 0, 3, 1)), ((2, 129, 5, 255, 13), (4, 2, 0, 3, 1)), ((19, 300, 31, 29), (0, 2, 1, 3)),
     ((2, 3, 5, 7, 11, 13, 14, 11), (7, 5, 3, 1, 6, 4, 2, 0)), ((41, 40, 50, 51), (1, 0, 3, 2)),
+    # on either side of the rules that choose between straight copies and boxes
+    ((2, 2100001), (1, 0)), ((2100001, 2), (1, 0)), ((7, 2400001), (1, 0)), ((13, 1300003), (1, 0)),
+    ((13, 1200000), (1, 0)), ((2, 10, 900, 250), (2, 0, 3, 1)), ((80, 70, 60, 13), (3, 0, 1, 2)),
+    ((1000, 41, 3, 41), (0, 3, 2, 1)), ((300, 300, 6, 9), (0, 1, 3, 2)),
 ])
 def test_permute_box_edges(bst, shape, perm):
     ctx = bst.Context(0)
@@ -89,4 +93,26 @@ def test_tables_made_where_they_are_read(bst):
     ref = ctx.contract(A, a, B, b, (1, 2), (1, 2), Cl=Cg)[1]
     ctx.sync()
     assert torch.equal(out, ref)
+    ctx.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 8000001), (8000001, 2), (5, 1600001), (1600001, 11)])
+def test_thin_transpositions_keep_up(bst, shape):
+    """Transposing a thin matrix takes no longer than a square one of the same
+    size, with a factor of two to spare (boxes of few runs took three times
+    as long)."""
+    ctx = bst.Context(0)
+
+    def time(sh):
+        L = ctx.layout([bst.Leg(1, (0,), (sh[0],)), bst.Leg(-1, (0,), (sh[1],))])
+        x = torch.zeros(L.nnz, dtype=torch.float64, device="cuda:0")
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(14)]
+        ctx.permute(L, x, (1, 0))
+        for i in range(7):
+            ev[2 * i].record()
+            ctx.permute(L, x, (1, 0))
+            ev[2 * i + 1].record()
+        torch.cuda.synchronize()
+        return sorted(a.elapsed_time(b) for a, b in zip(ev[::2], ev[1::2]))[3] / L.nnz
+    assert time(shape) <= 2 * time((4001, 4003))
     ctx.close()
