@@ -36,7 +36,7 @@ struct BatchTask {
 
 struct BatchRel {
   BatchTask* tasks = nullptr;
-  RelLegTab* legs = nullptr;
+  RelLegTab* legs = nullptr;  // null: offsets past 32 bits
   int2* chunks = nullptr;
   int nchunks = 0;
   int chunk = 2048;  // elements per CTA
@@ -59,6 +59,11 @@ struct BatchPlan {
   // the second half of the pointer table), the FP64 path's scatter
   BatchRel rab, rc;
   std::vector<GemmProb> probs;
+  double flops = 0;
+  // What FP64 calls alone use (rab, rc, g and the sector matrices) is made
+  // before the first of them: beside a tensor-core batch it held 16 bytes an
+  // operand element and as many an output element for nothing.
+  bool f64_made = false;
   DevGemm g;
   // schedule chosen by the autotuner (defaults until tuned)
   bool tuned_rel = false;
@@ -120,32 +125,67 @@ __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const Bat
     relayout_range<kBatchThreads>(bt.t, c.y, end, bases[bt.src], mat, dir, alpha, beta);
 }
 
-// (Re)build the chunk table of a relayout for `chunk` elements per CTA.
-static void upload_rel(BatchRel& r, int chunk) {
-  r.free_all();
+// Allocations and copies beside whatever stream is being captured: on a
+// stream of their own, finished when an upload returns.
+struct Aside {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaStream_t s = nullptr;
+  Aside() {
+    BST_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      throw Error(BST_E_CUDA, "cannot create a stream");
+    }
+  }
+  ~Aside() {
+    cudaStreamDestroy(s);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  template <class T>
+  void put(T** dst, const std::vector<T>& v) {
+    if (v.empty()) return;
+    BST_CUDA(cudaMalloc(dst, sizeof(T) * v.size()));
+    BST_CUDA(cudaMemcpyAsync(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s));
+    BST_CUDA(cudaStreamSynchronize(s));
+  }
+};
+
+// (Re)build the chunk table of a relayout for `chunk` elements per CTA; the
+// other tables with the first one.
+static void upload_rel(Aside& up, BatchRel& r, int chunk) {
+  if (!r.tasks) {
+    std::vector<RelLegTab> hl(r.host.size());
+    bool narrow = true;
+    for (size_t i = 0; i < hl.size(); ++i)
+      rel_make_legs(r.host[i].t, hl[i]), narrow = narrow && rel_narrow(r.host[i].t);
+    if (narrow) up.put(&r.legs, hl);
+    up.put(&r.tasks, r.host);
+  }
   r.chunk = chunk;
-  std::vector<int2> ch;
   r.elems = 0;
+  std::vector<int2> ch;
   for (int i = 0; i < int(r.host.size()); ++i) {
     r.elems += r.host[i].t.n;
     for (int s = 0; s < r.host[i].t.n; s += chunk) ch.push_back(make_int2(i, s));
   }
   r.nchunks = int(ch.size());
-  if (!r.host.empty()) {
-    BST_CUDA(cudaMalloc(&r.tasks, sizeof(BatchTask) * r.host.size()));
-    BST_CUDA(cudaMemcpy(r.tasks, r.host.data(), sizeof(BatchTask) * r.host.size(), cudaMemcpyHostToDevice));
-    std::vector<RelLegTab> hl(r.host.size());
-    bool ok = true;  // (no tables past 32-bit offsets)
-    for (size_t i = 0; i < hl.size(); ++i) rel_make_legs(r.host[i].t, hl[i]), ok = ok && rel_narrow(r.host[i].t);
-    if (ok) {
-      BST_CUDA(cudaMalloc(&r.legs, sizeof(RelLegTab) * hl.size()));
-      BST_CUDA(cudaMemcpy(r.legs, hl.data(), sizeof(RelLegTab) * hl.size(), cudaMemcpyHostToDevice));
-    }
-  }
-  if (!ch.empty()) {
-    BST_CUDA(cudaMalloc(&r.chunks, sizeof(int2) * ch.size()));
-    BST_CUDA(cudaMemcpy(r.chunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice));
-  }
+  cudaFree(r.chunks);
+  r.chunks = nullptr;
+  up.put(&r.chunks, ch);
+}
+
+static void make_f64(BatchPlan* bp) {
+  if (bp->f64_made) return;
+  Aside up;
+  bp->rab.free_all();  // (of a call that ran out of memory here)
+  bp->rc.free_all();
+  upload_rel(up, bp->rab, 2048);
+  upload_rel(up, bp->rc, 2048);
+  bp->g.upload(bp->probs, kF64TileM, kF64TileN, 0, up.s);
+  if (!bp->Am) BST_CUDA(cudaMalloc(&bp->Am, sizeof(double) * std::max<int64_t>(bp->amat + bp->bmat, 1)));
+  bp->Bm = bp->Am + bp->amat;
+  if (!bp->Cm) BST_CUDA(cudaMalloc(&bp->Cm, sizeof(double) * std::max<int64_t>(bp->cmat, 1)));
+  bp->f64_made = true;
 }
 
 static void launch_rel(Ctx* ctx, const BatchRel& r, double* const* bases, double* mat, int dir, double alpha,
@@ -206,8 +246,9 @@ static void autotune(Ctx* ctx, BatchPlan* bp, double* const* bases, size_t n, bs
   if (!bp->tuned_rel && prec == BST_FP64) {
     float best = 1e30f;
     int bc = 2048;
+    Aside up;
     for (int c : kChunkChoices) {
-      upload_rel(bp->rab, c);
+      upload_rel(up, bp->rab, c);
       const float t = time_ms(s, 3, [&] {
         launch_rel(ctx, bp->rab, bases, bp->Am, 0, 1.0, 0.0, s);
       });
@@ -215,8 +256,8 @@ static void autotune(Ctx* ctx, BatchPlan* bp, double* const* bases, size_t n, bs
       ctx->tune_log += line;
       if (t < best) best = t, bc = c;
     }
-    upload_rel(bp->rab, bc);
-    upload_rel(bp->rc, bc);
+    upload_rel(up, bp->rab, bc);
+    upload_rel(up, bp->rc, bc);
     snprintf(line, sizeof(line), "batch %p relayout chunk chosen %d\n", (void*)bp, bc);
     ctx->tune_log += line;
     bp->tuned_rel = true;
@@ -323,12 +364,7 @@ static BatchPlan* get_batch_plan(Ctx* ctx, const std::vector<Layout*>& A, const 
     t.t.mat_base += bp->amat;
     bp->rab.host.push_back(t);
   }
-  upload_rel(bp->rab, 2048);
-  upload_rel(bp->rc, 2048);
-  bp->g.upload(bp->probs, kF64TileM, kF64TileN);
-  BST_CUDA(cudaMalloc(&bp->Am, sizeof(double) * std::max<int64_t>(bp->amat + bp->bmat, 1)));
-  bp->Bm = bp->Am + bp->amat;
-  BST_CUDA(cudaMalloc(&bp->Cm, sizeof(double) * std::max<int64_t>(bp->cmat, 1)));
+  for (auto& g : bp->probs) bp->flops += 2.0 * double(g.M) * g.N * g.K;
   BatchPlan* raw = bp.get();
   std::lock_guard<std::mutex> g(ctx->mu);
   ctx->bplans[key] = std::move(bp);
@@ -363,8 +399,9 @@ void contract_batched(Ctx* ctx, const std::vector<Layout*>& A, const std::vector
   }
   double** bases = it->second.bases;
   const std::string tag = "batch/" + std::to_string(uintptr_t(bp));
+  if (prec == BST_FP64) make_f64(bp);
   if (ctx->autotune) autotune(ctx, bp, bases, n, prec, tag, s, C);
-  ctx->work_flops += bp->g.flops;
+  ctx->work_flops += bp->flops;
   if (prec == BST_FP64) {
     launch_rel(ctx, bp->rab, bases, bp->Am, 0, 1.0, 0.0, s);
     launch_gemm_f64(ctx, bp->g, bp->Am, bp->Bm, bp->Cm, s);

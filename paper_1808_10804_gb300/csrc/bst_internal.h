@@ -182,7 +182,8 @@ struct DevGemm {
   int64_t wtot = 0;          // sum of M*N
   int maxK = 0;
   // order 0: problem order; 1: tiles of the longest-K problems first
-  void upload(const std::vector<GemmProb>& p, int tm, int tn, int order = 0);
+  // (s: stream of the copies, which have ended on return)
+  void upload(const std::vector<GemmProb>& p, int tm, int tn, int order = 0, cudaStream_t s = 0);
   void free_all();
 };
 

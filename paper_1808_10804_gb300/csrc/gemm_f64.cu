@@ -15,8 +15,11 @@ const int kF64TileN = 64;
 constexpr int kBK = 16;
 constexpr int kPad = 2;
 
-void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order) {
+void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order, cudaStream_t s) {
   free_all();
+  auto copy = [&](void* dst, const void* src, size_t n) {
+    BST_CUDA(cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, s));
+  };
   nprobs = int(p.size());
   flops = 0;
   for (auto& x : p) flops += 2.0 * double(x.M) * x.N * x.K;
@@ -52,18 +55,19 @@ void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order) 
   }
   if (nprobs) {
     BST_CUDA(cudaMalloc(&probs, sizeof(GemmProb) * nprobs));
-    BST_CUDA(cudaMemcpy(probs, p.data(), sizeof(GemmProb) * nprobs, cudaMemcpyHostToDevice));
+    copy(probs, p.data(), sizeof(GemmProb) * nprobs);
   }
   if (nprobs) {
     BST_CUDA(cudaMalloc(&w_off, sizeof(int64_t) * nprobs));
-    BST_CUDA(cudaMemcpy(w_off, wo.data(), sizeof(int64_t) * nprobs, cudaMemcpyHostToDevice));
+    copy(w_off, wo.data(), sizeof(int64_t) * nprobs);
   }
   if (ntiles) {
     BST_CUDA(cudaMalloc(&tile_prob, sizeof(int32_t) * ntiles));
     BST_CUDA(cudaMalloc(&tile_idx, sizeof(int32_t) * ntiles));
-    BST_CUDA(cudaMemcpy(tile_prob, tp.data(), sizeof(int32_t) * ntiles, cudaMemcpyHostToDevice));
-    BST_CUDA(cudaMemcpy(tile_idx, ti.data(), sizeof(int32_t) * ntiles, cudaMemcpyHostToDevice));
+    copy(tile_prob, tp.data(), sizeof(int32_t) * ntiles);
+    copy(tile_idx, ti.data(), sizeof(int32_t) * ntiles);
   }
+  BST_CUDA(cudaStreamSynchronize(s));
 }
 
 void DevGemm::free_all() {

@@ -1422,6 +1422,7 @@ struct OzakiPlan {
   // packed operands (pack_split_kernel reads the tensors' blocks; no
   // sector matrices, no separate split)
   bool packed = false;
+  void* d_pack = nullptr;  // holds the following tables
   oz::PackGroup *d_pgA = nullptr, *d_pgB = nullptr;
   oz::PackSeg *d_psA = nullptr, *d_psB = nullptr;
   int2 *d_pcA = nullptr, *d_pcB = nullptr;
@@ -1429,12 +1430,7 @@ struct OzakiPlan {
   bool pack_apart = false;                 // one launch per operand
   int pack_cluster = 1;                    // CTAs that share the k of a block of rows
   ~OzakiPlan() {
-    cudaFree(d_pgA);
-    cudaFree(d_pgB);
-    cudaFree(d_psA);
-    cudaFree(d_psB);
-    cudaFree(d_pcA);
-    cudaFree(d_pcB);
+    cudaFree(d_pack);
     cudaFree(d_ca);
     cudaFree(d_cb);
     cudaFree(d_rowtab);
@@ -1636,8 +1632,10 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
                      [&](const oz::Tile& x, const oz::Tile& y) { return hp[x.prob].K > hp[y.prob].K; });
   P->nprobs = int(hp.size());
   P->ntiles = int(ht.size());
-  // CTAs of the split: eight contiguous rows each, or a cluster per 32
+  // CTAs of the split (a scattering plan's operands are packed, see
+  // attach_pack): split_cta_rows contiguous rows each, or a cluster per 32
   // interleaved rows (128 k per CTA and pass: one pass up to K = 1024)
+  if (sc) sa.clear(), sb.clear();
   int kcol = 0;
   for (auto* v : {&sa, &sb})
     for (auto& t : *v)
@@ -1881,18 +1879,27 @@ static void attach_pack(OzakiPlan* P, PackTables& ta, PackTables& tb) {
   while (P->pack_cluster > 1 && (ta.blocks + tb.blocks) * P->pack_cluster > 4 * num_sms()) P->pack_cluster /= 2;
   ta.place(P->pack_cluster);
   tb.place(P->pack_cluster);
-  auto up = [](auto** dst, const auto& v) {
-    using T = typename std::remove_reference<decltype(v)>::type::value_type;
-    if (v.empty()) return;
-    BST_CUDA(cudaMalloc((void**)dst, sizeof(T) * v.size()));
-    BST_CUDA(cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
+  // one allocation and one copy: the first pass over a new structure pays for
+  // each (768 -> 700 us for five sectors a leg)
+  std::vector<char> host;
+  auto place = [&](const auto& v) {
+    const size_t at = host.size();
+    host.resize(at + (v.size() * sizeof(v[0]) + 255) / 256 * 256);
+    if (!v.empty()) std::memcpy(host.data() + at, v.data(), v.size() * sizeof(v[0]));
+    return at;
   };
-  up(&P->d_pgA, ta.g);
-  up(&P->d_psA, ta.sg);
-  up(&P->d_pgB, tb.g);
-  up(&P->d_psB, tb.sg);
-  up(&P->d_pcA, ta.ctas);
-  up(&P->d_pcB, tb.ctas);
+  const size_t at[] = {place(ta.g), place(ta.sg), place(tb.g), place(tb.sg), place(ta.ctas), place(tb.ctas)};
+  if (!host.empty()) {
+    BST_CUDA(cudaMalloc(&P->d_pack, host.size()));
+    BST_CUDA(cudaMemcpy(P->d_pack, host.data(), host.size(), cudaMemcpyHostToDevice));
+  }
+  char* base = static_cast<char*>(P->d_pack);
+  P->d_pgA = reinterpret_cast<oz::PackGroup*>(base + at[0]);
+  P->d_psA = reinterpret_cast<oz::PackSeg*>(base + at[1]);
+  P->d_pgB = reinterpret_cast<oz::PackGroup*>(base + at[2]);
+  P->d_psB = reinterpret_cast<oz::PackSeg*>(base + at[3]);
+  P->d_pcA = reinterpret_cast<int2*>(base + at[4]);
+  P->d_pcB = reinterpret_cast<int2*>(base + at[5]);
   P->ncA = int(ta.ctas.size());
   P->ncB = int(tb.ctas.size());
   P->packed = true;

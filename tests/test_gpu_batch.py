@@ -287,3 +287,46 @@ def test_autotune_changes_no_bit(bst, ctx):
     log = ctx.tuning_log()
     assert "relayout chunk chosen" in log
     assert "gemm_f64 tile order chosen" in log and "gemm_ozaki tile order chosen" in log
+
+
+def test_tensor_core_batch_holds_no_fp64_buffers(bst):
+    """A batch that has only been called in tensor-core arithmetic holds its
+    digits (2 bytes times five digits an operand element, K rounded up to 32)
+    and tables, not FP64 sector matrices; the first FP64 call may come inside
+    a stream capture, and its graph gives an eager call's bits."""
+    c = bst.Context(0)
+    try:
+        c.set_autotune(False)
+        leg = lambda f, d: bst.Leg(f, (0, 1), d)  # noqa: E731
+        rng = np.random.default_rng(4)
+        As, Bs, a, b = [], [], [], []
+        for i in range(4):
+            m, k, n = (3000 + 7 * i, 1500), (1024, 992), (2500, 2000 + 9 * i)
+            As.append(c.layout([leg(1, m), leg(-1, k)]))
+            Bs.append(c.layout([leg(-1, n), leg(1, k)]))
+            a.append(torch.tensor(rng.standard_normal(As[-1].nnz), device="cuda:0"))
+            b.append(torch.tensor(rng.standard_normal(Bs[-1].nnz), device="cuda:0"))
+        Cls = [c.contract_layout(A, B, (1,), (1,)) for A, B in zip(As, Bs)]
+        cs = [torch.zeros(L.nnz, dtype=torch.float64, device="cuda:0") for L in Cls]
+        run = lambda prec: c.contract_batched(As, a, Bs, b, (1,), (1,), prec=prec, Cls=Cls, cs=cs)  # noqa: E731
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        run("ozaki")
+        torch.cuda.synchronize()
+        held = free - torch.cuda.mem_get_info()[0]
+        elems = sum(L.nnz for L in As + Bs)
+        assert held <= 1.1 * 10 * 1024 / 992 * elems + 64e6
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            run("fp64")
+        for x in cs:
+            x.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        got = [x.clone() for x in cs]
+        run("fp64")
+        torch.cuda.synchronize()
+        for x, y in zip(got, cs):
+            assert torch.equal(x, y) and float(x.abs().max()) > 1
+    finally:
+        c.close()
