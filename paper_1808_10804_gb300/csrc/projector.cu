@@ -719,11 +719,19 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
     double ratio = 1e300;
     for (size_t i = 0; i < secs.size(); ++i)
       if (lowest[i] > 0) {
-        double low = lowest[i];
+        double low = lowest[i], top = 0;
+        bool dropped = false;
         for (int j = 0; j < secs[i].c; ++j) {
           const double d = v[secs[i].val_off + j];
+          top = std::max(top, d);
           if (d > 0) low = std::min(low, d);
+          else dropped = true;
         }
+        // (a column that the FP32 factors dropped: its singular value is below
+        // ~1e-6 of the largest, so the plain steps have all but converged; the
+        // rest of the columns, taken for the block, had called for 14 products
+        // more, where 6 plain steps do)
+        if (dropped) low = std::min(low, 1e-12 * top);
         ratio = std::min(ratio, lowest[i] / low);
       }
     if (settled > 0 && ratio < 1e300) need /= std::pow(ratio, settled);
@@ -1091,6 +1099,8 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
         if (!x.direct) ctx->tune_log += " " + std::to_string(x.b);
       ctx->tune_log += ", Jacobi sweeps";
       for (int v : hsw) ctx->tune_log += " " + std::to_string(v);
+      if (!fplan.empty()) ctx->tune_log += ", filters of degree";
+      for (auto& f : fplan) ctx->tune_log += " " + std::to_string(f.m);
       ctx->tune_log += "\n";
     }
     const bool ok = worst <= tol || (round > 0 && fplan.empty() && worst > 0.5 * prev_worst && worst <= 100 * tol);

@@ -142,3 +142,54 @@ def test_operand_not_finite_is_refused(bst, prec, bad):
         assert e.value.code == 7  # BST_E_NUMERIC
         assert np.abs(sv[-1] - sv[0]).max() <= 1e-9 * sv[0].max()
     ctx.close()
+
+
+def run_spectrum(bst, prec, sing, chi=CHI):
+    """The projector of N = U diag(sing(s)) V^T over the sectors of DIMS and
+    the rounds that the tuning log names: (iterations, filter degrees)."""
+    rng = np.random.default_rng(11)
+    rows, cols = DIMS
+    N = []
+    for s in range(3):
+        n = min(rows[s], cols[s])
+        u, v = (np.linalg.qr(rng.standard_normal((d, n)))[0] for d in (rows[s], cols[s]))
+        N.append((u * sing(s, np.arange(n))) @ v.T)
+    ctx = bst.Context(0)
+    leg = lambda f, d: bst.Leg(f, (0, 1, 2), d)  # noqa: E731
+    Rt = ctx.layout([leg(1, rows), leg(-1, rows)])
+    Rb = ctx.layout([leg(-1, rows), leg(1, cols)])
+    flat = lambda xs: torch.tensor(np.concatenate([x.reshape(-1) for x in xs]), device="cuda:0")  # noqa: E731
+    sv, kept = ctx.svd_projector(Rt, flat([np.eye(r) for r in rows]), Rb, flat(N), 1, chi, 1e-14, 1, prec=prec)[4:]
+    ctx.sync()
+    lam = np.sort(np.concatenate([np.linalg.svd(x, compute_uv=False) for x in N]))[::-1] ** 2
+    assert np.abs(np.sort(np.square(sv))[::-1] - lam[:kept]).max() <= 100 * TOL[prec] * lam[0]
+    rounds = []
+    for line in ctx.tuning_log().splitlines():
+        if "iterations," in line:
+            deg = line.split("filters of degree")[1].split() if "filters" in line else []
+            rounds.append((int(line.split("subspace: ")[1].split()[0]), [int(d) for d in deg]))
+    ctx.close()
+    return rounds
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+@pytest.mark.parametrize("below", [0.0, 1e-7])
+def test_block_past_the_rank(bst, prec, below):
+    """A block that holds all of a low-rank N (or all above a wide gap) after
+    the plain steps takes no more products than the nine plain steps that
+    solve it."""
+    amp = (1.0, 0.9, 0.8)
+    rounds = run_spectrum(bst, prec, lambda s, j: amp[s] * np.where(j < 10, 0.9 ** j, below * 0.9 ** j))
+    assert rounds[-1][0] <= 9, rounds
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+def test_filters_run_where_they_should(bst, prec):
+    """A slowly decaying spectrum is filtered; in FP64 one that falls by more
+    than the growth between factorisations allows is not, in any round."""
+    amp = (1.0, 0.9, 0.8)
+    slow = run_spectrum(bst, prec, lambda s, j: amp[s] * 0.98 ** j)
+    assert slow[0][1] and max(slow[0][1]) <= 3 and slow[0][1][-1] == 2, slow
+    if prec == "fp64":
+        steep = run_spectrum(bst, prec, lambda s, j: amp[s] * 0.9 ** j)
+        assert not any(d for _, d in steep), steep
