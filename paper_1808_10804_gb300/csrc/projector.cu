@@ -696,28 +696,31 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   // when none fits: a spectrum so steep that the growth bound puts alpha
   // above a kept value (plain steps, which factor after every half).
   double gain = 1.0;  // growth that the plan gives every kept value
-  auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod, int settled = 0) {
+  // smallest value that counts as kept, per sector (0: none): down to a tenth
+  // of the truncation's (estimates are low by a small factor at most); empty
+  // when a value is not finite
+  auto kept_ends = [&](const std::vector<double>& v) {
     std::vector<std::pair<double, int>> all;
     for (size_t i = 0; i < secs.size(); ++i)
       if (!secs[i].direct)
         for (int j = 0; j < secs[i].c; ++j) {
           const double d = v[secs[i].val_off + j];
-          if (!std::isfinite(d)) return std::vector<Filter>();
+          if (!std::isfinite(d)) return std::vector<double>();
           all.push_back({d, int(i)});
         }
     std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    // smallest value that counts as kept, per sector: down to a tenth of the
-    // truncation's (estimates are low by a small factor at most)
     std::vector<double> lowest(secs.size(), 0.0);
     const double cut = all.empty() ? 0.0 : 0.1 * all[std::min<size_t>(all.size(), size_t(chi)) - 1].first;
     for (size_t t = 0; t < all.size() && all[t].first > cut; ++t) {
       double& l = lowest[all[t].second];
       if (int64_t(t) < chi || l == 0) l = all[t].first;
     }
-    // (plain steps before: the kept values have grown by their ratio to the
-    // block's lower end in each)
+    return lowest;
+  };
+  // growth of every kept value over the block's lower end in a plain step
+  auto plain_growth = [&](const std::vector<double>& v, const std::vector<double>& lowest) {
     double ratio = 1e300;
-    for (size_t i = 0; i < secs.size(); ++i)
+    for (size_t i = 0; i < lowest.size(); ++i)
       if (lowest[i] > 0) {
         double low = lowest[i], top = 0;
         bool dropped = false;
@@ -734,6 +737,12 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
         if (dropped) low = std::min(low, 1e-12 * top);
         ratio = std::min(ratio, lowest[i] / low);
       }
+    return ratio;
+  };
+  auto plan_filters = [&](const std::vector<double>& v, double need, int mmax, int nprod, int settled = 0) {
+    const std::vector<double> lowest = kept_ends(v);
+    if (lowest.empty()) return std::vector<Filter>();
+    const double ratio = plain_growth(v, lowest);  // (plain steps before)
     if (settled > 0 && ratio < 1e300) need /= std::pow(ratio, settled);
     // the filter of degree m and the growth of the kept values (0: does not fit)
     auto of_degree = [&](int m, Filter& f) {
@@ -1110,11 +1119,12 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       ctx->multi_round[rr_key] = true;
       return false;
     }
-    // length of the next round: from the second round on, extrapolate the
-    // residual's geometric decay per step to half the tolerance (at least
-    // `iters`, at most 6 * iters steps), so slowly converging sectors are
-    // checked with few Rayleigh-Ritz rounds
+    // length of the next round (plain_steps): from the second round on by the
+    // residual's decay over a plain round, after a filtered one by the Ritz
+    // values, so slowly converging sectors are checked with few Rayleigh-Ritz
+    // rounds
     int next = iters;
+    const bool filtered = !fplan.empty();
     // (a filtered round that did not bring the residual down by half: its
     // interval did not fit the spectrum, or its floor is reached; plain steps
     // from here)
@@ -1145,10 +1155,11 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
       next = 0;
     } else if (!fplan.empty()) {
       mixed_rr = false;  // sized to converge: its Rayleigh-Ritz step is the FP64 one
-    } else if (round > 0 && steps > 0 && worst > 0 && prev_worst > worst) {
-      const double rho = std::pow(worst / prev_worst, 1.0 / steps);
-      const double need = std::log(0.5 * tol / worst) / std::log(rho);
-      if (std::isfinite(need)) next = int(std::min<double>(6.0 * iters, std::max<double>(iters, std::ceil(need))));
+    } else if (filtered && !lost && !diverged) {
+      const std::vector<double> lowest = kept_ends(hl);
+      next = plain_steps(iters, worst, tol, 1.0 / plain_growth(hl, lowest));
+    } else if (round > 0 && steps > 0 && !filtered) {
+      next = plain_steps(iters, worst, tol, std::pow(worst / prev_worst, 1.0 / steps));
     }
     steps = next == 0 ? 0 : std::min(next, std::max(1, max_total - total));
     prev_worst = worst;

@@ -1,6 +1,7 @@
-// The projector's convergence measure (host only).
+// The projector's convergence measure and what follows from it (host only).
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 #include <cstddef>
 #include <limits>
@@ -17,6 +18,15 @@ inline double raise_worst(double worst, const double* res, std::size_t n) {
     if (res[j] > worst) worst = res[j];
   }
   return worst;
+}
+
+// Plain steps that bring a residual `worst` to half the tolerance when each
+// multiplies it by `decay`: at least `iters`, at most 6 iters, and `iters` when
+// the decay says nothing (not below one, or a residual that is not finite).
+inline int plain_steps(int iters, double worst, double tol, double decay) {
+  if (!(worst > 0) || !std::isfinite(worst) || !(decay > 0 && decay < 1)) return iters;
+  const double need = std::log(0.5 * tol / worst) / std::log(decay);
+  return int(std::min<double>(6.0 * iters, std::max<double>(iters, std::ceil(need))));
 }
 
 }  // namespace bst
