@@ -10,7 +10,7 @@
 // d = i + j (weight 2^-16-9d) in tensor memory:
 //   * d = 0, 1, 2 are read out every 64 K (two pipeline stages), where their
 //     FP32 sums are exact integers of magnitude <= 3 * 2^22 < 2^24, and
-//     added into one 64-bit integer per output (K <= 10000 keeps it from
+//     added into one 64-bit integer per output (K <= kMaxK keeps it from
 //     overflowing);
 //   * d = 3, 4 carry weights <= 2^-27 of the leading term and accumulate in
 //     FP32 over the whole K.
@@ -65,6 +65,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kTM = 128;           // tile rows (M)
 constexpr int kTK = 32;            // K per stage (64 bytes of BF16)
+constexpr int kMaxK = 10000;       // longest sum of a plan (at most 2^43 K < 2^57 in the accumulators)
 constexpr int kABytes = kTM * kTK * 2;   // 8 KB per slice
 constexpr int kEpiWarps = 16;            // four per quarter of the 128 tensor-memory lanes
 constexpr int kThreads = 32 * (2 + kEpiWarps);  // TMA, MMA and epilogue warps
@@ -97,12 +98,12 @@ struct Prob {
   int32_t M, N, K, pad;
   int32_t arow, brow;  // first row of this problem in the split A / B buffers
   int64_t c_off, c_m, c_n;
-  // output scatter (scatter != 0): element (m, n) of the problem goes to
-  // C[bbase[bb_off + r ncc + c] + mi w + ni] with (r, mi) = rowtab[rt_off + m]
+  // output scatter (plans with tables, see Scatter): element (m, n) of the
+  // problem goes to C[bbase[bb_off + r ncc + c] + mi w + ni] with (r, mi) = rowtab[rt_off + m]
   // and (c, ni, w) = coltab[ct_off + n]: the canonical block (r, c) of the
   // output tensor, row-major [rows of config r x w], instead of a strided
   // sector matrix
-  int32_t scatter, ncc;
+  int32_t ncc;
   int64_t rt_off, ct_off, bb_off;
 };
 
@@ -575,11 +576,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // d3 and d4 go back to the next tile's products, which wait for them,
       // before any output is written.  S3 + S4 2^-9 to the nearest integer as
-      // 2^12 H + R, both by the constant (sums up to 2^34, K of 32768: past
-      // that by the 64-bit conversion, which goes through the FP64 pipe)
-      const bool wide = t.nk > 1024;
-      const unsigned long long off0 = ((unsigned long long)npair * kMagicBits) << (18 + kUp);
-      const unsigned long long off = off0 + (S == 5 && !wide ? (unsigned long long)kMagicBits * 4097 : 0);
+      // 2^12 H + R, both by the constant (|S3| <= 4 K 2^16 < 2^32 for K up to
+      // kMaxK, S4 2^-9 is at most 1/400 of that: |H| stays far below 2^22)
+      const unsigned long long off = (((unsigned long long)npair * kMagicBits) << (18 + kUp)) +
+                                     (S == 5 ? (unsigned long long)kMagicBits * 4097 : 0);
 #pragma unroll
       for (int h = 0; h < kCols; h += 8) {
         if constexpr (S == 5) {
@@ -590,14 +590,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const float x = fmaf(__uint_as_float(w4[j]), 1.0f / 512.0f, __uint_as_float(w3[j]));
-            if (wide) {
-              T[h + j] += (unsigned long long)__float2ll_rn(x);
-            } else {
-              const float hc = fmaf(x, 1.0f / 4096.0f, kMagic);
-              const float r = fmaf(hc - kMagic, -4096.0f, x);  // exact, at most 2^11
-              T[h + j] = mad_wide(__float_as_int(hc), 4096, T[h + j]);
-              T[h + j] = mad_wide(__float_as_int(r + kMagic), 1, T[h + j]);
-            }
+            const float hc = fmaf(x, 1.0f / 4096.0f, kMagic);
+            const float r = fmaf(hc - kMagic, -4096.0f, x);  // exact, at most 2^11
+            T[h + j] = mad_wide(__float_as_int(hc), 4096, T[h + j]);
+            T[h + j] = mad_wide(__float_as_int(r + kMagic), 1, T[h + j]);
           }
         }
 #pragma unroll
@@ -1061,9 +1057,9 @@ struct alignas(16) PackLeg {
 
 struct PackSeg {
   int64_t off;          // block offset in its tensor (elements)
-  int32_t k0, w;        // columns [k0, k0 + w) of the row
+  int32_t k0;           // its first column of the row
   int32_t nr, nc;       // row legs, column legs
-  int32_t src, pad;     // index of the tensor in the job's pointer table
+  int32_t src;          // index of the tensor in the job's pointer table
   PackLeg leg[kMaxRank];  // row legs then column legs, matrix order
 };
 
@@ -1368,8 +1364,10 @@ static EncodeTiledFn encode_fn() {
 }
 
 // Map of a split buffer (S slices of `rows` rows of kpitch): one box is all
-// slices of box_rows rows of a K chunk.  Rows past a slice's end belong to
-// the next slice (past the last one: to the buffer's spare rows).
+// slices of box_rows rows of a K chunk.  Rows past a slice's end are filled
+// with zeros; with fewer rows than a box the map reaches into the next slice
+// (past the last one into the buffer's spare rows), and what a tile reads
+// there goes to rows or columns that are not stored.
 static CUtensorMap make_map(void* base, int kpitch, int rows, int box_rows, int S) {
   CUtensorMap m;
   std::memset(&m, 0, sizeof(m));
@@ -1540,7 +1538,6 @@ static void append_pack(PackTables& T, const Layout* L, const MatView& v, const 
             sg.leg[j] = {int32_t(sh[leg]), int32_t(bst[leg]), f.m, f.l};
             (j < nr ? hh : w) *= sh[leg];
           }
-          sg.w = int32_t(w);
           BST_REQUIRE(hh == h && sg.k0 == kcov, BST_E_SHAPE, "pack: segment does not tile the row");
           kcov += w;
           T.sg.push_back(sg);
@@ -1580,7 +1577,7 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
   int maxk = 1;
   P->ab_same = !probs.empty();
   for (auto& g : probs) {
-    BST_REQUIRE(g.K <= 10000, BST_E_UNSUPPORTED, "Ozaki GEMM: K above 10000");
+    BST_REQUIRE(g.K <= oz::kMaxK, BST_E_UNSUPPORTED, "Ozaki GEMM: K above 10000");
     maxk = std::max(maxk, g.K);
     P->ab_same = P->ab_same && g.M == g.N && g.a_off == g.b_off && g.a_m == g.b_n && g.a_k == g.b_k;
   }
@@ -1597,7 +1594,6 @@ static OzakiPlan* build_plan(Ctx* ctx, const std::vector<GemmProb>& probs, int o
     q.c_n = g.c_n;
     if (sc) {
       const size_t pi = hp.size();
-      q.scatter = 1;
       q.ncc = sc->ncc[pi];
       q.rt_off = sc->rt_off[pi];
       q.ct_off = sc->ct_off[pi];

@@ -204,11 +204,10 @@ __global__ void __launch_bounds__(kRelThreads) relayout_pair_kernel(RelPart a, R
 
 __global__ void __launch_bounds__(kRelThreads, kBoxCtas) relayout_box_kernel(const RelBox* __restrict__ boxes,
                                                                              const int2* __restrict__ tiles, double* blk,
-                                                                             double* mat, int dir, double alpha,
-                                                                             double beta) {
+                                                                             double* mat, int dir) {
   __shared__ RelShared sh;
   const int2 c = tiles[blockIdx.x];
-  relayout_box<kRelThreads, kBoxU>(sh, boxes[c.x], c.y, blk, mat, dir, alpha, beta);
+  relayout_box<kRelThreads, kBoxU>(sh, boxes[c.x], c.y, blk, mat, dir);
 }
 
 // Boxes only where rel_box_pays.  A straight copy reaches 5.8 TB/s when a
@@ -232,10 +231,12 @@ void launch_relayout(Ctx* ctx, const DevRelayout& r, const double* blk, double* 
                      double beta, cudaStream_t s, bool behind) {
   if (r.nchunks == 0) return;
   ProfScope ps(ctx, s, "relayout", 0.0, 16.0 * r.elems);
-  if (r.boxes)
-    relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir, alpha,
-                                                          beta);
-  else if (r.legs_made)
+  if (r.boxes) {
+    // (only uploaded lists have boxes, and those are permutations, fusions and
+    // gathers: plain copies)
+    BST_REQUIRE(dir == 0 || (alpha == 1.0 && beta == 0.0), BST_E_UNSUPPORTED, "copies by boxes are plain ones");
+    relayout_box_kernel<<<r.nchunks, kRelThreads, 0, s>>>(r.boxes, r.chunks, const_cast<double*>(blk), mat, dir);
+  } else if (r.legs_made)
     launch_behind(behind, relayout_legs_kernel, dim3(unsigned(r.nchunks)), kRelThreads, 0, s, (const RelTask*)r.tasks,
                   (const RelLegTab*)r.legs, (const int2*)r.chunks, const_cast<double*>(blk), mat, dir, alpha, beta);
   else

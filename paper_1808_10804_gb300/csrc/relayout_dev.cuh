@@ -331,11 +331,10 @@ __device__ __forceinline__ void rel_box(RelShared& sh, const RelBox& b, int tile
   }
 }
 
-// Box `tile` of one task, directions as relayout_range.
+// Box `tile` of one task, a plain copy in either direction (as
+// relayout_range).
 template <int kThreads, int kU>
-__device__ __forceinline__ void relayout_box(RelShared& sh, const RelBox& b, int tile, double* blk, double* mat, int dir,
-                                             double alpha, double beta) {
-  const bool plain = dir == 0 || (alpha == 1.0 && beta == 0.0);
+__device__ __forceinline__ void relayout_box(RelShared& sh, const RelBox& b, int tile, double* blk, double* mat, int dir) {
   if (threadIdx.x < 32) rel_box(sh, b, tile);
   __syncthreads();
   // (offset, position) of index i over the legs [j, je) of one side's list
@@ -398,15 +397,6 @@ __device__ __forceinline__ void relayout_box(RelShared& sh, const RelBox& b, int
 #pragma unroll
     for (int u = 0; u < kU; ++u)
       if (ok[u]) v[u] = sh.buf[pos[u]];
-    // (no FP64 arithmetic in a plain copy, see relayout_range)
-    if (!plain) {
-#pragma unroll
-      for (int u = 0; u < kU; ++u)
-        if (ok[u]) {
-          v[u] = alpha * v[u];
-          if (beta != 0.0) v[u] += beta * dst[off[u]];
-        }
-    }
 #pragma unroll
     for (int u = 0; u < kU; ++u)
       if (ok[u]) dst[off[u]] = v[u];

@@ -145,3 +145,108 @@ def test_output_over_an_operand(bst, ctx, inner, over, beta):
         ctx.contract(A, a, B, b, *pairs, prec=prec, beta=beta, Cl=C, c=c)
         ctx.sync()
         assert torch.equal(c, ref), prec
+
+
+@pytest.mark.parametrize("prec", ["ozaki", "bf16x3"])
+@pytest.mark.parametrize("inner", ["open", "contracted"])
+@pytest.mark.parametrize("M,N,K", [(40, 33, 1023), (33, 40, 1025), (70, 31, 1057), (31, 70, 2049), (9800, 33, 1100),
+                                   (2500, 31, 1057)])
+def test_product_edges_of_long_sums(bst, ctx, M, N, K, inner, prec):
+    """As above with more k than a table of the pack holds (1024): in a
+    cluster whose last CTAs have none, and in one CTA (many rows)."""
+    test_product_edges(bst, ctx, M, N, K, inner, prec)
+
+
+@pytest.mark.parametrize("prec", ["ozaki", "bf16x3"])
+@pytest.mark.parametrize("order", ["kkm", "mkk", "kmk"])
+@pytest.mark.parametrize("K", [0, 33, 129, 513, 1023, 1025, 2049])
+def test_rows_of_many_segments(bst, ctx, K, order, prec):
+    """Rows that run over several blocks: two contracted legs whose middle
+    charge has K columns in three segments of odd lengths, or (K = 0) three
+    whose middle charges have up to 192 short segments; two open legs, so that
+    a sector has several row configurations too."""
+    from oracle import u1
+    rng = np.random.default_rng([K, len(order)])
+    if K:
+        a, c = K // 9, K // 13
+        ks = [(bst.Leg(1, (0, 1, 2), (a, K - 2 * a - 3 * c, c))), bst.Leg(1, (0, 1, 2), (3, 1, 2))]
+        ms = [bst.Leg(-1, (0, 1, 2, 3, 4), (17, 20, 45, 33, 7)), bst.Leg(-1, (0, 1), (1, 2))]
+    else:
+        d = lambda n: tuple(int(x) for x in rng.integers(1, 3, n))  # noqa: E731
+        ks = [bst.Leg(1, tuple(range(16)), d(16)) for _ in range(3)]
+        ms = [bst.Leg(-1, (7, 21, 22, 23), (9, 35, 14, 5)), bst.Leg(-1, (0, 1), (1, 2))]
+    flip = lambda x: bst.Leg(-x.flow, x.charges, x.degs)  # noqa: E731
+    ns = [flip(m) for m in ms]
+    nk = len(ks)
+    # places of the contracted and the open legs
+    at = {"kkm": (list(range(nk)), [nk, nk + 1]), "mkk": (list(range(2, nk + 2)), [0, 1]),
+          "kmk": ([0, *range(3, nk + 2)], [1, 2])}[order]
+    def legs(k, m):
+        x = [None] * (nk + 2)
+        for i, leg in zip(at[0] + at[1], k + m):
+            x[i] = leg
+        return x
+    LA, LB = ctx.layout(legs(ks, ms)), ctx.layout(legs([flip(k) for k in ks], ns))
+    x, y = rng.standard_normal(LA.nnz), rng.standard_normal(LB.nnz)
+    Cl, z = ctx.contract(LA, torch.tensor(x, device="cuda:0"), LB, torch.tensor(y, device="cuda:0"), tuple(at[0]),
+                         tuple(at[0]), prec=prec)
+    ctx.sync()
+    olegs = lambda L: [u1.Leg(int(q.flow), tuple(q.charges), tuple(q.degs)) for q in L.legs]  # noqa: E731
+    A, B = (u1.to_dense(olegs(L), v).transpose(at[1] + at[0]) for L, v in ((LA, x), (LB, y)))
+    m, n = A.shape[0] * A.shape[1], B.shape[0] * B.shape[1]
+    got = u1.to_dense(olegs(Cl), z.cpu().numpy()).reshape(m, n)
+    check(got, A.reshape(m, -1), B.reshape(n, -1).T, prec)
+
+
+@pytest.mark.parametrize("prec", ["ozaki", "bf16x3"])
+@pytest.mark.parametrize("inner", ["open", "contracted"])
+def test_results_outside_the_normal_range(bst, ctx, inner, prec):
+    """Row and column scales of 2^+-600: results overflow to infinity, become
+    subnormal or vanish as the product does, beside ordinary ones."""
+    rng = np.random.default_rng(11)
+    M, K, N = 130, 70, 67
+    A, B = np.abs(rng.standard_normal((M, K))), np.abs(rng.standard_normal((K, N)))
+    ea, eb = rng.choice((-600, -470, 0, 500, 600), M), rng.choice((-600, -470, 0, 500, 600), N)
+    leg = lambda f, d: bst.Leg(f, (0,), (d,))  # noqa: E731
+    at = inner == "open"
+    LA = ctx.layout([leg(-1, K), leg(1, M)] if at else [leg(1, M), leg(-1, K)])
+    LB = ctx.layout([leg(1, K), leg(-1, N)] if at else [leg(-1, N), leg(1, K)])
+    x, y = np.ldexp(A, ea[:, None]), np.ldexp(B, eb)
+    put = lambda v, t: torch.tensor(np.ascontiguousarray(v.T if t else v), device="cuda:0").reshape(-1)  # noqa: E731
+    c = ctx.contract(LA, put(x, at), LB, put(y, not at), (0,) if at else (1,), (0,) if at else (1,), prec=prec)[1]
+    ctx.sync()
+    got, e = c.cpu().numpy().reshape(M, N), ea[:, None] + eb
+    with np.errstate(over="ignore"):
+        ref = np.ldexp(A @ B, e)
+        bound = np.ldexp(BOUND[prec] * K * np.outer(A.max(1), B.max(0)), e) + 2.0 ** -1074
+    inf = np.isinf(ref)
+    assert inf.any() and (ref == 0).any() and ((ref > 0) & (ref < 2.0 ** -1022)).any()
+    assert np.array_equal(got[inf], ref[inf])
+    assert np.all(np.abs(got - np.where(inf, 0, ref))[~inf] <= bound[~inf])
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("inner", ["open", "contracted"])
+def test_values_that_are_not_finite_stay_in_their_rows(bst, ctx, inner, bad):
+    """An infinity or NaN in some rows of A and columns of B: every other
+    element of the result keeps its bits."""
+    rng = np.random.default_rng(12)
+    M, K, N = 133, 150, 70
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((K, N))
+    leg = lambda f, d: bst.Leg(f, (0,), (d,))  # noqa: E731
+    at = inner == "open"
+    LA = ctx.layout([leg(-1, K), leg(1, M)] if at else [leg(1, M), leg(-1, K)])
+    LB = ctx.layout([leg(1, K), leg(-1, N)] if at else [leg(-1, N), leg(1, K)])
+    put = lambda v, t: torch.tensor(np.ascontiguousarray(v.T if t else v), device="cuda:0").reshape(-1)  # noqa: E731
+    rows, cols = (0, 31, 64, 132), (5, 69)
+    x, y = A.copy(), B.copy()
+    for r in rows:
+        x[r, rng.integers(0, K)] = bad
+    for q in cols:
+        y[rng.integers(0, K), q] = bad
+    got = []
+    for u, v in ((A, B), (x, y)):
+        c = ctx.contract(LA, put(u, at), LB, put(v, not at), (0,) if at else (1,), (0,) if at else (1,), prec="ozaki")[1]
+        ctx.sync()
+        got.append(np.delete(np.delete(c.cpu().numpy().reshape(M, N), rows, 0), cols, 1))
+    assert np.array_equal(*got)
