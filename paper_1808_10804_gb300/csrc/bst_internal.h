@@ -181,11 +181,14 @@ struct DevGemm {
   std::vector<int64_t> hw_off;  // the same offsets on the host
   int64_t wtot = 0;          // sum of M*N
   int maxK = 0;
+  int ctas = 3;              // resident on an SM (f64_ctas)
   // order 0: problem order; 1: tiles of the longest-K problems first
   // (s: stream of the copies, which have ended on return)
   void upload(const std::vector<GemmProb>& p, int tm, int tn, int order = 0, cudaStream_t s = 0);
   void free_all();
 };
+
+int f64_ctas(const std::vector<GemmProb>& p);
 
 struct OzakiPlan;  // mixed-precision GEMM plan (gemm_ozaki.cu)
 struct BatchPlan;  // batched-contraction plan (batch.cu)

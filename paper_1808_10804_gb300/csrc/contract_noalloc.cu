@@ -181,6 +181,7 @@ void contract_noalloc(Ctx* ctx, Layout* A, const double* a, Layout* B, const dou
   g.tile_idx = reinterpret_cast<int32_t*>(base + o_tidx);
   g.ntiles = int(tprob.size());
   g.nprobs = int(probs.size());
+  g.ctas = f64_ctas(probs);
   double* Am = reinterpret_cast<double*>(base + o_am);
   double* Bm = reinterpret_cast<double*>(base + o_bm);
   double* Cm = reinterpret_cast<double*>(base + o_cm);

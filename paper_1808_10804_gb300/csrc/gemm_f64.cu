@@ -14,6 +14,27 @@ const int kF64TileM = 64;
 const int kF64TileN = 64;
 constexpr int kBK = 16;
 constexpr int kPad = 2;
+constexpr int kSms = 152;
+
+// CTAs an SM: three, but two where three would take all tiles at once although
+// the deep ones (three quarters of the deepest or more) find room among two:
+// the others then go to the SMs that are free first.  Three / two CTAs, four
+// sectors of decreasing sizes: 372 tiles (1000 x 1000 x 1000 and three
+// smaller) 2.98 / 2.66 ms, 363 of depth 5 to 2 32.7 / 27.6 us, the odd-sized
+// corner (354) 524 / 439 us; equal depths: 450 tiles of depth 256 0.88 / 1.17
+// ms, 1024 of 512 4.07 / 4.64; more tiles of different depths: 1515 4.85 /
+// 5.16 ms, 899 1.55 / 1.47.
+int f64_ctas(const std::vector<GemmProb>& p) {
+  int deepest = 0;
+  for (auto& x : p) deepest = std::max(deepest, x.K);
+  long long tiles = 0, deep = 0;
+  for (auto& x : p) {
+    const long long n = ((long long)x.M + kF64TileM - 1) / kF64TileM * ((x.N + kF64TileN - 1) / kF64TileN);
+    tiles += n;
+    if (4ll * x.K >= 3ll * deepest) deep += n;
+  }
+  return tiles <= 3 * kSms && deep <= 2 * kSms ? 2 : 3;
+}
 
 void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order, cudaStream_t s) {
   free_all();
@@ -32,6 +53,7 @@ void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order, 
     }
   }
   ntiles = int(tp.size());
+  ctas = f64_ctas(p);
   std::vector<int64_t> wo(std::max(nprobs, 1), 0);
   wtot = 0;
   maxK = 0;
@@ -94,10 +116,14 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 // multiplied.
 //
 // What bounds it: the DMMA units, one a scheduler (an 8x8x4 product takes one
-// about 570 cycles), so a product is issued only where it counts, and the
-// 8x8 tiles are dealt to the warps one by one:
-//   * none past M or N (an odd-sized FP64 corner, 0.33 GFLOP: 594 -> 428 us, with
-//     two CTAs an SM so that nothing spills: three took 512);
+// about 600 cycles: 2048 x 2048 x 512 in 4.07 ms at 2070 MHz), so a product is
+// issued only where it counts:
+//   * whole tiles: a warp takes a quarter, 4x4 products from 4 + 4 fragments;
+//   * tiles at an edge: the 8x8 tiles inside M and N are dealt to the warps one
+//     by one (an odd-sized FP64 corner, 0.33 GFLOP: 594 -> 439 us).  Whole tiles
+//     dealt likewise need 16 + 16 fragments, hence registers for two CTAs an SM
+//     only: 4096 x 4096 x 4 180 -> 132 us, 2048 x 2048 x 512 4.65 -> 4.07 ms
+//     with quarters and three (f64_ctas);
 //   * of a Gram matrix (both operands the same) only those on and above its
 //     diagonal; the sums below are the same products in the same order, so
 //     they are mirrored.
@@ -116,13 +142,21 @@ __device__ __forceinline__ void f64_tile(const GemmProb& p, int m0, int n0, int 
   const int r8 = min(8, (p.M - m0 + 7) >> 3), c8 = min(8, (p.N - n0 + 7) >> 3);
   const bool tri = sym && m0 == n0;
   const int total = tri ? r8 * (r8 + 1) / 2 : r8 * c8, cnt = (total - part + 3) >> 2;
-  int at[16];  // row and column of the t-th (in 8s: row << 8 | column)
-  {
+  const bool whole = total == 64;
+  const int wi = (part >> 1) * 4, wj = (part & 1) * 4;
+  // row and column of the t-th (in 8s), a byte each four to a register
+  uint32_t at[4] = {};
+  auto row8 = [&](int t) { return int(at[t / 4] >> (t % 4 * 8 + 3) & 7u) * 8; };
+  auto col8 = [&](int t) { return int(at[t / 4] >> (t % 4 * 8) & 7u) * 8; };
+  if (whole) {
+#pragma unroll
+    for (int t = 0; t < 16; ++t) at[t / 4] |= uint32_t((wi + t / 4) << 3 | (wj + t % 4)) << (t % 4 * 8);
+  } else {
     int i = 0, j = part;  // (counted in a row that starts at column 0, then moved)
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
       while (i < r8 && j >= c8) ++i, j -= c8 - (tri ? i : 0);
-      at[t] = i << 8 | j;
+      if (t < cnt) at[t / 4] |= uint32_t(i << 3 | j) << (t % 4 * 8);
       j += 4;
     }
   }
@@ -160,17 +194,17 @@ __device__ __forceinline__ void f64_tile(const GemmProb& p, int m0, int n0, int 
       if (kk >= kn) break;
       const double* a = &sA[buf][kk + tg][g];
       const double* b = &sB[buf][kk + tg][g];
-      if (cnt == 16) {  // (without a branch per tile the loads run ahead)
-        double af[16], bf[16];
+      if (whole) {
+        double af[4], bf[4];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) af[t] = a[(at[t] >> 8) * 8], bf[t] = b[(at[t] & 255) * 8];
+        for (int t = 0; t < 4; ++t) af[t] = a[(wi + t) * 8], bf[t] = b[(wj + t) * 8];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) dmma(acc[t][0], acc[t][1], af[t], bf[t]);
+        for (int t = 0; t < 16; ++t) dmma(acc[t][0], acc[t][1], af[t / 4], bf[t % 4]);
       } else {
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
           if (t >= cnt) break;
-          dmma(acc[t][0], acc[t][1], a[(at[t] >> 8) * 8], b[(at[t] & 255) * 8]);
+          dmma(acc[t][0], acc[t][1], a[row8(t)], b[col8(t)]);
         }
       }
     }
@@ -180,16 +214,17 @@ __device__ __forceinline__ void f64_tile(const GemmProb& p, int m0, int n0, int 
     if (t >= cnt) break;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int gm = m0 + (at[t] >> 8) * 8 + g;
-      const int gn = n0 + (at[t] & 255) * 8 + tg * 2 + h;
+      const int gm = m0 + row8(t) + g;
+      const int gn = n0 + col8(t) + tg * 2 + h;
       if (gm >= p.M || gn >= p.N) continue;
       out[(long long)gm * om + (long long)gn * on] = acc[t][h];
-      if (sym && (at[t] >> 8) * 8 + m0 < (at[t] & 255) * 8 + n0) out[(long long)gn * om + (long long)gm * on] = acc[t][h];
+      if (sym && row8(t) + m0 < col8(t) + n0) out[(long long)gn * om + (long long)gm * on] = acc[t][h];
     }
   }
 }
 
-__global__ void __launch_bounds__(128, 2) gemm_f64_kernel(const GemmProb* __restrict__ probs,
+template <int kCtas>  // an SM
+__global__ void __launch_bounds__(128, kCtas) gemm_f64_kernel(const GemmProb* __restrict__ probs,
                                                        const int32_t* __restrict__ tile_prob,
                                                        const int32_t* __restrict__ tile_idx,
                                                        const double* __restrict__ A,
@@ -280,8 +315,8 @@ void launch_gemm_f64(Ctx* ctx, const DevGemm& g, const double* A, const double* 
                      bool behind) {
   if (g.ntiles == 0) return;
   ProfScope ps(ctx, s, "gemm_f64", g.flops, 0.0);
-  launch_behind(behind, gemm_f64_kernel, dim3(unsigned(g.ntiles)), 128, 0, s, (const GemmProb*)g.probs,
-                (const int32_t*)g.tile_prob, (const int32_t*)g.tile_idx, A, B, C);
+  launch_behind(behind, g.ctas == 3 ? gemm_f64_kernel<3> : gemm_f64_kernel<2>, dim3(unsigned(g.ntiles)), 128, 0, s,
+                (const GemmProb*)g.probs, (const int32_t*)g.tile_prob, (const int32_t*)g.tile_idx, A, B, C);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
 }

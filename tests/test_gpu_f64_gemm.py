@@ -50,3 +50,45 @@ def test_gram_products(ctx, n):
     bound = 16 * max(n, 8) * 2.0 ** -52
     assert np.abs(X.T @ X - np.eye(n)).max() <= bound
     assert np.abs(H @ X - X * lam).max() <= bound
+
+
+@pytest.mark.parametrize("sizes", [
+    ((64, 64, 64),), ((128, 192, 5),), ((64, 65, 16),), ((71, 128, 33),),  # whole tiles, and one beside an edge
+    ((1500, 1600, 9),), ((1536, 1600, 4),),                                  # 600 tiles of one depth
+    ((640, 640, 50), (322, 300, 21), (65, 63, 1), (9, 64, 3)),               # fewer, of different depths
+    ((1216, 1280, 20), (610, 641, 7), (300, 64, 2)),                         # more, of different depths
+])
+def test_whole_tiles(ctx, sizes):
+    """Whole tiles beside edges, several sectors, with few and many tiles: by
+    three CTAs an SM or two."""
+    from paper_1808_10804_gb300 import bst
+    rng = np.random.default_rng([x for s in sizes for x in s])
+    A = [rng.standard_normal((m, k)) for m, n, k in sizes]
+    B = [rng.standard_normal((k, n)) for m, n, k in sizes]
+    leg = lambda f, i: bst.Leg(f, tuple(range(len(sizes))), tuple(s[i] for s in sizes))  # noqa: E731
+    flat = lambda xs: torch.tensor(np.concatenate([x.reshape(-1) for x in xs]), device="cuda:0")  # noqa: E731
+    LA, LB = ctx.layout([leg(1, 0), leg(-1, 2)]), ctx.layout([leg(1, 2), leg(-1, 1)])
+    c = ctx.contract(LA, flat(A), LB, flat(B), (1,), (0,))[1]
+    ctx.sync()
+    got = np.split(c.cpu().numpy(), np.cumsum([m * n for m, n, _ in sizes])[:-1])
+    for x, a, b, (m, n, k) in zip(got, A, B, sizes):
+        assert np.all(np.abs(x.reshape(m, n) - a @ b) <= (k + 1) * 2.0 ** -52 * (np.abs(a) @ np.abs(b)))
+
+
+def test_three_tiles_an_sm_take_three_times_one(ctx):
+    """450 whole tiles against 304: three a multiprocessor against two, so half
+    as long again (with two CTAs an SM they took twice as long)."""
+    from paper_1808_10804_gb300 import bst
+
+    def time(m, n, k=256):
+        LA, LB = (ctx.layout([bst.Leg(1, (0,), (r,)), bst.Leg(-1, (0,), (c,))]) for r, c in ((m, k), (k, n)))
+        a, b = (torch.zeros(L.nnz, dtype=torch.float64, device="cuda:0") for L in (LA, LB))
+        Cl, c = ctx.contract(LA, a, LB, b, (1,), (0,))
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(14)]
+        for i in range(7):
+            ev[2 * i].record()
+            ctx.contract(LA, a, LB, b, (1,), (0,), Cl=Cl, c=c)
+            ev[2 * i + 1].record()
+        torch.cuda.synchronize()
+        return sorted(x.elapsed_time(y) for x, y in zip(ev[::2], ev[1::2]))[3]
+    assert time(18 * 64, 25 * 64) <= 1.75 * time(16 * 64, 19 * 64)
