@@ -17,23 +17,41 @@ constexpr int kPad = 2;
 constexpr int kSms = 152;
 
 // CTAs an SM: three, but two where three would take all tiles at once although
-// the deep ones (three quarters of the deepest or more) find room among two:
-// the others then go to the SMs that are free first.  Three / two CTAs, four
-// sectors of decreasing sizes: 372 tiles (1000 x 1000 x 1000 and three
-// smaller) 2.98 / 2.66 ms, 363 of depth 5 to 2 32.7 / 27.6 us, the odd-sized
-// corner (354) 524 / 439 us; equal depths: 450 tiles of depth 256 0.88 / 1.17
-// ms, 1024 of 512 4.07 / 4.64; more tiles of different depths: 1515 4.85 /
-// 5.16 ms, 899 1.55 / 1.47.
+// the dear ones (three quarters of the dearest or more) find room among two:
+// the others then go to the SMs that are free first.  Two as well for Gram
+// matrices, whose tiles are dear, half as dear and empty by turns.  Three / two
+// CTAs, four sectors of decreasing sizes: 372 tiles (1000 x 1000 x 1000 and
+// three smaller) 2.98 / 2.66 ms, 363 of depth 5 to 2 32.7 / 27.6 us, the
+// odd-sized corner (354) 524 / 439 us; equal depths: 450 tiles of depth 256
+// 0.88 / 1.17 ms, 1024 of 512 4.07 / 4.64; more tiles of different depths:
+// 1515 4.85 / 5.16 ms, 899 1.55 / 1.47; the products of 40 eigenproblems of 133
+// values 5.8 / 4.3 ms.
 int f64_ctas(const std::vector<GemmProb>& p) {
-  int deepest = 0;
-  for (auto& x : p) deepest = std::max(deepest, x.K);
-  long long tiles = 0, deep = 0;
+  // 8x8 products of a problem's tiles, times K: in whole tiles, along its last
+  // column and row of tiles, in the corner
+  struct Kind {
+    long long n, cost;
+  };
+  auto kinds = [](const GemmProb& x, Kind (&k)[4]) {
+    const long long m = x.M / kF64TileM, n = x.N / kF64TileN;
+    const int r = (x.M % kF64TileM + 7) / 8, c = (x.N % kF64TileN + 7) / 8;
+    k[0] = {m * n, 64ll * x.K};
+    k[1] = {c ? m : 0, 8ll * c * x.K};
+    k[2] = {r ? n : 0, 8ll * r * x.K};
+    k[3] = {r && c ? 1 : 0, (long long)r * c * x.K};
+  };
+  Kind k[4];
+  long long dearest = 0, tiles = 0, dear = 0;
   for (auto& x : p) {
-    const long long n = ((long long)x.M + kF64TileM - 1) / kF64TileM * ((x.N + kF64TileN - 1) / kF64TileN);
-    tiles += n;
-    if (4ll * x.K >= 3ll * deepest) deep += n;
+    if (x.M == x.N && x.a_off == x.b_off && x.a_m == x.b_n && x.a_k == x.b_k && x.K > 1) return 2;
+    kinds(x, k);
+    for (auto& y : k) dearest = y.n ? std::max(dearest, y.cost) : dearest, tiles += y.n;
   }
-  return tiles <= 3 * kSms && deep <= 2 * kSms ? 2 : 3;
+  for (auto& x : p) {
+    kinds(x, k);
+    for (auto& y : k) dear += 4 * y.cost >= 3 * dearest ? y.n : 0;
+  }
+  return tiles <= 3 * kSms && dear <= 2 * kSms ? 2 : 3;
 }
 
 void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order, cudaStream_t s) {
