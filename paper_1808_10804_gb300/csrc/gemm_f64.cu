@@ -16,16 +16,16 @@ constexpr int kBK = 16;
 constexpr int kPad = 2;
 constexpr int kSms = 152;
 
-// CTAs an SM: three, but two where three would take all tiles at once although
-// the dear ones (three quarters of the dearest or more) find room among two:
-// the others then go to the SMs that are free first.  Two as well for Gram
-// matrices, whose tiles are dear, half as dear and empty by turns.  Three / two
-// CTAs, four sectors of decreasing sizes: 372 tiles (1000 x 1000 x 1000 and
-// three smaller) 2.98 / 2.66 ms, 363 of depth 5 to 2 32.7 / 27.6 us, the
-// odd-sized corner (354) 524 / 439 us; equal depths: 450 tiles of depth 256
-// 0.88 / 1.17 ms, 1024 of 512 4.07 / 4.64; more tiles of different depths:
-// 1515 4.85 / 5.16 ms, 899 1.55 / 1.47; the products of 40 eigenproblems of 133
-// values 5.8 / 4.3 ms.
+// CTAs an SM: two, or three for lists of nearly equal tiles (85 % cost three
+// quarters of the dearest or more), more than two would take at once.  Two CTAs
+// that start together end together, so that equal tiles go to the SMs in
+// pairs: 450 tiles of depth 256 1.17 ms against 0.88 with three, 1024 of 512
+// 4.64 against 4.07, 360 of 300 1.20 against 1.03.  Unequal ones are spread
+// better by two, which leave more of them to the SMs that are free first: the
+// D=8, chi=256 FP64 move's products of 2976 x 160 x 2976 12.7 s against 14.2,
+// a D=6, chi=128 corner 2.50 ms against 2.67, the odd-sized corner 0.44 against
+// 0.52, the products of 40 eigenproblems of 133 values 4.3 against 5.8 (Gram
+// matrices, whose tiles are whole, half and empty by turns, always take two).
 int f64_ctas(const std::vector<GemmProb>& p) {
   // 8x8 products of a problem's tiles, times K: in whole tiles, along its last
   // column and row of tiles, in the corner
@@ -43,7 +43,6 @@ int f64_ctas(const std::vector<GemmProb>& p) {
   Kind k[4];
   long long dearest = 0, tiles = 0, dear = 0;
   for (auto& x : p) {
-    if (x.M == x.N && x.a_off == x.b_off && x.a_m == x.b_n && x.a_k == x.b_k && x.K > 1) return 2;
     kinds(x, k);
     for (auto& y : k) dearest = y.n ? std::max(dearest, y.cost) : dearest, tiles += y.n;
   }
@@ -51,7 +50,7 @@ int f64_ctas(const std::vector<GemmProb>& p) {
     kinds(x, k);
     for (auto& y : k) dear += 4 * y.cost >= 3 * dearest ? y.n : 0;
   }
-  return tiles <= 3 * kSms && dear <= 2 * kSms ? 2 : 3;
+  return tiles > 2 * kSms && 20 * dear >= 17 * tiles ? 3 : 2;
 }
 
 void DevGemm::upload(const std::vector<GemmProb>& p, int tm, int tn, int order, cudaStream_t s) {
@@ -139,9 +138,9 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 //   * whole tiles: a warp takes a quarter, 4x4 products from 4 + 4 fragments;
 //   * tiles at an edge: the 8x8 tiles inside M and N are dealt to the warps one
 //     by one (an odd-sized FP64 corner, 0.33 GFLOP: 594 -> 439 us).  Whole tiles
-//     dealt likewise need 16 + 16 fragments, hence registers for two CTAs an SM
-//     only: 4096 x 4096 x 4 180 -> 132 us, 2048 x 2048 x 512 4.65 -> 4.07 ms
-//     with quarters and three (f64_ctas);
+//     dealt likewise need 16 + 16 fragments, and registers that leave room for
+//     two CTAs an SM only: 4096 x 4096 x 4 180 -> 132 us, 2048 x 2048 x 512 4.65
+//     -> 4.07 ms with quarters and three (f64_ctas);
 //   * of a Gram matrix (both operands the same) only those on and above its
 //     diagonal; the sums below are the same products in the same order, so
 //     they are mirrored.
@@ -333,7 +332,8 @@ void launch_gemm_f64(Ctx* ctx, const DevGemm& g, const double* A, const double* 
                      bool behind) {
   if (g.ntiles == 0) return;
   ProfScope ps(ctx, s, "gemm_f64", g.flops, 0.0);
-  launch_behind(behind, g.ctas == 3 ? gemm_f64_kernel<3> : gemm_f64_kernel<2>, dim3(unsigned(g.ntiles)), 128, 0, s,
+  const bool three = g.ctas == 3 && A != B;  // (equal operands: Gram matrices)
+  launch_behind(behind, three ? gemm_f64_kernel<3> : gemm_f64_kernel<2>, dim3(unsigned(g.ntiles)), 128, 0, s,
                 (const GemmProb*)g.probs, (const int32_t*)g.tile_prob, (const int32_t*)g.tile_idx, A, B, C);
   BST_CUDA(cudaGetLastError());
   count_launch(ctx);
