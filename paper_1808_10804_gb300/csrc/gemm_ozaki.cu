@@ -24,10 +24,11 @@
 // products, each an A slice times a run of stacked B slices), warps 2..17
 // drain tensor memory.
 //
-// What bounds it: a 32-K chunk's 16 products take the tensor core 1014 cycles
-// (measured alone; 960 at its peak rate), a chunk of a running tile 1450 with
-// the epilogue idle and 1850 with it.  The rest is the issuing thread, whose
-// products queue only a few deep: whatever it does between the last product
+// What bounds it: a 32-K chunk's 16 products take the tensor core 960 cycles at
+// its peak rate, a chunk of a running tile about 1900 (2432 x 2432 x 2432: five
+// tiles of 76 chunks a CTA in 352 us at 2070 MHz; 1450 with the epilogue
+// idle); over a batch of 8 corners the tensor pipe is active 49 % of the time.
+// The rest is the issuing thread, whose products queue only a few deep: whatever it does between the last product
 // of a chunk and the first of the next leaves the tensor core idle, and it
 // shares its issue slots with the epilogue.  Hence counters in place of
 // divisions, tile tables that hold all a role needs, one copy per operand and
@@ -742,8 +743,9 @@ __device__ __forceinline__ void zero_part(const ZeroJob& z, int cta) {
 // a table gives every CTA its task (a search over hundreds of tasks is a
 // chain of that many loads, longer than the CTA's work).
 //
-// The kernel moves 8 bytes in and 2 S out per element, so what bounds it is
-// how the rows lie in memory:
+// The kernel moves 8 bytes in and 2 S out per element (80 registers for three
+// CTAs an SM, as the pack below), so what bounds it is how the rows lie in
+// memory:
 //   * rows contiguous along k (s_k = 1): four consecutive k per lane (two
 //     16-byte loads where the row is 16-byte aligned, 8-byte stores).  Rows
 //     up to 512 long stay in registers between the maximum and the digits;
@@ -1037,8 +1039,11 @@ __global__ void __launch_bounds__(kSplitThreads, 3) ozaki_split_kernel(SplitJob 
 // 4096 rows x segments at a time), so the index arithmetic over the legs is
 // paid once per row and segment and once per k, not per element.
 //
-// What bounds it: the latency of the loads, with 24 warps an SM (registers),
-// at a third of the memory's rate.  Against the gather and split it replaced:
+// What bounds it: the latency of the loads (9 of 16 cycles that a warp waits per issue),
+// with 24 warps an SM (80 registers: the five-digit form spills some 90 bytes;
+// with two CTAs and none of it the D=8, chi=192 move takes 3 % longer, a half
+// system in three digits 49 us instead of 44, the batch as long), at a third of
+// the memory's rate.  Against the gather and split it replaced:
 // the batch of 64 corners 3.30 -> 2.05 ms, the D=6 corner (22 MB) 0.045 ->
 // 0.029 ms, the D=8, chi=192 single-layer move's contractions 44 -> 28 ms;
 // with the innermost leg contracted, 2432 x 2432 twice, 200 -> 90 us.

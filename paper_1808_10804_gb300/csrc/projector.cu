@@ -627,7 +627,8 @@ static bool factors_subspace(Ctx* ctx, double* Nm, std::vector<PSec>& secs, int6
   // Once the columns have settled towards individual singular vectors (the
   // first steps, or Ritz vectors), the block is filtered instead: m products
   // with N^T N as the Chebyshev polynomial of degree m on [0, alpha], one
-  // CholQR after them.  alpha is the block's lower end, so what the block
+  // CholQR after them (Chebyshev-filtered subspace iteration: Zhou, Saad, Tiago
+  // and Chelikowsky, J. Comput. Phys. 219, 172, 2006).  alpha is the block's lower end, so what the block
   // does not hold stays below 1 in magnitude while a kept value lambda grows
   // by cosh(m acosh(2 lambda / alpha - 1)): two to four times the plain
   // steps' decay per product, at a quarter of their factorisations (which
