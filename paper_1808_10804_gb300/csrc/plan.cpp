@@ -214,13 +214,18 @@ void run_contract(Ctx* ctx, ContractPlan* p, const double* a, const double* b, b
   double* Bm = (double*)ctx->buf("contract.B", sizeof(double) * std::max<int64_t>(p->bmat, 1), s);
   // The gathers start when everything before the call is done; the other
   // launches overlap the one before (a D = 4, chi = 16 edge by itself 53 ->
-  // 41 us).  The GEMM only while it is as short
-  // as a launch: blocks that start on the SMs that the copies leave first end
-  // up two on one and none on another (an odd-sized corner of 0.33 GFLOP
-  // 447 -> 509 us).
+  // 41 us).  The GEMM only while it is as short as a launch, and only where its
+  // blocks find an SM each beside the gathers', or are so many more that every
+  // SM gets several: else those that start on the SMs that the copies leave
+  // first end up two on one and none on another.  One after another, behind the
+  // gathers / after them: 172 gather blocks and 60 tiles 115 / 68 us, 228 and 9
+  // 834 / 632, 38 and 141 18.1 / 13.8 (in a graph); 14 and 5 17.5 / 19.3, 14 and
+  // 363 30.6 / 32.9 (an odd-sized corner of 0.33 GFLOP 509 / 447).
   prepare_legs(ctx, {&p->ra, &p->rb, &p->rc}, s);
   launch_gathers(ctx, p->ra, a, Am, p->rb, b, Bm, s);
-  launch_gemm_f64(ctx, p->g, Am, Bm, Cm, s, p->g.flops < 1.5e7 && (p->ra.nchunks || p->rb.nchunks));
+  const int gathers = p->ra.nchunks + p->rb.nchunks, sms = 152;
+  const bool spread = gathers + p->g.ntiles <= sms || (gathers <= sms / 4 && p->g.ntiles > 2 * sms);
+  launch_gemm_f64(ctx, p->g, Am, Bm, Cm, s, p->g.flops < 1.5e7 && gathers > 0 && spread);
   launch_relayout(ctx, p->rc, c, Cm, 1, alpha, beta, s, p->g.ntiles > 0);
 }
 

@@ -92,3 +92,33 @@ def test_three_tiles_an_sm_take_three_times_one(ctx):
         torch.cuda.synchronize()
         return sorted(x.elapsed_time(y) for x, y in zip(ev[::2], ev[1::2]))[3]
     assert time(18 * 64, 25 * 64) <= 1.75 * time(16 * 64, 19 * 64)
+
+
+@pytest.mark.parametrize("degs,cut", [((3, 7, 11, 7, 3), (1, 2)), ((3, 7, 11, 7, 3), (2, 3)), ((6, 14, 22, 14, 6), (0, 3))])
+def test_contractions_in_a_row(ctx, degs, cut):
+    """Twenty contractions in a graph take no longer than twenty single calls
+    with the host's part (they did, by up to 40 %, when the tiles started on
+    the SMs that many gather blocks had left first)."""
+    from paper_1808_10804_gb300 import bst
+    q = (-2, -1, 0, 1, 2)
+    inner = tuple(d // 4 if degs[0] == 6 else max(1, d // 2) for d in degs)
+    legs = [bst.Leg(f, q, d) for f, d in ((1, degs), (-1, inner), (1, inner), (-1, degs))]
+    LA, LB = ctx.layout(legs), ctx.layout([bst.Leg(-x.flow, x.charges, x.degs) for x in legs])
+    a, b = (torch.zeros(L.nnz, dtype=torch.float64, device="cuda:0") for L in (LA, LB))
+    Cl, c = ctx.contract(LA, a, LB, b, cut, cut)
+    torch.cuda.synchronize()
+
+    def time(f):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(22)]
+        for x, y in zip(ev[::2], ev[1::2]):
+            x.record()
+            f()
+            y.record()
+            torch.cuda.synchronize()
+        return sorted(x.elapsed_time(y) for x, y in zip(ev[::2], ev[1::2]))[5]
+    one = time(lambda: ctx.contract(LA, a, LB, b, cut, cut, Cl=Cl, c=c))
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        for _ in range(20):
+            ctx.contract(LA, a, LB, b, cut, cut, Cl=Cl, c=c, stream=s)
+    assert time(g.replay) <= 20 * one
