@@ -125,31 +125,6 @@ __global__ void __launch_bounds__(kBatchThreads) relayout_batch_kernel(const Bat
     relayout_range<kBatchThreads>(bt.t, c.y, end, bases[bt.src], mat, dir, alpha, beta);
 }
 
-// Allocations and copies beside whatever stream is being captured: on a
-// stream of their own, finished when an upload returns.
-struct Aside {
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaStream_t s = nullptr;
-  Aside() {
-    BST_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
-    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaThreadExchangeStreamCaptureMode(&mode);
-      throw Error(BST_E_CUDA, "cannot create a stream");
-    }
-  }
-  ~Aside() {
-    cudaStreamDestroy(s);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-  }
-  template <class T>
-  void put(T** dst, const std::vector<T>& v) {
-    if (v.empty()) return;
-    BST_CUDA(cudaMalloc(dst, sizeof(T) * v.size()));
-    BST_CUDA(cudaMemcpyAsync(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s));
-    BST_CUDA(cudaStreamSynchronize(s));
-  }
-};
-
 // (Re)build the chunk table of a relayout for `chunk` elements per CTA; the
 // other tables with the first one.
 static void upload_rel(Aside& up, BatchRel& r, int chunk) {

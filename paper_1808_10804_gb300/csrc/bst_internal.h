@@ -306,6 +306,31 @@ void plan_relayouts_on_device(Ctx* ctx, ContractPlan* p, const std::vector<int>&
 int64_t plan_check(Ctx* ctx, Layout* A, Layout* B, const std::vector<int>& la, const std::vector<int>& lb,
                    cudaStream_t s);
 
+// Allocations, copies and launches beside whatever stream is being captured:
+// on a stream of their own, finished when an upload returns.
+struct Aside {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaStream_t s = nullptr;
+  Aside() {
+    BST_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      throw Error(BST_E_CUDA, "cannot create a stream");
+    }
+  }
+  ~Aside() {
+    cudaStreamDestroy(s);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  template <class T>
+  void put(T** dst, const std::vector<T>& v) {
+    if (v.empty()) return;
+    BST_CUDA(cudaMalloc(dst, sizeof(T) * v.size()));
+    BST_CUDA(cudaMemcpyAsync(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s));
+    BST_CUDA(cudaStreamSynchronize(s));
+  }
+};
+
 // relayout.cu
 std::vector<int2> relayout_chunks(const std::vector<RelTask>& t);  // chunk table of a task list
 // makes the leg tables that are still missing (of up to three lists), on the device

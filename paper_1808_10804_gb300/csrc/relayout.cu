@@ -74,23 +74,30 @@ __global__ void rel_legs_kernel(RelLists l) {
   if (i < l.n[r]) rel_make_legs(l.tasks[r][i], l.legs[r][i]);
 }
 
-// A stream that is being captured makes none (its graph keeps the kernel
-// without).
+// Beside a capture they are made at once, on a stream aside: a graph that
+// copies without them is slower for as long as it lives.
 void prepare_legs(Ctx* ctx, std::initializer_list<DevRelayout*> rels, cudaStream_t s) {
   DevRelayout* todo[3];
   int k = 0, longest = 0;
   for (DevRelayout* r : rels)
     if (r->narrow && !r->legs_made && r->ntasks > 0) todo[k++] = r, longest = std::max(longest, r->ntasks);
   if (k == 0) return;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  BST_CUDA(cudaStreamIsCapturing(s, &cap));
-  if (cap != cudaStreamCaptureStatusNone) return;
   RelLists l{};
   for (int i = 0; i < k; ++i) l.tasks[i] = todo[i]->tasks, l.legs[i] = todo[i]->legs, l.n[i] = todo[i]->ntasks;
-  rel_legs_kernel<<<dim3(unsigned((longest + 63) / 64), unsigned(k)), 64, 0, s>>>(l);
-  BST_CUDA(cudaGetLastError());
-  count_launch(ctx);
-  BST_CUDA(cudaStreamSynchronize(s));  // (the next launch may be on another stream)
+  auto make = [&](cudaStream_t t) {
+    rel_legs_kernel<<<dim3(unsigned((longest + 63) / 64), unsigned(k)), 64, 0, t>>>(l);
+    BST_CUDA(cudaGetLastError());
+    count_launch(ctx);
+    BST_CUDA(cudaStreamSynchronize(t));  // (the next launch may be on another stream)
+  };
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  BST_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap == cudaStreamCaptureStatusNone) {
+    make(s);
+  } else {
+    Aside aside;
+    make(aside.s);
+  }
   for (int i = 0; i < k; ++i) todo[i]->legs_made = true;
 }
 

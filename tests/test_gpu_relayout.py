@@ -96,6 +96,35 @@ def test_tables_made_where_they_are_read(bst):
     ctx.close()
 
 
+def test_captured_copies_read_tables(bst):
+    """A captured first FP64 call of a structure that was only planned copies
+    by the leg tables, as an eager one does: they are made beside the capture,
+    and the calls after it find them."""
+    ctx = bst.Context(0)
+    rng = np.random.default_rng(4)
+    legs = [bst.Leg(1, (-1, 0, 1), (3, 7, 4)), bst.Leg(-1, (-1, 0, 1), (5, 2, 6)), bst.Leg(-1, (0, 1), (9, 8))]
+    A = ctx.layout(legs)
+    B = ctx.layout([bst.Leg(-leg.flow, leg.charges, leg.degs) for leg in legs])
+    a, b = (torch.tensor(rng.standard_normal(L.nnz), device="cuda:0") for L in (A, B))
+    ctx.contract(A, a, B, b, (0,), (0,))  # (workspace for the next one)
+    C = ctx.contract_layout(A, B, (1, 2), (1, 2))
+    out = torch.zeros(C.nnz, dtype=torch.float64, device="cuda:0")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    n0 = ctx.launches
+    with torch.cuda.graph(g, stream=s):
+        ctx.contract(A, a, B, b, (1, 2), (1, 2), Cl=C, c=out, stream=s)
+    assert ctx.launches - n0 == 4  # (tables, both gathers, product, scatter)
+    n0 = ctx.launches
+    ref = ctx.contract(A, a, B, b, (1, 2), (1, 2), Cl=C)[1]
+    assert ctx.launches - n0 == 3
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    ctx.close()
+
+
 @pytest.mark.parametrize("shape", [(2, 8000001), (8000001, 2), (5, 1600001), (1600001, 11)])
 def test_thin_transpositions_keep_up(bst, shape):
     """Transposing a thin matrix takes no longer than a square one of the same
